@@ -34,7 +34,7 @@ bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int
 bbl_status chol_seg(int b, int nseg, const double* G, const double* thresh2, int relative, double* R, double* Rinv,
                     int* ndefl, int* mask, int* status, const int* active, cudaStream_t st);
 bbl_status trmul_seg(int b, int nseg, const double* R2, const double* R1, double* B, const int* active, cudaStream_t st);
-size_t ritz_seg_workspace_doubles(int m_max, int p, int nev);
+size_t ritz_batch_workspace_bytes(int m_max, int p, int nev, int nseg);
 int gram_seg_chunk_rows(int b, int dtype);
 bbl_status ritz_dev_batched(int m_max, int p, int nev, int nseg, const double* Tb, int64_t sT, double* theta,
                             int64_t sTh, double* width, double* S, int64_t sS, double* ws, double* tmp, const int* d_m,
@@ -407,7 +407,7 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
     BBL_TRY(width.alloc(sizeof(double) * (size_t)nseg * nev));
     BBL_TRY(S.alloc(sizeof(double) * (size_t)nseg * m_max * nev));
     BBL_TRY(est.alloc(sizeof(double) * (size_t)nseg * nev));
-    BBL_TRY(ws.alloc(sizeof(double) * (size_t)nseg * ritz_seg_workspace_doubles(m_max, b, nev)));
+    BBL_TRY(ws.alloc(ritz_batch_workspace_bytes(m_max, b, nev, nseg)));
     BBL_TRY(tmp.alloc(sizeof(double) * (size_t)nseg * m_max * nev));
     // ints: d_j, d_m, d_b, iters, then per segment: active, final_j, status, ndefl, mask[b], ms, due, next_chk,
     // jprev

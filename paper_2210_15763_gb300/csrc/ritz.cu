@@ -3,7 +3,10 @@
 // off-diagonal blocks B_j from CholQR2 are upper triangular), stored as a
 // lower band: Tb[i*(p+1) + d] = T[i][i-d].
 //
-// Three kernels, all on the device:
+// Isolated eigenvalues are computed by slicing and block cyclic reduction
+// (ritz_cr.cu); the sequential kernels here run for bands that path does not
+// take (ritz_cr_supports) and for segments it could not certify (degenerate
+// or nearly degenerate values), and otherwise return at once:
 //  1. bisect  - one CTA per wanted eigenvalue index i.  Sylvester's law of
 //               inertia: the number of negative pivots of the LDL^T
 //               factorisation of T - sigma I is the number of eigenvalues below
@@ -29,8 +32,8 @@
 //               entry positive).
 #include <algorithm>
 
-#include "common.cuh"
 #include "df32.cuh"
+#include "ritz.cuh"
 
 namespace bbl {
 namespace {
@@ -39,17 +42,7 @@ constexpr int kMaxP = kMaxB;            // bandwidth limit
 constexpr int kWin = kMaxP + 1;         // LDL^T window edge
 constexpr int kBisectWarps = 8;
 constexpr size_t kBandSmemMax = 160 * 1024;  // band bytes staged in shared memory
-constexpr int kMaxNev = 32;
 constexpr size_t kInvitSmemMax = 220 * 1024;  // inverse iteration: window, vector and LU factors
-
-// Per-segment addressing for a batch of independent T's (blockIdx.y = segment
-// in bisect / invit, blockIdx.x in cluster).  The single-problem path passes
-// d_m = active = nullptr and zero strides.
-struct SegArgs {
-    const int* d_m;       // current order m in device memory (overrides the argument)
-    const int* active;    // per-segment flag; inactive segments are skipped
-    int64_t sT, sTh, sS, sWs, sTmp;
-};
 
 __device__ __forceinline__ double band_get(const double* __restrict__ Tb, int p, int m, int r, int c) {
     // T[r][c] for any r, c (0 outside the band or the matrix)
@@ -303,6 +296,7 @@ __global__ void __launch_bounds__(256) bisect_lane_kernel(int m, int nev, const 
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
+    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
     Tg += seg * sa.sT;
@@ -483,6 +477,7 @@ __global__ void __launch_bounds__(32 * kBisectWarps) bisect_kernel(int m, int p,
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
+    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
     Tg += seg * sa.sT;
@@ -630,6 +625,7 @@ __global__ void __launch_bounds__(32) invit_kernel(int m, int p, const double* _
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
+    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
     Tg += seg * sa.sT;
@@ -817,6 +813,7 @@ __global__ void __launch_bounds__(32) invit_df_kernel(int m, const double* __res
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
+    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
     Tg += seg * sa.sT;
@@ -1026,20 +1023,37 @@ __global__ void __launch_bounds__(32) invit_df_kernel(int m, const double* __res
     for (int r = lane; r < m; r += 32) S[(int64_t)r * nev + i] = xd[r];
 }
 
+// sum over the 256 threads of a CTA (every thread gets it; two barriers)
+__device__ __forceinline__ double cta_sum(double s, double* red /* 8 */) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    double t = red[threadIdx.x & 7];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    __syncthreads();
+    return t;
+}
+
 // Groups close eigenvalues, orthonormalises their vectors, Rayleigh-Ritz in
-// each group (cyclic Jacobi), sorts, applies the sign convention.
+// each group (cyclic Jacobi), sorts, applies the sign convention.  Pairs of
+// the fast path (sa.need clear) come sorted, with the sign convention
+// applied: without a group there is nothing to do.
 __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, const double* __restrict__ Tb,
                                                       double* __restrict__ theta, double* __restrict__ S,
                                                       double* __restrict__ tmp /* m x ldS */, SegArgs sa) {
     __shared__ double K[kMaxNev * kMaxNev];
     __shared__ double Z[kMaxNev * kMaxNev];
-    __shared__ double red[256];
+    __shared__ double red[8];
     __shared__ double th[kMaxNev];
+    __shared__ int order[kMaxNev];
     __shared__ int start[kMaxNev + 1];
-    __shared__ int ngroups;
-    __shared__ double s_scale;
+    __shared__ int ngroups, sorted;
+    __shared__ unsigned long long s_scale_bits;
     const int seg = blockIdx.x;
     if (sa.active && !sa.active[seg]) return;
+    const bool certified = sa.need && !sa.need[seg];
     if (sa.d_m) m = *sa.d_m;
     const int nev = min(ldS, m);  // columns computed; S keeps row stride ldS
     Tb += seg * sa.sT;
@@ -1047,50 +1061,53 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
     S += seg * sa.sS;
     tmp += seg * sa.sTmp;
     const int tid = threadIdx.x;
-    // scale = max |theta|, at least the largest diagonal magnitude
-    double sc = 0.0;
-    for (int r = tid; r < m; r += 256) sc = fmax(sc, fabs(band_get(Tb, p, m, r, r)));
-    for (int k = tid; k < nev; k += 256) sc = fmax(sc, fabs(theta[k]));
-    red[tid] = sc;
+    if (tid == 0) s_scale_bits = 0;
     __syncthreads();
-    if (tid == 0) {
-        for (int t = 1; t < 256; ++t) sc = fmax(sc, red[t]);
-        s_scale = fmax(sc, 1e-300);
-        // sort theta (and remember the permutation in start[] temporarily): insertion sort
-        for (int k = 0; k < nev; ++k) th[k] = theta[k];
+    // scale = max |theta|, at least the largest diagonal magnitude (non-negative
+    // doubles order as their bits)
+    {
+        unsigned long long sc = 0;
+        for (int r = tid; r < m; r += 256)
+            sc = max(sc, (unsigned long long)__double_as_longlong(Tb[(int64_t)r * (p + 1)]) & 0x7fffffffffffffffull);
+        if (tid < nev) sc = max(sc, (unsigned long long)__double_as_longlong(theta[tid]) & 0x7fffffffffffffffull);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, o));
+        if ((tid & 31) == 0) atomicMax(&s_scale_bits, sc);
+    }
+    // rank of each value (ties by index)
+    if (tid < nev) {
+        const double v = theta[tid];
+        int rank = 0;
+        for (int k = 0; k < nev; ++k) {
+            const double o = theta[k];
+            rank += (o < v || (o == v && k < tid)) ? 1 : 0;
+        }
+        th[rank] = v;
+        order[rank] = tid;
     }
     __syncthreads();
-    // sort columns by theta (selection on thread 0, column swaps in parallel)
-    for (int a = 0; a < nev; ++a) {
-        __shared__ int sel;
-        if (tid == 0) {
-            int best = a;
-            for (int k = a + 1; k < nev; ++k)
-                if (th[k] < th[best]) best = k;
-            sel = best;
-            const double t = th[a];
-            th[a] = th[best];
-            th[best] = t;
-        }
-        __syncthreads();
-        if (sel != a) {
-            for (int r = tid; r < m; r += 256) {
-                const double t = S[(int64_t)r * ldS + a];
-                S[(int64_t)r * ldS + a] = S[(int64_t)r * ldS + sel];
-                S[(int64_t)r * ldS + sel] = t;
-            }
-        }
-        __syncthreads();
-    }
+    const double s_scale = fmax(__longlong_as_double((long long)s_scale_bits), 1e-300);
     if (tid == 0) {
-        int g = 0;
+        int g = 0, ok = 1;
         start[0] = 0;
-        for (int k = 1; k < nev; ++k)
+        for (int k = 1; k < nev; ++k) {
             if (th[k] - th[k - 1] > 1e-3 * s_scale) start[++g] = k;
+            ok = ok && order[k] > order[k - 1];
+        }
         start[++g] = nev;
         ngroups = g;
+        sorted = ok;
     }
     __syncthreads();
+    if (certified && sorted && ngroups == nev) return;
+    if (!sorted) {
+        for (int r = tid; r < m; r += 256) {
+            double row[kMaxNev];
+            for (int a = 0; a < nev; ++a) row[a] = S[(int64_t)r * ldS + order[a]];
+            for (int a = 0; a < nev; ++a) S[(int64_t)r * ldS + a] = row[a];
+        }
+        __syncthreads();
+    }
     for (int g = 0; g < ngroups; ++g) {
         const int a0 = start[g], a1 = start[g + 1], k = a1 - a0;
         if (k < 2) continue;
@@ -1100,31 +1117,16 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
                 for (int q = a0; q < a; ++q) {
                     double s = 0.0;
                     for (int r = tid; r < m; r += 256) s += S[(int64_t)r * ldS + q] * S[(int64_t)r * ldS + a];
-                    red[tid] = s;
-                    __syncthreads();
-                    for (int w = 128; w > 0; w >>= 1) {
-                        if (tid < w) red[tid] += red[tid + w];
-                        __syncthreads();
-                    }
-                    const double dot = red[0];
-                    __syncthreads();
+                    const double dot = cta_sum(s, red);
                     for (int r = tid; r < m; r += 256) S[(int64_t)r * ldS + a] -= dot * S[(int64_t)r * ldS + q];
-                    __syncthreads();
                 }
                 double s = 0.0;
                 for (int r = tid; r < m; r += 256) s += S[(int64_t)r * ldS + a] * S[(int64_t)r * ldS + a];
-                red[tid] = s;
-                __syncthreads();
-                for (int w = 128; w > 0; w >>= 1) {
-                    if (tid < w) red[tid] += red[tid + w];
-                    __syncthreads();
-                }
-                const double inv = 1.0 / sqrt(red[0]);
-                __syncthreads();
+                const double inv = 1.0 / sqrt(cta_sum(s, red));
                 for (int r = tid; r < m; r += 256) S[(int64_t)r * ldS + a] *= inv;
-                __syncthreads();
             }
         }
+        __syncthreads();
         // tmp = T * S_group
         for (int r = tid; r < m; r += 256) {
             for (int a = a0; a < a1; ++a) {
@@ -1133,21 +1135,15 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
                 tmp[(int64_t)r * ldS + a] = t;
             }
         }
-        __syncthreads();
-        // K = S_g^T T S_g
+        // K = S_g^T T S_g (each thread's own rows)
         for (int e = 0; e < k * k; ++e) {
             const int a = a0 + e / k, q = a0 + e % k;
             double s = 0.0;
             for (int r = tid; r < m; r += 256) s += S[(int64_t)r * ldS + a] * tmp[(int64_t)r * ldS + q];
-            red[tid] = s;
-            __syncthreads();
-            for (int w = 128; w > 0; w >>= 1) {
-                if (tid < w) red[tid] += red[tid + w];
-                __syncthreads();
-            }
-            if (tid == 0) K[e] = red[0];
-            __syncthreads();
+            s = cta_sum(s, red);
+            if (tid == 0) K[e] = s;
         }
+        __syncthreads();
         // cyclic Jacobi on K (thread 0; k <= 64)
         if (tid == 0) {
             for (int e = 0; e < k * k; ++e) Z[e] = (e / k == e % k) ? 1.0 : 0.0;
@@ -1216,45 +1212,44 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
         }
         __syncthreads();
     }
-    // sign convention: the first entry of largest magnitude is positive
-    for (int a = 0; a < nev; ++a) {
-        double best = -1.0;
-        int bi = 0;
-        for (int r = tid; r < m; r += 256) {
-            const double v = fabs(S[(int64_t)r * ldS + a]);
-            if (v > best) {
-                best = v;
+    // sign convention: the first entry of largest magnitude is positive (a warp per column)
+    for (int a = tid >> 5; a < nev; a += 8) {
+        const int lane = tid & 31;
+        unsigned long long best = 0;
+        for (int r = lane; r < m; r += 32)
+            best = max(best, (unsigned long long)__double_as_longlong(S[(int64_t)r * ldS + a]) & 0x7fffffffffffffffull);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+        int bi = 0x7fffffff;
+        for (int r = lane; r < m; r += 32)
+            if (((unsigned long long)__double_as_longlong(S[(int64_t)r * ldS + a]) & 0x7fffffffffffffffull) == best) {
                 bi = r;
+                break;
             }
-        }
-        __shared__ double bv[256];
-        __shared__ int bix[256];
-        bv[tid] = best;
-        bix[tid] = bi;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (tid < w) {
-                if (bv[tid + w] > bv[tid] || (bv[tid + w] == bv[tid] && bix[tid + w] < bix[tid])) {
-                    bv[tid] = bv[tid + w];
-                    bix[tid] = bix[tid + w];
-                }
-            }
-            __syncthreads();
-        }
-        const bool flip = S[(int64_t)bix[0] * ldS + a] < 0.0;
-        __syncthreads();
+        bi = __reduce_min_sync(0xffffffffu, bi);
+        const bool flip = S[(int64_t)bi * ldS + a] < 0.0;
+        __syncwarp();
         if (flip)
-            for (int r = tid; r < m; r += 256) S[(int64_t)r * ldS + a] = -S[(int64_t)r * ldS + a];
-        __syncthreads();
+            for (int r = lane; r < m; r += 32) S[(int64_t)r * ldS + a] = -S[(int64_t)r * ldS + a];
     }
     for (int k = tid; k < nev; k += 256) theta[k] = th[k];
 }
 
 }  // namespace
 
+// One problem's workspace: the sequential kernels' factors (U, L, pivots) or
+// the cyclic reduction's matrices in the same place, then the bracket widths,
+// T S of a group of close values, and the slicing's counts.
+namespace {
+size_t ritz_factor_doubles(int m, int p, int nev) {
+    const size_t seq = (size_t)nev * m * (3 * p + 1) + (sizeof(int) * (size_t)nev * m + 7) / 8;
+    return (std::max(seq, (size_t)nev * ritz_cr_vec_doubles(m, p)) + 31) & ~size_t(31);
+}
+}  // namespace
+
 size_t ritz_workspace_bytes(int m, int p, int nev) {
-    return sizeof(double) * ((size_t)nev * m * (3 * p + 1) + (size_t)m * nev + 2 * (size_t)nev) +
-           sizeof(int) * (size_t)nev * m + 256;
+    const size_t d = ritz_factor_doubles(m, p, nev) + (size_t)m * nev + nev + 32;
+    return ((sizeof(double) * d + 255) & ~size_t(255)) + ritz_cr_bytes(m, p, nev, 1) + 256;
 }
 
 namespace {
@@ -1348,14 +1343,19 @@ bbl_status ritz_dev(int m, int p, int nev, const double* Tb, double* theta, doub
     const size_t need = ritz_workspace_bytes(m, p, nev);
     if (work.bytes < need) BBL_TRY(work.alloc(need + need / 2));
     double* ws = work.as<double>();
-    double* width = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + sizeof(double) * (size_t)nev * m * (3 * p + 1) +
-                                      sizeof(int) * (size_t)nev * m + 64);
-    width = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(width) + 15) & ~uintptr_t(15));
-    double* tmp = width + nev + 2;
+    double* width = ws + ritz_factor_doubles(m, p, nev);
+    double* tmp = width + ((nev + 15) & ~15);
+    void* fast = reinterpret_cast<char*>(ws) +
+                 ((sizeof(double) * (ritz_factor_doubles(m, p, nev) + (size_t)m * nev + nev + 32) + 255) & ~size_t(255));
     const size_t band_bytes = sizeof(double) * (size_t)m * (p + 1);
     const int band_smem = band_bytes <= kBandSmemMax ? 1 : 0;
     BBL_TRY(set_ritz_attrs());
-    const SegArgs one{nullptr, nullptr, 0, 0, 0, 0, 0};
+    SegArgs one{nullptr, nullptr, 0, 0, 0, 0, 0};
+    if (ritz_cr_supports(m, p)) {
+        int* flag = nullptr;
+        BBL_TRY(ritz_cr(m, p, nev, 1, Tb, theta, S, ws, fast, &flag, one, st));
+        one.need = flag;
+    }
     BBL_TRY(launch_bisect(dim3(nev), m, p, nev, Tb, theta, width, band_smem, band_bytes, one, warm, warm_count, st));
     BBL_TRY(launch_invit(dim3(nev), m, p, nev, Tb, theta, S, ws, one, st));
     cluster_kernel<<<1, 256, 0, st>>>(m, p, nev, Tb, theta, S, tmp, one);
@@ -1365,14 +1365,19 @@ bbl_status ritz_dev(int m, int p, int nev, const double* Tb, double* theta, doub
 
 // Per-segment workspace (doubles) for orders up to m_max.
 size_t ritz_seg_workspace_doubles(int m_max, int p, int nev) {
-    const size_t d = (size_t)nev * m_max * (3 * p + 1) + (sizeof(int) * (size_t)nev * m_max + 7) / 8 + 16;
-    return (d + 31) & ~size_t(31);
+    return ritz_factor_doubles(m_max, p, nev);
+}
+
+// bytes of `ws` for nseg segments in ritz_dev_batched
+size_t ritz_batch_workspace_bytes(int m_max, int p, int nev, int nseg) {
+    return ((sizeof(double) * (size_t)nseg * ritz_seg_workspace_doubles(m_max, p, nev) + 255) & ~size_t(255)) +
+           ritz_cr_bytes(m_max, p, nev, nseg);
 }
 
 // Batched Ritz solves: nseg independent band matrices Tb + s*sT (order *d_m,
 // at most m_max, bandwidth p), k = min(nev, m) lowest pairs each into
 // theta + s*sTh and S + s*sS (row stride nev); segments with active[s] == 0
-// are skipped.  ws: nseg * ritz_seg_workspace_doubles; tmp: nseg * m_max * nev.
+// are skipped.  ws: ritz_batch_workspace_bytes; tmp: nseg * m_max * nev.
 bbl_status ritz_dev_batched(int m_max, int p, int nev, int nseg, const double* Tb, int64_t sT, double* theta,
                             int64_t sTh, double* width, double* S, int64_t sS, double* ws, double* tmp, const int* d_m,
                             const int* active, cudaStream_t st) {
@@ -1380,7 +1385,13 @@ bbl_status ritz_dev_batched(int m_max, int p, int nev, int nseg, const double* T
     const size_t band_bytes = sizeof(double) * (size_t)m_max * (p + 1);
     const int band_smem = band_bytes <= kBandSmemMax ? 1 : 0;
     const int64_t sWs = (int64_t)ritz_seg_workspace_doubles(m_max, p, nev);
-    const SegArgs sa{d_m, active, sT, sTh, sS, sWs, (int64_t)m_max * nev};
+    SegArgs sa{d_m, active, sT, sTh, sS, sWs, (int64_t)m_max * nev};
+    if (ritz_cr_supports(m_max, p)) {
+        void* fast = reinterpret_cast<char*>(ws) + ((sizeof(double) * (size_t)nseg * (size_t)sWs + 255) & ~size_t(255));
+        int* flag = nullptr;
+        BBL_TRY(ritz_cr(m_max, p, nev, nseg, Tb, theta, S, ws, fast, &flag, sa, st));
+        sa.need = flag;
+    }
     dim3 g(nev, nseg);
     BBL_TRY(launch_bisect(g, m_max, p, nev, Tb, theta, width, band_smem, band_bytes, sa, nullptr, 0, st));
     BBL_TRY(launch_invit(g, m_max, p, nev, Tb, theta, S, ws, sa, st));
