@@ -1550,6 +1550,8 @@ int gram_worker_sms() { return std::max(1, sm_count() - kRitzReserveSMs); }
 bbl_status gram(int64_t n, int b, int nblocks, int dtype, const void* Q, const void* W, double* C, DevBuf& partials,
                 cudaStream_t st) {
     const int m = nblocks * b;
+    if (dtype == BBL_FP64 && tc64_gram_supports(b, m))
+        return gram_tc64(n, b, m, static_cast<const double*>(Q), static_cast<const double*>(W), C, partials, st);
     if (dtype == BBL_FP64)
         return gram_typed<double>(n, b, m, static_cast<const double*>(Q), static_cast<const double*>(W), C, partials, st);
     if (dtype == kDF32)
@@ -1572,6 +1574,8 @@ bbl_status to_half(int64_t count, const float* in, void* out, cudaStream_t st) {
 
 bbl_status update(int64_t n, int b, int nblocks, int dtype, const void* Q, const double* C, void* W, cudaStream_t st) {
     const int m = nblocks * b;
+    if (dtype == BBL_FP64 && tc64_update_supports(b, m))
+        return update_tc64(n, b, m, b, static_cast<const double*>(Q), C, static_cast<double*>(W), true, st);
     if (dtype == BBL_FP64)
         return apply_typed<double, true, double, double>(n, b, m, b, static_cast<const double*>(Q), C,
                                                          static_cast<double*>(W), st);
@@ -1612,6 +1616,8 @@ bbl_status update_df32_f32old(int64_t n, int nblocks, int nnew, const float* Q32
 bbl_status ritz_vectors(int64_t n, int b, int nblocks, int dtype, const void* Q, int k, const double* S, double* X,
                         cudaStream_t st) {
     const int m = nblocks * b;
+    if (dtype == BBL_FP64 && tc64_update_supports(b, m))
+        return update_tc64(n, b, m, k, static_cast<const double*>(Q), S, X, false, st);
     if (dtype == BBL_FP64)
         return apply_typed<double, false, double, double>(n, b, m, k, static_cast<const double*>(Q), S, X, st);
     if (dtype == kDF32)

@@ -1,0 +1,675 @@
+// FP64 Gram and update of the Gram-Schmidt passes on the tensor cores, to
+// FP64 accuracy (splitting after Ozaki, Ogita, Oishi, Rump 2012 in the FP16
+// tensor-core form of Mukunoki, Ozaki, Ogita, Imamura 2020).
+//
+// GB300's FP64 pipes (1.06 TFLOP/s measured) bind C = Q^T W and W -= Q C at
+// 16 operations per 8-byte basis element (b = 8): 12 times the time HBM needs.
+// Here an FP64 number becomes an integer of 56 bits relative to a power of
+// two near its row's (or column's) largest entry, cut into seven digits of 8
+// bits; a digit with its sign is an FP16 number, and a product of two digit
+// matrices is exact in the tensor cores' FP32 sums as long as these stay
+// below 2^24.  Digit products i, j of one order o = i + j share an
+// accumulator: 34 products give the orders 0..7.  Orders 0..3 are exact:
+// after 64 terms (at most 64 (1023 * 128 + 2 * 255 * 128 + 255 * 256) < 2^24) they move to
+// 32-bit integers; orders 4..7 weigh 2^-32 and less, where FP32 rounding is
+// below 2^-56.  The basis is cut in sign and magnitude (the first digit has
+// two spare bits, so a line may outgrow its first entries fourfold); the
+// other operand, cut once per CTA, into balanced digits -128..127 of the
+// rounded value, so that the dropped orders (below 2^-62 of the largest
+// products) have random signs instead of the products' own.
+//
+// Digits are cut by integer instructions in registers from a ring of
+// asynchronous copies.  At n = 2e5, b = 8, 50 blocks (640 MB, 94 us at the copy
+// rate) the Gram takes 0.25 ms and the update 0.24 ms; the FP64 FMA kernels
+// took 1.67 and 1.20 ms.  What bounds them now is instruction issue (integer
+// pipe 51-55 %, tensor pipe 33 % active, DRAM a third of the copy rate).
+#include <algorithm>
+#include <cstdint>
+
+#include <cuda_fp16.h>
+
+#include "common.cuh"
+
+namespace bbl {
+namespace {
+
+constexpr int kT = 256;            // threads per CTA
+constexpr int kWarps = kT / 32;
+constexpr int kDig = 7;            // digits of 8 bits
+constexpr int kOrd = 8;            // orders summed (of the products' 13)
+constexpr int kExact = 4;          // orders kept exactly
+constexpr int kOver = 2;           // bits by which an entry may exceed its line's scale (the first digit's spare bits)
+constexpr int kMaxRows = 512;      // Gram: rows per CTA
+constexpr int kMaxCols = 512;      // update: coefficient rows staged at once
+constexpr int kEmin = 100;         // smallest exponent field used for a scale
+constexpr int kRing = 3;           // steps of a warp in its shared-memory ring
+constexpr int kStepBytes = 2048;   // 16 x 16 basis entries
+
+struct Acc {
+    float f[kOrd][4];   // order sums
+    int h[kExact][4];   // exact sums of the first orders
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int o = 0; o < kOrd; ++o)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) f[o][e] = 0.0f;
+#pragma unroll
+        for (int o = 0; o < kExact; ++o)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) h[o][e] = 0;
+    }
+    __device__ __forceinline__ void to_int() {
+#pragma unroll
+        for (int o = 0; o < kExact; ++o)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                h[o][e] += __float2int_rn(f[o][e]);
+                f[o][e] = 0.0f;
+            }
+    }
+    // the sum over the orders in units of order 3 (call to_int before)
+    __device__ __forceinline__ double value(int e) const {
+        const long long H = ((long long)h[0][e] << 24) + ((long long)h[1][e] << 16) + ((long long)h[2][e] << 8) +
+                            (long long)h[3][e];
+        const float L = fmaf(f[4][e], 0x1p-8f, fmaf(f[5][e], 0x1p-16f, fmaf(f[6][e], 0x1p-24f, f[7][e] * 0x1p-32f)));
+        return (double)H + (double)L;
+    }
+};
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], const unsigned (&a)[4], const uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+// exponent field of a double's high word, in place (bits 20..30)
+__device__ __forceinline__ int exp_bits(double v) { return __double2hiint(v) & 0x7ff00000; }
+
+// 2^e, e clamped to the normal range
+__device__ __forceinline__ double pow2(int e) {
+    e = max(-1022, min(1023, e));
+    return __hiloint2double((e + 1023) << 20, 0);
+}
+
+// v * 2^e for any e (two exact powers of two)
+__device__ __forceinline__ double scale_by(double v, int e) {
+    const int h = e / 2;
+    return v * pow2(h) * pow2(e - h);
+}
+
+// The right shift that cuts an entry's mantissa (left-aligned as below) to the
+// scale of exponent field E, plus 2048 for a negative entry: modulo 2048 it is
+// at most 31 for entries down to 2^-29 of the scale, and its bits 5..10 tell
+// smaller entries and entries above the scale by more than kOver bits.
+// It is the high word of (E + kOver) 2^32 + 2^32 - 1 - hi 2^12, one multiply-add.
+__device__ __forceinline__ unsigned shift_word(int E, double v) {
+    unsigned s;
+    asm("{.reg .b64 t, c; .reg .b32 l; mov.b64 c, {%1, %2}; mad.wide.s32 t, %3, -4096, c; mov.b64 {l, %0}, t;}"
+        : "=r"(s)
+        : "r"(0xffffffffu), "r"(E + kOver), "r"(__double2hiint(v)));
+    return s;
+}
+
+// the mantissa times 2^5 (its leading bit at 57 = 55 + kOver)
+__device__ __forceinline__ void aligned_mantissa(double v, unsigned& yl, unsigned& yh) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    // products, not shifts: the integer ALU is the busiest pipe, the multiplier idles
+    unsigned c;
+    asm("{.reg .b64 t; mul.wide.u32 t, %2, 32; mov.b64 {%0, %1}, t;}" : "=r"(yl), "=r"(c) : "r"(lo));
+    yh = ((hi * 32u + c) & 0x01ffffffu) | 0x02000000u;
+}
+
+// The magnitude of v relative to the exponent field E: floor(|v| 2^(55 - (E
+// - 1023))), below 2^56 if v's exponent field is at most E; s = shift_word
+// with bits 5..10 clear.
+__device__ __forceinline__ uint2 magnitude(double v, unsigned s) {
+    unsigned yl, yh;
+    aligned_mantissa(v, yl, yh);
+    return make_uint2(__funnelshift_r(yl, yh, s), __funnelshift_r(yh, 0u, s));
+}
+
+// the same for any s with v at most kOver bits above the scale
+__device__ __forceinline__ uint2 magnitude_any(double v, unsigned s) {
+    unsigned yl, yh;
+    aligned_mantissa(v, yl, yh);
+    s &= 0x7ffu;
+    if (s >= 64) return make_uint2(0u, 0u);
+    if (s >= 32) return make_uint2(yh >> (s - 32), 0u);
+    return make_uint2(__funnelshift_r(yl, yh, s), yh >> s);
+}
+
+// Two magnitudes and the high words that carry their signs: digit i
+// (0 = most significant) of both as a pair of signed FP16 numbers.
+struct Pair {
+    uint2 u, v;
+    unsigned sg, off;  // +-1 and -+1024 as FP16 pairs
+    template <bool ANY>
+    __device__ __forceinline__ void set(double a, double b, unsigned sa, unsigned sb) {
+        u = ANY ? magnitude_any(a, sa) : magnitude(a, sa);
+        v = ANY ? magnitude_any(b, sb) : magnitude(b, sb);
+        const unsigned s = __byte_perm((unsigned)__double2hiint(a), (unsigned)__double2hiint(b), 0x7430) & 0x80008000u;
+        sg = s | 0x3c003c00u;
+        off = s ^ 0xe400e400u;
+    }
+    template <int I>
+    __device__ __forceinline__ unsigned digit() const {
+        unsigned x;  // 1024 + digit
+        if constexpr (I == 0) {
+            x = __byte_perm(u.y, v.y, 0x7632) | 0x64006400u;  // the bits from 48 on: up to ten
+        } else {
+            constexpr int byte = I < 3 ? 2 - I : 6 - I;
+            constexpr unsigned sel = (unsigned)(byte | (byte << 4) | ((4 + byte) << 8) | ((4 + byte) << 12));
+            x = (__byte_perm(I < 3 ? u.y : u.x, I < 3 ? v.y : v.x, sel) & 0x00ff00ffu) | 0x64006400u;
+        }
+        unsigned r;
+        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(sg), "r"(off));
+        return r;
+    }
+};
+
+template <int I>
+__device__ __forceinline__ void mma_digit(Acc& acc, const Pair (&p)[4], const uint2 (&b)[kDig]) {
+    const unsigned a[4] = {p[0].digit<I>(), p[1].digit<I>(), p[2].digit<I>(), p[3].digit<I>()};
+#pragma unroll
+    for (int j = 0; j < kDig && I + j < kOrd; ++j) mma_f16(acc.f[I + j], a, b[j]);
+}
+
+// 16 terms: pairs p (fragment registers 0..3 of A), B's digits at frag[j * 32 + lane]
+__device__ __forceinline__ void mma_step(Acc& acc, const Pair (&p)[4], const uint2* __restrict__ frag, int lane) {
+    uint2 b[kDig];
+#pragma unroll
+    for (int j = 0; j < kDig; ++j) b[j] = frag[j * 32 + lane];
+    mma_digit<0>(acc, p, b);
+    mma_digit<1>(acc, p, b);
+    mma_digit<2>(acc, p, b);
+    mma_digit<3>(acc, p, b);
+    mma_digit<4>(acc, p, b);
+    mma_digit<5>(acc, p, b);
+    mma_digit<6>(acc, p, b);
+}
+
+// round(v 2^(55 - (E - 1023))) plus 128 in each of the low six bytes and 384 in
+// the bits above: balanced digits -128 .. 127 (the first -256 .. 256) in
+// unsigned fields; E at least v's exponent field.
+constexpr unsigned long long kBalance = 0x0180808080808080ull;
+__device__ __forceinline__ unsigned long long balanced(double v, int E) {
+    if (exp_bits(v) == 0) return kBalance;  // zero (or denormal)
+    const uint2 q = magnitude_any(v, shift_word(E - 1, v));
+    const unsigned long long r = ((((unsigned long long)q.y << 32) | q.x) + 1) >> 1;
+    return (v < 0.0 ? 0ull - r : r) + kBalance;
+}
+
+// B's digits of one lane: terms x[0], x[1] and x[2], x[3] of its column,
+// exponent field E of the column's scale
+__device__ __forceinline__ void store_frag(uint2* __restrict__ frag, int lane, const double (&x)[4], int E) {
+    unsigned long long q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = balanced(x[i], E);
+#pragma unroll
+    for (int j = 0; j < kDig; ++j) {
+        const int sh = 8 * (kDig - 1 - j);
+        unsigned w[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned mask = j == 0 ? 0x3ffu : 0xffu;
+            const unsigned lo = (unsigned)(q[2 * h] >> sh) & mask, hi = (unsigned)(q[2 * h + 1] >> sh) & mask;
+            const unsigned b = 0x64006400u | lo | (hi << 16);  // 1024 + 128 (or 384) + digit
+            asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w[h]) : "r"(b), "r"(j == 0 ? 0xe580e580u : 0xe480e480u));
+        }
+        frag[j * 32 + lane] = make_uint2(w[0], w[1]);
+    }
+}
+
+// The A operand's scales: a lane's registers 0 and 2 belong to line g (a basis
+// column in the Gram, a row in the update), 1 and 3 to line g + 8.  E0, E1:
+// the exponent fields of the two scales, shared by the four lanes of a line.
+// x: the lane's eight entries, pairs (0,1) (2,3) (4,5) (6,7) of registers 0..3.
+struct LineScale {
+    int E0 = 0, E1 = 0;
+    // shift words of the entries; for the whole warp: 0 if all are at most 31,
+    // bit 0 if some are larger, bit 1 if an entry exceeds its scale by more than
+    // kOver bits
+    __device__ __forceinline__ unsigned shifts(const double (&x)[8], unsigned (&s)[8]) const {
+        unsigned bits = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            s[k] = shift_word((k & 2) ? E1 : E0, x[k]);
+            bits |= s[k] & 0x7e0u;
+        }
+        if (!__any_sync(0xffffffffu, bits)) return 0;
+        bool over = false;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            over = over || (int)(((unsigned)__double2hiint(x[k]) >> 20) & 0x7ffu) > ((k & 2) ? E1 : E0) + kOver;
+        return __any_sync(0xffffffffu, over) ? 3 : 1;
+    }
+    __device__ __forceinline__ void raise(const double (&x)[8]) {
+        int m0 = max(max(exp_bits(x[0]), exp_bits(x[1])), max(exp_bits(x[4]), exp_bits(x[5])));
+        int m1 = max(max(exp_bits(x[2]), exp_bits(x[3])), max(exp_bits(x[6]), exp_bits(x[7])));
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        }
+        E0 = limit(max(m0 >> 20, E0));
+        E1 = limit(max(m1 >> 20, E1));
+    }
+    // a zero's shift word is E + kOver modulo 2048: E stays below 2048 - kOver
+    // (finite entries above are within kOver bits), or is 0x7ff, whose sums are NaN
+    static __device__ __forceinline__ int limit(int E) { return E >= 0x7ff ? 0x7ff : max(kEmin, min(E, 0x7fd)); }
+};
+
+// One step of 16 terms; flush() moves the accumulators to the sums at the old
+// scales (nothing before the first step).
+template <typename Flush>
+__device__ __forceinline__ void step(Acc& acc, LineScale& sc, const double (&x)[8], const uint2* __restrict__ frag,
+                                     int lane, bool first, Flush&& flush) {
+    unsigned s[8];
+    Pair p[4];
+    const unsigned how = first ? 3u : sc.shifts(x, s);
+    if (how == 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) p[r].template set<false>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
+    } else {
+        if (how & 2) {
+            if (!first) flush();
+            sc.raise(x);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[k] = shift_word((k & 2) ? sc.E1 : sc.E0, x[k]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) p[r].template set<true>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
+    }
+    mma_step(acc, p, frag, lane);
+}
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool ok) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ double not_a_number() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// v: the sum over orders in units of order 3 (2^72); the scales of A and B are
+// 2^(EA - 1078) and 2^(EB - 1078).  An entry that is not finite has the field
+// 0x7ff: its line's (column's) sums are NaN.
+__device__ __forceinline__ double unscale(double v, int ea, int eb) {
+    if (ea >= 0x7ff || eb >= 0x7ff) return not_a_number();
+    return scale_by(v, 72 + ea + eb - 2156);
+}
+
+// -------------------------------------------------------------------- C = Q^T W
+// Persistent CTAs take chunks of rc rows from a ticket counter: columns c0 ..
+// c0 + 7 of W (n x B) against all m basis columns.  W's digits of a chunk are
+// staged as B fragments; a warp's items are (tile of 16 basis columns, one of
+// `parts` shares of the chunk's steps).  A warp copies its tile's next steps
+// (16 rows, 2 KB) into its ring with cp.async, so that no register holds data
+// in flight; terms 2t, 2t+1, 2t+8, 2t+9 of a step are its rows t, t+4, t+8, t+12,
+// which with the swizzle below makes the fragment reads conflict-free.  An
+// item's sums are added to its CTA's slot (m x B); the slots are summed
+// afterwards in a fixed order (adding every chunk's sums straight to C cost two
+// to three times the FP64 kernels' rounding error).
+template <int B>
+__device__ __forceinline__ int swizzle(int row, int q) {  // 16-byte chunk q of a row of B entries
+    return B == 16 ? q ^ (2 * (row & 3)) : B == 8 ? q ^ (row & 2) : q;
+}
+
+template <int B>
+__global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int rc, int nchunks, int parts,
+                                                          const double* __restrict__ Q, const double* __restrict__ W,
+                                                          double* __restrict__ partial, int* __restrict__ tickets) {
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char* ring = tc_smem + warp * kRing * kStepBytes;
+    uint2* frag = reinterpret_cast<uint2*>(tc_smem + kWarps * kRing * kStepBytes);
+    __shared__ int ew[8];
+    __shared__ int s_chunk;
+    const int g = lane >> 2, t = lane & 3;
+    const int c0 = blockIdx.y * 8;
+    const bool col = c0 + g < B;
+    const int ntiles = (m + 15) / 16, items = ntiles * parts;
+    double* slot = partial + (int64_t)blockIdx.x * m * B;
+    for (int e = tid; e < m * B; e += kT)
+        if (e % B >= c0 && e % B < c0 + 8) slot[e] = 0.0;
+    // a step of a tile in the ring: block-major, then rows of B entries
+    constexpr int CPR = B / 2;                       // 16-byte chunks per row
+    constexpr int CPB = 16 * CPR;                    // chunks per block (B = 2, 4, 8, 16: 16 .. 128)
+    const int ob = (g / B) * 16 * B * 8;             // line g's block, and line g + 8's
+    const int ob8 = ((g + 8) / B) * 16 * B * 8;
+    const int og = g % B, og8 = (g + 8) % B;
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_chunk = atomicAdd(tickets + blockIdx.y, 1);
+        if (tid < 8) ew[tid] = 0;
+        __syncthreads();
+        const int chunk = s_chunk;
+        if (chunk >= nchunks) break;
+        const int64_t r0 = (int64_t)chunk * rc;
+        const int rows = (int)min((int64_t)rc, n - r0);
+        const int steps = (rows + 15) / 16;
+        // the columns' scales, then the digits: a warp per step, a lane's four rows of column c0 + g
+        constexpr int SW = kMaxRows / 16 / kWarps;
+        {
+            double xw[SW][4];
+            int mx = 0;
+#pragma unroll
+            for (int k = 0; k < SW; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = 16 * (warp + k * kWarps) + t + 4 * i;
+                    xw[k][i] = (col && r < rows) ? __ldg(W + (r0 + r) * B + c0 + g) : 0.0;
+                    mx = max(mx, exp_bits(xw[k][i]));
+                }
+#pragma unroll
+            for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
+            __syncthreads();
+            const int eg = max(ew[g], kEmin);
+#pragma unroll
+            for (int k = 0; k < SW; ++k)
+                if (warp + k * kWarps < steps) store_frag(frag + (warp + k * kWarps) * kDig * 32, lane, xw[k], eg);
+        }
+        __syncthreads();
+        const int per = (steps + parts - 1) / parts;
+        for (int w = warp; w < items; w += kWarps) {
+            const int tile = w / parts, part = w % parts;
+            const int s0 = part * per, s1 = min(steps, s0 + per);
+            if (s0 >= s1) continue;
+            const int j0 = 16 * tile / B, nblk = (m - 16 * tile) / B;  // first block and blocks left
+            const bool whole = nblk * B >= 16;
+            const double* p = Q + ((int64_t)j0 * n + r0) * B;
+            auto issue = [&](int s) {
+                if (s < s1) {
+                    unsigned char* buf = ring + (s % kRing) * kStepBytes;
+                    const bool full = whole && 16 * s + 16 <= rows;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int e = lane + 32 * i;
+                        const int j = e / CPB, r = (e % CPB) / CPR, q = e % CPR;
+                        void* dst = buf + (j * CPB + r * CPR + swizzle<B>(r, q)) * 16;
+                        const double* src = p + (int64_t)j * n * B + (16 * s + r) * B + 2 * q;
+                        if (full) cp_async16(dst, src);
+                        else cp_async16(dst, (j < nblk && 16 * s + r < rows) ? src : Q, j < nblk && 16 * s + r < rows);
+                    }
+                }
+                cp_async_commit();
+            };
+#pragma unroll
+            for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
+            Acc acc;
+            acc.clear();
+            LineScale sc;
+            auto flush = [&]() {
+                acc.to_int();
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int a = 16 * tile + g + ((e & 2) ? 8 : 0), c = c0 + 2 * t + (e & 1);
+                    if (a < m && c < B)
+                        atomicAdd(slot + (int64_t)a * B + c,
+                                  unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin)));
+                }
+                acc.clear();
+            };
+            for (int s = s0; s < s1; ++s) {
+                cp_async_wait<kRing - 2>();
+                __syncwarp();
+                issue(s + kRing - 1);  // into the buffer of step s - 1
+                const unsigned char* buf = ring + (s % kRing) * kStepBytes;
+                double x[8];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = t + 4 * i;
+                    const int k = (i >> 1) * 4 + (i & 1);  // register 0 / 2 of line g, 1 / 3 of line g + 8
+                    x[k] = *reinterpret_cast<const double*>(buf + ob + r * B * 8 + swizzle<B>(r, og >> 1) * 16 + (og & 1) * 8);
+                    x[k + 2] = *reinterpret_cast<const double*>(buf + ob8 + r * B * 8 + swizzle<B>(r, og8 >> 1) * 16 + (og8 & 1) * 8);
+                }
+                step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
+                if (((s - s0) & 3) == 3) acc.to_int();
+            }
+            cp_async_wait<0>();
+            __syncwarp();
+            flush();
+        }
+    }
+}
+
+// -------------------------------------------------------------------- W (-)= Q C
+// W[r][c0 .. c0 + 7] (SUB ? -= : =) sum_a Q[r][a] C[a][c], row stride kc of C
+// and W.  A warp takes 16 rows; the digits of up to kMaxCols rows of C are
+// staged as B fragments (in one go, kept over the CTA's row groups, when they
+// are all of C).
+template <int B, bool SUB>
+__global__ void __launch_bounds__(kT, 2) update_tc64_kernel(int64_t n, int m, int kc, int ks, const double* Q,
+                                                            const double* __restrict__ C, double* W) {
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double2* ring = reinterpret_cast<double2*>(tc_smem + warp * kRing * kStepBytes) + lane;
+    uint2* frag = reinterpret_cast<uint2*>(tc_smem + kWarps * kRing * kStepBytes);
+    __shared__ int ew[8];
+    const int g = lane >> 2, t = lane & 3;
+    const int c0 = blockIdx.y * 8;
+    const bool col = c0 + g < kc;
+    // ks warps share a tile of 16 rows, each a share of the steps
+    __shared__ double part[kWarps][4][32];
+    const int tiles = kWarps / ks, sub = warp % ks;
+    const int64_t groups = (n + 16 * tiles - 1) / (16 * tiles);
+    bool staged = false;
+    for (int64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+        const int64_t ra = grp * 16 * tiles + (warp / ks) * 16 + g, rb = ra + 8;
+            double out[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int k0 = 0; k0 < m; k0 += kMaxCols) {
+            const int cols = min(kMaxCols, m - k0), steps = (cols + 15) / 16;
+            if (!staged) {
+                __syncthreads();
+                if (tid < 8) ew[tid] = 0;
+                __syncthreads();
+                int mx = 0;
+                for (int s = warp; s < steps; s += kWarps)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
+                        if (col && a < cols) mx = max(mx, exp_bits(C[(int64_t)(k0 + a) * kc + c0 + g]));
+                    }
+#pragma unroll
+                for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
+                __syncthreads();
+                const int eg = max(ew[g], kEmin);
+                for (int s = warp; s < steps; s += kWarps) {
+                    double x[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
+                        x[i] = (col && a < cols) ? C[(int64_t)(k0 + a) * kc + c0 + g] : 0.0;
+                    }
+                    store_frag(frag + s * kDig * 32, lane, x, eg);
+                }
+                __syncthreads();
+                staged = m <= kMaxCols;
+            }
+            // registers 0, 1: columns 2t, 2t+1 of rows g, g+8; 2, 3: columns 2t+8,
+            // 2t+9.  A lane copies its own 16-byte pairs into its ring and reads them back.
+            const int per = (steps + ks - 1) / ks, s0 = sub * per, s1 = min(steps, s0 + per);
+            const bool rows_in = grp * 16 * tiles + (warp / ks) * 16 + 16 <= n;
+            auto issue = [&](int s) {
+                if (s < s1) {
+                    const bool full = rows_in && k0 + 16 * s + 16 <= m;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int a = k0 + 16 * s + 8 * (i >> 1) + 2 * t;
+                        const int64_t r = (i & 1) ? rb : ra;
+                        const double* src = Q + ((int64_t)(a / B) * n + r) * B + a % B;
+                        double2* dst = ring + (s % kRing) * 128 + i * 32;
+                        if (full) cp_async16(dst, src);
+                        else cp_async16(dst, (a < m && r < n) ? src : Q, a < m && r < n);
+                    }
+                }
+                cp_async_commit();
+            };
+#pragma unroll
+            for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
+            Acc acc;
+            acc.clear();
+            LineScale sc;
+            auto flush = [&]() {
+                acc.to_int();
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    out[e] += unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin));
+                acc.clear();
+            };
+            for (int s = s0; s < s1; ++s) {
+                cp_async_wait<kRing - 2>();
+                double x[8];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double2 v = ring[(s % kRing) * 128 + i * 32];
+                    x[2 * i] = v.x;
+                    x[2 * i + 1] = v.y;
+                }
+                issue(s + kRing - 1);  // into the buffer of step s - 1
+                step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
+                if (((s - s0) & 3) == 3) acc.to_int();
+            }
+            cp_async_wait<0>();
+            if (s0 < s1) flush();
+        }
+        if (ks > 1) {
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) part[warp][e][lane] = out[e];
+            __syncthreads();
+            if (sub != 0) continue;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                for (int q = 1; q < ks; ++q) out[e] += part[warp + q][e][lane];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int64_t r = (e & 2) ? rb : ra;
+            const int c = c0 + 2 * t + (e & 1);
+            if (r < n && c < kc) {
+                double* w = W + r * kc + c;
+                *w = SUB ? *w - out[e] : out[e];
+            }
+        }
+    }
+}
+
+int sms() {
+    static int n = 0;
+    if (n == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
+    }
+    return n;
+}
+
+// Shares of a chunk's steps per tile: the fewest rounds of steps over the
+// CTA's warps, counting an item's end (its FP64 conversions) as two steps.
+int gram_parts(int ntiles, int steps) {
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int p = 1; p <= kWarps && p <= steps; p <<= 1) {
+        const int64_t c = ceil_div((int64_t)ntiles * p, kWarps) * (ceil_div(steps, p) + 2);
+        if (c < cost) {
+            cost = c;
+            best = p;
+        }
+    }
+    return best;
+}
+
+constexpr int kFragBytes = kDig * 32 * (int)sizeof(uint2);  // a step's B fragments
+constexpr int kRingBytes = kWarps * kRing * kStepBytes;
+
+template <int B>
+bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, double* C, DevBuf& partials, cudaStream_t st) {
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(gram_tc64_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kRingBytes + kMaxRows / 16 * kFragBytes));
+        attr = true;
+    }
+    constexpr int NH = (B + 7) / 8;
+    // rows per chunk: at least two chunks per SM where n allows it, at most the staged 512
+    int64_t rc = ceil_div(ceil_div(n, (int64_t)2 * sms()), 64) * 64;
+    rc = std::min<int64_t>(std::max<int64_t>(rc, 64), kMaxRows);
+    const int parts = gram_parts((m + 15) / 16, (int)rc / 16);
+    const int64_t chunks = ceil_div(n, rc);
+    const int64_t ctas = std::min<int64_t>(chunks, (int64_t)2 * gram_worker_sms());
+    const int64_t per = (int64_t)m * B;
+    BBL_TRY(partials.grow(sizeof(double) * (size_t)(ctas * per) + 256));
+    int* tickets = reinterpret_cast<int*>(partials.as<double>() + ctas * per);
+    BBL_CUDA(cudaMemsetAsync(tickets, 0, sizeof(int) * NH, st));
+    gram_tc64_kernel<B><<<dim3((unsigned)ctas, NH), kT, kRingBytes + (size_t)(rc / 16) * kFragBytes, st>>>(
+        n, m, (int)rc, (int)chunks, parts, Q, W, partials.as<double>(), tickets);
+    BBL_LAUNCH_CHECK();
+    reduce_partials(per, (int)ctas, partials.as<double>(), C, st);
+    BBL_LAUNCH_CHECK();
+    return BBL_OK;
+}
+
+template <int B, bool SUB>
+bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double* C, double* W, cudaStream_t st) {
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(update_tc64_kernel<B, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kRingBytes + kMaxCols / 16 * kFragBytes));
+        attr = true;
+    }
+    // few rows: up to eight warps share a row tile's steps, so that the SMs' 16
+    // warps have work
+    const int64_t rtiles = ceil_div(n, 16);
+    const int cols = std::min(m, kMaxCols), steps = (cols + 15) / 16;
+    int ks = 1;
+    while (ks < kWarps && rtiles * ks * 2 <= (int64_t)sms() * 2 * kWarps && steps >= ks * 4) ks <<= 1;
+    const int64_t groups = ceil_div(rtiles, kWarps / ks);
+    const dim3 grid((unsigned)std::min<int64_t>(groups, (int64_t)sms() * 8), (unsigned)((kc + 7) / 8));
+    update_tc64_kernel<B, SUB><<<grid, kT, kRingBytes + (size_t)steps * kFragBytes, st>>>(n, m, kc, ks, Q, C, W);
+    BBL_LAUNCH_CHECK();
+    return BBL_OK;
+}
+
+}  // namespace
+
+// Measured against the FP64 FMA kernels (GB300): at b >= 4 the split is faster
+// from 16 columns on (n = 1e6, b = 8, m = 80: Gram 1592 us, update 1052 us);
+// with one block (m = 8) half of each tile is padding and the operands' own
+// split is not shared by many columns, and with b = 1 (Gram, update) and
+// b = 2 (update) the FMA kernels have no more than two products per entry.
+bool tc64_gram_supports(int b, int m) { return (b == 2 && m >= 32) || ((b == 4 || b == 8 || b == 16) && m >= 16); }
+bool tc64_update_supports(int b, int m) { return (b == 4 || b == 8 || b == 16) && m >= 16; }
+
+bbl_status gram_tc64(int64_t n, int b, int m, const double* Q, const double* W, double* C, DevBuf& partials,
+                     cudaStream_t st) {
+    switch (b) {
+        case 2: return launch_gram<2>(n, m, Q, W, C, partials, st);
+        case 4: return launch_gram<4>(n, m, Q, W, C, partials, st);
+        case 8: return launch_gram<8>(n, m, Q, W, C, partials, st);
+        default: return launch_gram<16>(n, m, Q, W, C, partials, st);
+    }
+}
+
+bbl_status update_tc64(int64_t n, int b, int m, int kc, const double* Q, const double* C, double* W, bool sub,
+                       cudaStream_t st) {
+    switch (b) {
+        case 4: return sub ? launch_update<4, true>(n, m, kc, Q, C, W, st) : launch_update<4, false>(n, m, kc, Q, C, W, st);
+        case 8: return sub ? launch_update<8, true>(n, m, kc, Q, C, W, st) : launch_update<8, false>(n, m, kc, Q, C, W, st);
+        default: return sub ? launch_update<16, true>(n, m, kc, Q, C, W, st) : launch_update<16, false>(n, m, kc, Q, C, W, st);
+    }
+}
+
+}  // namespace bbl
