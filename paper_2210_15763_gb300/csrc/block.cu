@@ -13,8 +13,9 @@
 //  apply    W (-)= Q C  (thread per row; C staged in shared memory in
 //                        256-row tiles; used for the Gram-Schmidt update, for
 //                        W R^{-1} in CholQR2 and for the Ritz vectors X = Q S).
-//  cholqr2  G = W^T W -> R = chol(G) (one thread, b <= 16) -> W <- W R^{-1},
-//           twice; B = R2 R1 (Sec. II.B normalisation, CholQR2 form).
+//  cholqr2  G = W^T W -> R = chol(G) (one CTA, b <= 16) -> W <- W R^{-1},
+//           twice, the first R^{-1} applied in the pass that forms the second
+//           G; B = R2 R1 (Sec. II.B normalisation, CholQR2 form).
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -76,6 +77,48 @@ __device__ __forceinline__ void ldvec(const T* p, T (&out)[N]) {
     } else {
 #pragma unroll
         for (int q = 0; q < N; ++q) out[q] = __ldg(p + q);
+    }
+}
+
+// the same loads for memory the kernel also writes, and the stores
+template <typename T, int N>
+__device__ __forceinline__ void ldvec_rw(const T* p, T (&out)[N]) {
+    if constexpr (is_df32<T>::value && N == 2) {
+        const float4 x = *reinterpret_cast<const float4*>(p);
+        out[0] = df32(x.x, x.y);
+        out[1] = df32(x.z, x.w);
+    } else if constexpr (!is_df32<T>::value && N * sizeof(T) == 16 && sizeof(T) == 8) {
+        const double2 x = *reinterpret_cast<const double2*>(p);
+        out[0] = x.x;
+        out[1] = x.y;
+    } else if constexpr (N * sizeof(T) == 16 && sizeof(T) == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(p);
+        out[0] = x.x;
+        out[1] = x.y;
+        out[2] = x.z;
+        out[3] = x.w;
+    } else if constexpr (N * sizeof(T) == 8 && sizeof(T) == 4) {
+        const float2 x = *reinterpret_cast<const float2*>(p);
+        out[0] = x.x;
+        out[1] = x.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) out[q] = p[q];
+    }
+}
+template <typename T, int N>
+__device__ __forceinline__ void stvec(T* p, const T (&v)[N]) {
+    if constexpr (is_df32<T>::value && N == 2) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo);
+    } else if constexpr (!is_df32<T>::value && N * sizeof(T) == 16 && sizeof(T) == 8) {
+        *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+    } else if constexpr (N * sizeof(T) == 16 && sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (N * sizeof(T) == 8 && sizeof(T) == 4) {
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) p[q] = v[q];
     }
 }
 
@@ -585,130 +628,182 @@ __global__ void __launch_bounds__(kThreads) gram_generic_kernel(int64_t n, int m
     }
 }
 
-// out[e] = sum_p partial[p * count + e]: 32 entries per CTA, the parts split
-// over 8 warps (coalesced 256-byte rows), combined in a fixed order.
-__global__ void __launch_bounds__(256) reduce_partials_kernel(int64_t count, int nparts,
-                                                              const double* __restrict__ partial,
-                                                              double* __restrict__ out) {
-    __shared__ double red[8][33];
-    const int tx = threadIdx.x & 31, pg = threadIdx.x >> 5;
-    const int64_t e = (int64_t)blockIdx.x * 32 + tx;
-    double s = 0.0;
-    if (e < count) {
-        int p = pg;
-        for (; p + 24 < nparts; p += 32) {
-            const double a0 = partial[(int64_t)p * count + e];
-            const double a1 = partial[(int64_t)(p + 8) * count + e];
-            const double a2 = partial[(int64_t)(p + 16) * count + e];
-            const double a3 = partial[(int64_t)(p + 24) * count + e];
-            s += a0;
-            s += a1;
-            s += a2;
-            s += a3;
-        }
-        for (; p < nparts; p += 8) s += partial[(int64_t)p * count + e];
+// out[e] = sum_p partial[p * count + e]: 8 entries per CTA (64-byte rows), the
+// parts split over 32 groups of threads whose loads are issued together,
+// combined in a fixed order.  (With 32 entries and 8 groups a thread added 38
+// to 76 parts in turn: 8 to 9 us for the 304 to 608 parts of a Gram, most of it
+// load latency.)
+constexpr int kRedE = 8, kRedG = kThreads / kRedE;
+__device__ __forceinline__ double sum_parts(int64_t count, int nparts, const double* __restrict__ partial, int64_t e,
+                                            int g, int groups) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int p = g;
+    for (; p + 7 * groups < nparts; p += 8 * groups) {
+        double a[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a[q] = partial[(int64_t)(p + q * groups) * count + e];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s[q & 3] += a[q];
     }
-    red[pg][tx] = s;
+    for (; p < nparts; p += groups) s[0] += partial[(int64_t)p * count + e];
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+__global__ void __launch_bounds__(kThreads) reduce_partials_kernel(int64_t count, int nparts,
+                                                                   const double* __restrict__ partial,
+                                                                   double* __restrict__ out) {
+    __shared__ double red[kRedG][kRedE];
+    const int tx = threadIdx.x % kRedE, pg = threadIdx.x / kRedE;
+    const int64_t e = (int64_t)blockIdx.x * kRedE + tx;
+    red[pg][tx] = e < count ? sum_parts(count, nparts, partial, e, pg, kRedG) : 0.0;
     __syncthreads();
-    if (pg == 0 && e < count) {
-        double t = red[0][tx];
-        for (int q = 1; q < 8; ++q) t += red[q][tx];
-        out[e] = t;
+    for (int w = kRedG / 2; w > 0; w >>= 1) {
+        if (pg < w) red[pg][tx] += red[pg + w][tx];
+        __syncthreads();
     }
+    if (pg == 0 && e < count) out[e] = red[0][tx];
 }
 
 void launch_reduce(int64_t count, int nparts, const double* partial, double* out, cudaStream_t st) {
-    reduce_partials_kernel<<<(unsigned)ceil_div(count, 32), 256, 0, st>>>(count, nparts, partial, out);
+    reduce_partials_kernel<<<(unsigned)ceil_div(count, kRedE), kThreads, 0, st>>>(count, nparts, partial, out);
 }
 
-// Self Gram G = W^T W for b <= 8 (CholQR2): a thread per row (grid-strided),
-// the b(b+1)/2 distinct products in registers, then a warp-shuffle and
-// shared-memory reduction to one B x B partial per CTA.
-template <typename T, int B>
-__global__ void __launch_bounds__(kThreads) syrk_kernel(int64_t n, const T* __restrict__ W, double* __restrict__ partial) {
+// Sums v[0 .. N-1] over the warp and hands each sum to put(index, sum) in one
+// lane: every round a lane keeps half of its values and sends the other half (37
+// additions for N = 36 where an all-reduce of each value takes 180; the same
+// pairs are added, so the sums are the same).
+template <int N, typename T, typename Put>
+__device__ __forceinline__ void warp_sum_scatter(T (&v)[N], Put&& put) {
+    const int lane = threadIdx.x & 31;
+    int cnt = N, base = 0, lim = N;  // values held (padded with zeros), index of the first, valid ones
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool up = (lane & off) != 0;
+        const int hv = (cnt + 1) / 2;
+#pragma unroll
+        for (int x = 0; x < (N + 1) / 2; ++x) {
+            if (x < hv) {
+                const T hi = x + hv < cnt ? v[x + hv < N ? x + hv : 0] : T(0);
+                const T send = up ? v[x] : hi, keep = up ? hi : v[x];
+                v[x] = add_any(keep, shfl_xor_any(0xffffffffu, send, off));
+            }
+        }
+        base += up ? hv : 0;
+        lim = up ? max(lim - hv, 0) : min(lim, hv);
+        cnt = hv;
+    }
+    constexpr int K = (N + 31) / 32;
+#pragma unroll
+    for (int x = 0; x < K; ++x)
+        if (x < lim) put(base + x, v[x]);
+}
+
+// One pass of CholQR2 over W (n x B, B <= 8), a thread per row (grid-strided,
+// the next row's loads issued before the current row's arithmetic): APPLY:
+// W <- W R^{-1} (upper triangular: c takes i <= c); GRAM: the partial Gram of
+// the rows as stored, the B(B+1)/2 distinct products in registers, then a
+// warp-shuffle and shared-memory reduction to one B x B partial per CTA.
+// Applying the first factor and forming the second Gram in one pass saves a
+// read of W and a launch.
+// LONG: a lane sees more than 64 rows, and runs of 64 are summed in FP64 (their
+// sums cost 72 registers at b = 8, and with them all but one CTA per SM).
+template <typename T, int B, bool APPLY, bool GRAM, bool LONG = false>
+__global__ void __launch_bounds__(kThreads) qr_pass_kernel(int64_t n, const double* __restrict__ Rinv, T* W,
+                                                           double* __restrict__ partial) {
     constexpr int NP = B * (B + 1) / 2;
-    __shared__ double red[kThreads / 32][NP];
-    T acc[NP];
+    __shared__ double red[GRAM ? kThreads / 32 : 1][NP];
+    __shared__ T rs[B * B];
+    if constexpr (APPLY) {
+        for (int e = threadIdx.x; e < B * B; e += kThreads) rs[e] = (T)Rinv[e];
+        __syncthreads();
+    }
+    T acc[GRAM ? NP : 1];
+    double acc64[LONG ? NP : 1];
 #pragma unroll
-    for (int e = 0; e < NP; ++e) acc[e] = T(0);
-    double acc64[NP];
+    for (int e = 0; e < (GRAM ? NP : 1); ++e) acc[e] = T(0);
 #pragma unroll
-    for (int e = 0; e < NP; ++e) acc64[e] = 0.0;
+    for (int e = 0; e < (LONG ? NP : 1); ++e) acc64[e] = 0.0;
     int cnt = 0;
-    for (int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x; r < n; r += (int64_t)gridDim.x * kThreads) {
+    constexpr int CH = B * sizeof(T) >= 16 ? 16 / (int)sizeof(T) : B;  // elements per load
+    auto load = [&](int64_t r, T (&w)[B]) {
+#pragma unroll
+        for (int ch = 0; ch < B / CH; ++ch) {
+            T t[CH];
+            ldvec_rw<T, CH>(W + r * B + ch * CH, t);
+#pragma unroll
+            for (int q = 0; q < CH; ++q) w[ch * CH + q] = t[q];
+        }
+    };
+    const int64_t stride = (int64_t)gridDim.x * kThreads;
+    int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    T nx[B];
+    if (r < n) load(r, nx);
+    for (; r < n; r += stride) {
         T w[B];
-        if constexpr (B * sizeof(T) >= 16) {
-            constexpr int CH = 16 / (int)sizeof(T);
+#pragma unroll
+        for (int c = 0; c < B; ++c) w[c] = nx[c];
+        if (r + stride < n) load(r + stride, nx);
+        if constexpr (APPLY) {
+            T v[B];
+#pragma unroll
+            for (int c = 0; c < B; ++c) v[c] = T(0);
+#pragma unroll
+            for (int i = 0; i < B; ++i)
+#pragma unroll
+                for (int c = i; c < B; ++c) v[c] = fma(w[i], rs[i * B + c], v[c]);
+#pragma unroll
+            for (int c = 0; c < B; ++c) w[c] = v[c];
 #pragma unroll
             for (int ch = 0; ch < B / CH; ++ch) {
                 T t[CH];
-                ldvec<T, CH>(W + r * B + ch * CH, t);
 #pragma unroll
-                for (int q = 0; q < CH; ++q) w[ch * CH + q] = t[q];
+                for (int q = 0; q < CH; ++q) t[q] = w[ch * CH + q];
+                stvec<T, CH>(W + r * B + ch * CH, t);
             }
-        } else {
-            ldvec<T, B>(W + r * B, w);
         }
-        int e = 0;
+        if constexpr (GRAM) {
+            int e = 0;
 #pragma unroll
-        for (int i = 0; i < B; ++i)
+            for (int i = 0; i < B; ++i)
 #pragma unroll
-            for (int k = i; k < B; ++k) {
-                acc[e] = fma(w[i], w[k], acc[e]);
-                ++e;
+                for (int k = i; k < B; ++k) {
+                    acc[e] = fma(w[i], w[k], acc[e]);
+                    ++e;
+                }
+            if (LONG && ++cnt == 64) {  // FP32 runs of at most 64 rows, summed in FP64
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    acc64[LONG ? q : 0] += (double)acc[q];
+                    acc[q] = T(0);
+                }
+                cnt = 0;
             }
-        if (++cnt == 64) {  // FP32 runs of at most 64 rows, summed in FP64
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                acc64[q] += (double)acc[q];
-                acc[q] = T(0);
-            }
-            cnt = 0;
         }
     }
-    // warp tree in the data type (FP32 sums of at most 64 rows per lane,
-    // then 32 lanes); the FP64 flushes only exist when a lane saw more rows
-    const bool flushed = n > (int64_t)64 * gridDim.x * kThreads;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        T vt = acc[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) vt = add_any(vt, shfl_xor_any(0xffffffffu, vt, off));
-        double v = (double)vt;
-        if (flushed) {
-            double v64 = acc64[q];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v64 += __shfl_xor_sync(0xffffffffu, v64, off);
-            v += v64;
+    if constexpr (GRAM) {
+        // warp tree in the data type (FP32 sums of at most 64 rows per lane,
+        // then 32 lanes)
+        const int warp = threadIdx.x / 32;
+        warp_sum_scatter<NP>(acc, [&](int q, T v) { red[warp][q] = (double)v; });
+        if constexpr (LONG) {
+            __syncwarp();
+            warp_sum_scatter<NP>(acc64, [&](int q, double v) { red[warp][q] += v; });
         }
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32][q] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NP) {
-        double v = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) v += red[w][threadIdx.x];
-        // unpack the upper-triangle index into (i, k) and store both halves
-        int i = 0, e = threadIdx.x;
-        while (e >= B - i) {
-            e -= B - i;
-            ++i;
+        __syncthreads();
+        if (threadIdx.x < NP) {
+            double v = 0.0;
+            for (int w = 0; w < kThreads / 32; ++w) v += red[w][threadIdx.x];
+            // unpack the upper-triangle index into (i, k) and store both halves
+            int i = 0, e = threadIdx.x;
+            while (e >= B - i) {
+                e -= B - i;
+                ++i;
+            }
+            const int k = i + e;
+            partial[(int64_t)blockIdx.x * B * B + i * B + k] = v;
+            partial[(int64_t)blockIdx.x * B * B + k * B + i] = v;
         }
-        const int k = i + e;
-        partial[(int64_t)blockIdx.x * B * B + i * B + k] = v;
-        partial[(int64_t)blockIdx.x * B * B + k * B + i] = v;
     }
-}
-
-template <typename T, int B>
-bbl_status launch_syrk(int64_t n, const T* W, double* G, DevBuf& partials, cudaStream_t st) {
-    const int grid = (int)std::min<int64_t>(152 * 4, std::max<int64_t>(1, ceil_div(n, kThreads)));
-    const size_t need = sizeof(double) * (size_t)grid * B * B;
-    BBL_TRY(partials.grow(need));
-    syrk_kernel<T, B><<<grid, kThreads, 0, st>>>(n, W, partials.as<double>());
-    BBL_LAUNCH_CHECK();
-    launch_reduce((int64_t)B * B, grid, partials.as<double>(), G, st);
-    BBL_LAUNCH_CHECK();
-    return BBL_OK;
 }
 
 int sm_count() {
@@ -1462,80 +1557,127 @@ __device__ void chol_body(int b, const double* __restrict__ G, double thresh2, i
     if (bad && status) atomicOr(status, 1);
 }
 
-// The same Cholesky with deflation by one warp: rows of R are formed one
-// after the other (lane k computes R[i][k]), then lane c forms column c of
-// R^{-1}.  Deflated columns get zero rows in R and zero columns in R^{-1}.
-__global__ void __launch_bounds__(32) chol_warp_kernel(int b, const double* __restrict__ G, double thresh2, int relative,
-                                                      double* __restrict__ R, double* __restrict__ Rinv,
-                                                      int* __restrict__ ndefl, int* __restrict__ mask,
-                                                      int* __restrict__ status) {
-    __shared__ double Gs[kMaxB * kMaxB];
-    __shared__ double Rs[kMaxB * kMaxB];
-    __shared__ int dm[kMaxB];
-    const int lane = threadIdx.x;
-    int bad = 0;
-    double gmax = 0.0;
-    for (int e = lane; e < b * b; e += 32) {
-        const double g = G[e];
-        Gs[e] = g;
-        Rs[e] = 0.0;
-        if (!isfinite(g)) bad = 1;
-    }
-    bad = __any_sync(0xffffffffu, bad);
-    __syncwarp();
-    for (int q = 0; q < b; ++q) gmax = fmax(gmax, Gs[q * b + q]);
-    if (relative) thresh2 *= gmax;
-    int cnt = 0;
-    for (int i = 0; i < b; ++i) {
-        double d = Gs[i * b + i];
-        for (int l = 0; l < i; ++l) d -= Rs[l * b + i] * Rs[l * b + i];
-        const int defl = !(d > thresh2) || bad;
-        cnt += defl;
-        if (lane == 0) dm[i] = defl;
-        if (!defl) {
-            const double rii = sqrt(d);
-            if (lane == i) Rs[i * b + i] = rii;
-            if (lane > i && lane < b) {
-                double t = Gs[i * b + lane];
-                for (int l = 0; l < i; ++l) t -= Rs[l * b + i] * Rs[l * b + lane];
-                Rs[i * b + lane] = t / rii;
-            }
-        }
-        __syncwarp();
-    }
-    for (int e = lane; e < b * b; e += 32) R[e] = Rs[e];
-    if (lane < b) {
-        const int c = lane;
-        double col[kMaxB];
-#pragma unroll
-        for (int q = 0; q < kMaxB; ++q) col[q] = 0.0;
-        if (!dm[c]) {
-            col[c] = 1.0 / Rs[c * b + c];
-            for (int i = c - 1; i >= 0; --i) {
-                if (dm[i]) continue;
-                double t = 0.0;
-                for (int k = i + 1; k <= c; ++k)
-                    if (!dm[k]) t += Rs[i * b + k] * col[k];
-                col[i] = -t / Rs[i * b + i];
-            }
-        }
-        for (int q = 0; q < b; ++q) Rinv[q * b + c] = col[q];
-        if (mask) mask[c] = dm[c];
-    }
-    if (lane == 0) {
-        if (ndefl) *ndefl += cnt;
-        if (bad && status) atomicOr(status, 1);
-    }
+// 1 / d of a normal finite d, to about one unit in the last place: an FP32
+// seed on the mantissa and two Newton steps (four FP64 instructions in a chain;
+// an FP64 instruction occupies its scheduler for 64 cycles here, and the
+// division takes about ten).
+__device__ __forceinline__ double recip(double d) {
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+    if (ex < 64 || ex > 1980) return 1.0 / d;
+    const double m = __hiloint2double(hi - (ex - 1023) * (1 << 20), __double2loint(d));
+    double y = (double)__frcp_rn((float)m);
+    y = fma(y, fma(-m, y, 1.0), y);
+    y = fma(y, fma(-m, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - (ex - 1023) * (1 << 20), __double2loint(y));
 }
 
-// B = R2 R1 (upper triangular product)
-__global__ void trmul_kernel(int b, const double* __restrict__ R2, const double* __restrict__ R1, double* __restrict__ B) {
-    const int e = threadIdx.x;
-    if (e >= b * b) return;
-    const int i = e / b, k = e % b;
-    double s = 0.0;
-    for (int l = 0; l < b; ++l) s += R2[i * b + l] * R1[l * b + k];
-    B[e] = s;
+constexpr int kCholThreads = 256;
+constexpr int kCholParts = 128;  // most partial Grams one CTA adds itself (two FP64 additions per cycle)
+
+// The Cholesky step of CholQR2 by one CTA: G = the sum of nparts partial b x b
+// Grams, R = chol(G) with deflation and R^{-1}, and, with Bout, B = R R1.
+// G = L D L^T right-looking by one warp, whose lanes keep the entries of G and of
+// L^{-1} in registers: a step is one reciprocal, one product and one update deep;
+// the square roots (R = D^{1/2} L^T) follow together.  Deflated columns get zero
+// rows in R and zero columns in R^{-1}.
+__global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, const double* __restrict__ partial,
+                                                            double thresh2, int relative, double* __restrict__ R,
+                                                            double* __restrict__ Rinv, int* __restrict__ ndefl,
+                                                            int* __restrict__ mask, int* __restrict__ status,
+                                                            const double* __restrict__ R1, double* __restrict__ Bout) {
+    __shared__ double Gs[kMaxB * kMaxB];
+    __shared__ double Ls[kMaxB * kMaxB];  // row k: L[.][k] = R[k][.] / sqrt(d_k)
+    __shared__ double Zs[kMaxB * kMaxB];  // row k of L^{-1}
+    __shared__ double row[2][2][kMaxB];   // row k of the Schur complement and of L^{-1}
+    __shared__ double dk[kMaxB], root[kMaxB];
+    __shared__ double red[kCholThreads];
+    __shared__ int dm[kMaxB];
+    const int tid = threadIdx.x, bb = b * b;
+    {  // groups of bb threads add the parts
+        const int groups = kCholThreads / bb, e = tid % bb, g = tid / bb;
+        red[tid] = g < groups ? sum_parts(bb, nparts, partial, e, g, groups) : 0.0;
+        __syncthreads();
+        if (tid < bb) {
+            double s = red[tid];
+            for (int q = 1; q < groups; ++q) s += red[tid + q * bb];
+            Gs[tid] = s;
+        }
+        __syncthreads();
+    }
+    if (tid < 32) {
+        const int lane = tid;
+        constexpr int E = kMaxB * kMaxB / 32;
+        double a[E], z[E];
+        int ei[E], ec[E];
+        int bad = 0;
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            const int q = lane + 32 * x;
+            ei[x] = q < bb ? q / b : -1;
+            ec[x] = q < bb ? q - ei[x] * b : 0;
+            a[x] = q < bb ? Gs[q] : 0.0;
+            z[x] = ei[x] == ec[x] ? 1.0 : 0.0;
+            if (!isfinite(a[x])) bad = 1;
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        double gmax = 0.0;
+        for (int q = 0; q < b; ++q) gmax = fmax(gmax, Gs[q * b + q]);
+        if (relative) thresh2 *= gmax;
+        int cnt = 0;
+#pragma unroll
+        for (int x = 0; x < E; ++x)
+            if (ei[x] == 0) {
+                row[0][0][ec[x]] = a[x];
+                row[0][1][ec[x]] = z[x];
+            }
+        __syncwarp();
+        for (int k = 0; k < b; ++k) {
+            const double* ra = row[k & 1][0];
+            const double* rz = row[k & 1][1];
+            const double d = ra[k];
+            const int defl = !(d > thresh2) || bad;
+            cnt += defl;
+            const double y = defl ? 0.0 : recip(d);
+            if (lane == 0) {
+                dm[k] = defl;
+                dk[k] = defl ? 0.0 : d;
+            }
+            if (lane < b) {
+                Ls[k * b + lane] = lane < k || defl ? 0.0 : ra[lane] * y;
+                Zs[k * b + lane] = lane > k || defl ? 0.0 : rz[lane];
+            }
+#pragma unroll
+            for (int x = 0; x < E; ++x) {
+                if (32 * x < bb && ei[x] > k) {
+                    const double l = ra[ei[x]] * y;
+                    if (ec[x] >= ei[x]) a[x] = fma(-l, ra[ec[x]], a[x]);
+                    if (ec[x] <= k && !defl) z[x] = fma(-l, rz[ec[x]], z[x]);
+                    if (ei[x] == k + 1) {
+                        row[(k + 1) & 1][0][ec[x]] = a[x];
+                        row[(k + 1) & 1][1][ec[x]] = z[x];
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        if (lane < b) root[lane] = sqrt(dk[lane]);
+        if (lane == 0) {
+            if (ndefl) *ndefl += cnt;
+            if (bad && status) atomicOr(status, 1);
+        }
+    }
+    __syncthreads();
+    if (tid < bb) {
+        const int i = tid / b, c = tid % b;
+        R[tid] = Ls[tid] * root[i];
+        Rinv[tid] = c >= i && !dm[c] ? Zs[c * b + i] / root[c] : 0.0;
+        if (Bout) {
+            double s = 0.0;
+            for (int l = i; l <= c; ++l) s += Ls[i * b + l] * root[i] * R1[l * b + c];
+            Bout[tid] = s;
+        }
+    }
+    if (mask && tid < b) mask[tid] = dm[tid];
 }
 
 }  // namespace
@@ -1627,40 +1769,46 @@ bbl_status ritz_vectors(int64_t n, int b, int nblocks, int dtype, const void* Q,
     return apply_typed<float, false, float, double>(n, b, m, k, static_cast<const float*>(Q), S, X, st);
 }
 
-// small: >= 8*b*b doubles + 4*b ints.  B (device, b x b) receives R2 R1.
-// G = W^T W (b x b): the dedicated kernel for b in {1, 2, 4, 8}, else the general Gram.
-bbl_status self_gram(int64_t n, int b, int dtype, const void* W, double* G, DevBuf& partials, cudaStream_t st) {
-    if (dtype == BBL_FP64) {
-        auto w = static_cast<const double*>(W);
-        switch (b) {
-            case 1: return launch_syrk<double, 1>(n, w, G, partials, st);
-            case 2: return launch_syrk<double, 2>(n, w, G, partials, st);
-            case 4: return launch_syrk<double, 4>(n, w, G, partials, st);
-            case 8: return launch_syrk<double, 8>(n, w, G, partials, st);
-            default: break;
-        }
-    } else if (dtype == kDF32) {
-        auto w = static_cast<const df32*>(W);
-        switch (b) {
-            case 1: return launch_syrk<df32, 1>(n, w, G, partials, st);
-            case 2: return launch_syrk<df32, 2>(n, w, G, partials, st);
-            case 4: return launch_syrk<df32, 4>(n, w, G, partials, st);
-            case 8: return launch_syrk<df32, 8>(n, w, G, partials, st);
-            default: break;
-        }
+// One pass over W for b in {1, 2, 4, 8}: W <- W Rinv (Rinv not NULL), then with
+// gram the partial Grams of the result; *nparts of them in partials.
+template <typename T, int B>
+bbl_status launch_qr_pass(int64_t n, const double* Rinv, T* W, bool gram, DevBuf& partials, int* nparts,
+                          cudaStream_t st) {
+    const int grid = (int)std::min<int64_t>(152 * 4, std::max<int64_t>(1, ceil_div(n, kThreads)));
+    if (gram) {
+        BBL_TRY(partials.grow(sizeof(double) * (size_t)grid * B * B));
+        *nparts = grid;
+        const bool lng = n > (int64_t)64 * grid * kThreads;
+        double* out = partials.as<double>();
+        if (Rinv && lng) qr_pass_kernel<T, B, true, true, true><<<grid, kThreads, 0, st>>>(n, Rinv, W, out);
+        else if (Rinv) qr_pass_kernel<T, B, true, true><<<grid, kThreads, 0, st>>>(n, Rinv, W, out);
+        else if (lng) qr_pass_kernel<T, B, false, true, true><<<grid, kThreads, 0, st>>>(n, Rinv, W, out);
+        else qr_pass_kernel<T, B, false, true><<<grid, kThreads, 0, st>>>(n, Rinv, W, out);
     } else {
-        auto w = static_cast<const float*>(W);
-        switch (b) {
-            case 1: return launch_syrk<float, 1>(n, w, G, partials, st);
-            case 2: return launch_syrk<float, 2>(n, w, G, partials, st);
-            case 4: return launch_syrk<float, 4>(n, w, G, partials, st);
-            case 8: return launch_syrk<float, 8>(n, w, G, partials, st);
-            default: break;
-        }
+        const int g2 = (int)std::min<int64_t>(152 * 8, std::max<int64_t>(1, ceil_div(n, kThreads)));
+        qr_pass_kernel<T, B, true, false><<<g2, kThreads, 0, st>>>(n, Rinv, W, nullptr);
     }
-    return gram(n, b, 1, dtype, W, W, G, partials, st);
+    BBL_LAUNCH_CHECK();
+    return BBL_OK;
 }
 
+template <typename T>
+bbl_status qr_pass_typed(int64_t n, int b, const double* Rinv, T* W, bool want_gram, DevBuf& partials,
+                         int* nparts, cudaStream_t st) {
+    switch (b) {
+        case 1: return launch_qr_pass<T, 1>(n, Rinv, W, want_gram, partials, nparts, st);
+        case 2: return launch_qr_pass<T, 2>(n, Rinv, W, want_gram, partials, nparts, st);
+        case 4: return launch_qr_pass<T, 4>(n, Rinv, W, want_gram, partials, nparts, st);
+        case 8: return launch_qr_pass<T, 8>(n, Rinv, W, want_gram, partials, nparts, st);
+        default: break;
+    }
+    // other b: the general update; the caller forms the Gram (nparts 0)
+    if (Rinv) BBL_TRY((apply_typed<T, false, T, T>(n, b, b, b, W, Rinv, W, st)));
+    *nparts = 0;
+    return BBL_OK;
+}
+
+// small: >= 8*b*b doubles + 4*b ints.  B (device, b x b) receives R2 R1.
 bbl_status cholqr2_dev(int64_t n, int b, int dtype, void* W, double* B, double defl_abs2, int* d_ndefl, int* d_mask,
                        DevBuf& partials, DevBuf& small, cudaStream_t st) {
     const size_t need = sizeof(double) * 8 * kMaxB * kMaxB + sizeof(int) * 4 * kMaxB;
@@ -1673,37 +1821,42 @@ bbl_status cholqr2_dev(int64_t n, int b, int dtype, void* W, double* B, double d
     int* status = reinterpret_cast<int*>(G + 8 * kMaxB * kMaxB);
     const int relative = defl_abs2 < 0 ? 1 : 0;
     const double t1 = relative ? -defl_abs2 : defl_abs2;
-    BBL_TRY(self_gram(n, b, dtype, W, G, partials, st));
-    chol_warp_kernel<<<1, 32, 0, st>>>(b, G, t1, relative, R1, R1i, d_ndefl, d_mask, status);
+    // W <- W Rinv (if given), then the Gram of W (if wanted): its partial sums, or
+    // G itself (many partial sums are added by more than one CTA)
+    const double* gsum = nullptr;
+    int nparts = 0;
+    auto pass = [&](const double* Rinv, bool want_gram) -> bbl_status {
+        if (dtype == BBL_FP64)
+            BBL_TRY(qr_pass_typed<double>(n, b, Rinv, static_cast<double*>(W), want_gram, partials, &nparts, st));
+        else if (dtype == kDF32)
+            BBL_TRY(qr_pass_typed<df32>(n, b, Rinv, static_cast<df32*>(W), want_gram, partials, &nparts, st));
+        else
+            BBL_TRY(qr_pass_typed<float>(n, b, Rinv, static_cast<float*>(W), want_gram, partials, &nparts, st));
+        if (!want_gram) return BBL_OK;
+        if (nparts == 0) {
+            BBL_TRY(gram(n, b, 1, dtype, W, W, G, partials, st));
+            nparts = 1;
+            gsum = G;
+        } else if (nparts > kCholParts) {
+            launch_reduce((int64_t)b * b, nparts, partials.as<double>(), G, st);
+            BBL_LAUNCH_CHECK();
+            nparts = 1;
+            gsum = G;
+        } else {
+            gsum = partials.as<double>();
+        }
+        return BBL_OK;
+    };
+    BBL_TRY(pass(nullptr, true));
+    chol_kernel<<<1, kCholThreads, 0, st>>>(b, nparts, gsum, t1, relative, R1, R1i, d_ndefl, d_mask, status, nullptr,
+                                            nullptr);
     BBL_LAUNCH_CHECK();
-    if (dtype == BBL_FP64)
-        BBL_TRY((apply_typed<double, false, double, double>(n, b, b, b, static_cast<double*>(W), R1i,
-                                                             static_cast<double*>(W), st)));
-    else if (dtype == kDF32)
-        BBL_TRY((apply_typed<df32, false, df32, df32>(n, b, b, b, static_cast<df32*>(W), R1i, static_cast<df32*>(W),
-                                                       st)));
-    else
-        BBL_TRY((apply_typed<float, false, float, float>(n, b, b, b, static_cast<float*>(W), R1i,
-                                                          static_cast<float*>(W), st)));
-    BBL_TRY(self_gram(n, b, dtype, W, G, partials, st));
+    BBL_TRY(pass(R1i, true));
     // second pass: columns of Q1 have norm ~1; a pivot below 1e-6 means the
     // first pass produced no usable direction (it was deflated or lost).
-    chol_warp_kernel<<<1, 32, 0, st>>>(b, G, 1e-6, 0, R2, R2i, nullptr, nullptr, status);
+    chol_kernel<<<1, kCholThreads, 0, st>>>(b, nparts, gsum, 1e-6, 0, R2, R2i, nullptr, nullptr, status, R1, B);
     BBL_LAUNCH_CHECK();
-    if (dtype == BBL_FP64)
-        BBL_TRY((apply_typed<double, false, double, double>(n, b, b, b, static_cast<double*>(W), R2i,
-                                                             static_cast<double*>(W), st)));
-    else if (dtype == kDF32)
-        BBL_TRY((apply_typed<df32, false, df32, df32>(n, b, b, b, static_cast<df32*>(W), R2i, static_cast<df32*>(W),
-                                                       st)));
-    else
-        BBL_TRY((apply_typed<float, false, float, float>(n, b, b, b, static_cast<float*>(W), R2i,
-                                                          static_cast<float*>(W), st)));
-    if (B) {
-        trmul_kernel<<<1, 256, 0, st>>>(b, R2, R1, B);
-        BBL_LAUNCH_CHECK();
-    }
-    return BBL_OK;
+    return pass(R2i, false);
 }
 
 // -------------------------------------------------------------------- segmented (batched) forms
