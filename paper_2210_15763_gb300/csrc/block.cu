@@ -1479,20 +1479,6 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
 
 // -------------------------------------------------------------------- Cholesky of the b x b Gram
 // status bits: 1 = non-finite Gram.  mask[i] = 1 for deflated columns.
-__device__ void chol_body(int b, const double* __restrict__ G, double thresh2, int relative, double* __restrict__ R,
-                          double* __restrict__ Rinv, int* __restrict__ ndefl, int* __restrict__ mask,
-                          int* __restrict__ status);
-
-// One thread per segment: Cholesky of G + s*b*b with threshold thresh2[s].
-__global__ void chol_seg_kernel(int b, int nseg, const double* __restrict__ G, const double* __restrict__ thresh2,
-                                int relative, double* __restrict__ R, double* __restrict__ Rinv, int* __restrict__ ndefl,
-                                int* __restrict__ mask, int* __restrict__ status, const int* __restrict__ active) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg || (active && !active[s])) return;
-    const int64_t o = (int64_t)s * b * b;
-    chol_body(b, G + o, thresh2 ? thresh2[s] : 0.0, relative, R + o, Rinv + o, ndefl ? ndefl + s : nullptr,
-              mask ? mask + (int64_t)s * b : nullptr, status ? status + s : nullptr);
-}
 
 __global__ void trmul_seg_kernel(int b, int nseg, const double* __restrict__ R2, const double* __restrict__ R1,
                                  double* __restrict__ B, const int* __restrict__ active) {
@@ -1504,57 +1490,6 @@ __global__ void trmul_seg_kernel(int b, int nseg, const double* __restrict__ R2,
     double acc = 0.0;
     for (int l = 0; l < b; ++l) acc += R2[o + i * b + l] * R1[o + l * b + k];
     B[o + e] = acc;
-}
-
-__device__ void chol_body(int b, const double* __restrict__ G, double thresh2, int relative, double* __restrict__ R,
-                          double* __restrict__ Rinv, int* __restrict__ ndefl, int* __restrict__ mask,
-                          int* __restrict__ status) {
-    double Rl[kMaxB * kMaxB];
-    int dm[kMaxB];
-    bool bad = false;
-    double gmax = 0.0;
-    for (int i = 0; i < b * b; ++i) {
-        Rl[i] = 0.0;
-        if (!isfinite(G[i])) bad = true;
-    }
-    for (int i = 0; i < b; ++i) gmax = fmax(gmax, G[i * b + i]);
-    if (relative) thresh2 *= gmax;
-    int cnt = 0;
-    for (int i = 0; i < b; ++i) {
-        double d = G[i * b + i];
-        for (int l = 0; l < i; ++l) d -= Rl[l * b + i] * Rl[l * b + i];
-        dm[i] = !(d > thresh2) || bad;
-        if (dm[i]) {
-            ++cnt;
-            continue;
-        }
-        const double rii = sqrt(d);
-        Rl[i * b + i] = rii;
-        for (int k = i + 1; k < b; ++k) {
-            double s = G[i * b + k];
-            for (int l = 0; l < i; ++l) s -= Rl[l * b + i] * Rl[l * b + k];
-            Rl[i * b + k] = s / rii;
-        }
-    }
-    for (int i = 0; i < b * b; ++i) {
-        R[i] = Rl[i];
-        Rinv[i] = 0.0;
-    }
-    for (int c = 0; c < b; ++c) {
-        if (dm[c]) continue;
-        Rinv[c * b + c] = 1.0 / Rl[c * b + c];
-        for (int i = c - 1; i >= 0; --i) {
-            if (dm[i]) continue;
-            double s = 0.0;
-            for (int k = i + 1; k <= c; ++k)
-                if (!dm[k]) s += Rl[i * b + k] * Rinv[k * b + c];
-            Rinv[i * b + c] = -s / Rl[i * b + i];
-        }
-    }
-    if (mask)
-        for (int i = 0; i < b; ++i) mask[i] = dm[i];
-    if (ndefl) *ndefl += cnt;
-    if (bad && status) atomicOr(status, 1);
 }
 
 // 1 / d of a normal finite d, to about one unit in the last place: an FP32
@@ -1574,24 +1509,98 @@ __device__ __forceinline__ double recip(double d) {
 constexpr int kCholThreads = 256;
 constexpr int kCholParts = 128;  // most partial Grams one CTA adds itself (two FP64 additions per cycle)
 
+// G = L D L^T with deflation, right-looking by one warp, whose lanes keep the
+// entries of G's Schur complement and of L^{-1} in registers: a step is one
+// reciprocal, one product and one update deep.  (The left-looking form with a
+// square root and divisions in the chain took 15 us at b = 8 by a warp and 14 us
+// by one thread per segment, this one about 8.)
+struct CholShared {
+    double G[kMaxB * kMaxB];
+    double L[kMaxB * kMaxB];      // row k: L[.][k]
+    double Z[kMaxB * kMaxB];      // row k of L^{-1}
+    double row[2][2][kMaxB];      // row k of the Schur complement and of L^{-1}
+    double d[kMaxB], root[kMaxB]; // D (0 for deflated columns) and its square roots
+    int deflated[kMaxB];
+};
+
+__device__ __forceinline__ void chol_core(int b, double thresh2, int relative, CholShared& sh, int& cnt, int& bad) {
+    const int lane = threadIdx.x & 31, bb = b * b;
+    constexpr int E = kMaxB * kMaxB / 32;
+    double a[E], z[E];
+    int ei[E], ec[E];
+    bad = 0;
+#pragma unroll
+    for (int x = 0; x < E; ++x) {
+        const int q = lane + 32 * x;
+        ei[x] = q < bb ? q / b : -1;
+        ec[x] = q < bb ? q - ei[x] * b : 0;
+        a[x] = q < bb ? sh.G[q] : 0.0;
+        z[x] = ei[x] == ec[x] ? 1.0 : 0.0;
+        if (!isfinite(a[x])) bad = 1;
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (relative) {
+        double gmax = 0.0;
+        for (int q = 0; q < b; ++q) gmax = fmax(gmax, sh.G[q * b + q]);
+        thresh2 *= gmax;
+    }
+    cnt = 0;
+#pragma unroll
+    for (int x = 0; x < E; ++x)
+        if (ei[x] == 0) {
+            sh.row[0][0][ec[x]] = a[x];
+            sh.row[0][1][ec[x]] = z[x];
+        }
+    __syncwarp();
+    for (int k = 0; k < b; ++k) {
+        const double* ra = sh.row[k & 1][0];
+        const double* rz = sh.row[k & 1][1];
+        const double d = ra[k];
+        const int defl = !(d > thresh2) || bad;
+        cnt += defl;
+        const double y = defl ? 0.0 : recip(d);
+        if (lane == 0) {
+            sh.deflated[k] = defl;
+            sh.d[k] = defl ? 0.0 : d;
+        }
+        if (lane < b) {
+            sh.L[k * b + lane] = lane < k || defl ? 0.0 : ra[lane] * y;
+            sh.Z[k * b + lane] = lane > k || defl ? 0.0 : rz[lane];
+        }
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            if (32 * x < bb && ei[x] > k) {
+                const double l = ra[ei[x]] * y;
+                if (!defl && ec[x] >= ei[x]) a[x] = fma(-l, ra[ec[x]], a[x]);
+                if (!defl && ec[x] <= k) z[x] = fma(-l, rz[ec[x]], z[x]);
+                if (ei[x] == k + 1) {
+                    sh.row[(k + 1) & 1][0][ec[x]] = a[x];
+                    sh.row[(k + 1) & 1][1][ec[x]] = z[x];
+                }
+            }
+        }
+        __syncwarp();
+    }
+    if (lane < b) sh.root[lane] = sqrt(sh.d[lane]);
+    __syncwarp();
+}
+
+// entry e of R = D^{1/2} L^T and of R^{-1}: zero rows (columns) for deflated columns
+__device__ __forceinline__ double chol_R(const CholShared& sh, int b, int e) { return sh.L[e] * sh.root[e / b]; }
+__device__ __forceinline__ double chol_Rinv(const CholShared& sh, int b, int e) {
+    const int i = e / b, c = e % b;
+    return c >= i && !sh.deflated[c] ? sh.Z[c * b + i] / sh.root[c] : 0.0;
+}
+
 // The Cholesky step of CholQR2 by one CTA: G = the sum of nparts partial b x b
 // Grams, R = chol(G) with deflation and R^{-1}, and, with Bout, B = R R1.
-// G = L D L^T right-looking by one warp, whose lanes keep the entries of G and of
-// L^{-1} in registers: a step is one reciprocal, one product and one update deep;
-// the square roots (R = D^{1/2} L^T) follow together.  Deflated columns get zero
-// rows in R and zero columns in R^{-1}.
 __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, const double* __restrict__ partial,
                                                             double thresh2, int relative, double* __restrict__ R,
                                                             double* __restrict__ Rinv, int* __restrict__ ndefl,
                                                             int* __restrict__ mask, int* __restrict__ status,
                                                             const double* __restrict__ R1, double* __restrict__ Bout) {
-    __shared__ double Gs[kMaxB * kMaxB];
-    __shared__ double Ls[kMaxB * kMaxB];  // row k: L[.][k] = R[k][.] / sqrt(d_k)
-    __shared__ double Zs[kMaxB * kMaxB];  // row k of L^{-1}
-    __shared__ double row[2][2][kMaxB];   // row k of the Schur complement and of L^{-1}
-    __shared__ double dk[kMaxB], root[kMaxB];
+    __shared__ CholShared sh;
     __shared__ double red[kCholThreads];
-    __shared__ int dm[kMaxB];
     const int tid = threadIdx.x, bb = b * b;
     {  // groups of bb threads add the parts
         const int groups = kCholThreads / bb, e = tid % bb, g = tid / bb;
@@ -1600,68 +1609,14 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, c
         if (tid < bb) {
             double s = red[tid];
             for (int q = 1; q < groups; ++q) s += red[tid + q * bb];
-            Gs[tid] = s;
+            sh.G[tid] = s;
         }
         __syncthreads();
     }
     if (tid < 32) {
-        const int lane = tid;
-        constexpr int E = kMaxB * kMaxB / 32;
-        double a[E], z[E];
-        int ei[E], ec[E];
-        int bad = 0;
-#pragma unroll
-        for (int x = 0; x < E; ++x) {
-            const int q = lane + 32 * x;
-            ei[x] = q < bb ? q / b : -1;
-            ec[x] = q < bb ? q - ei[x] * b : 0;
-            a[x] = q < bb ? Gs[q] : 0.0;
-            z[x] = ei[x] == ec[x] ? 1.0 : 0.0;
-            if (!isfinite(a[x])) bad = 1;
-        }
-        bad = __any_sync(0xffffffffu, bad);
-        double gmax = 0.0;
-        for (int q = 0; q < b; ++q) gmax = fmax(gmax, Gs[q * b + q]);
-        if (relative) thresh2 *= gmax;
-        int cnt = 0;
-#pragma unroll
-        for (int x = 0; x < E; ++x)
-            if (ei[x] == 0) {
-                row[0][0][ec[x]] = a[x];
-                row[0][1][ec[x]] = z[x];
-            }
-        __syncwarp();
-        for (int k = 0; k < b; ++k) {
-            const double* ra = row[k & 1][0];
-            const double* rz = row[k & 1][1];
-            const double d = ra[k];
-            const int defl = !(d > thresh2) || bad;
-            cnt += defl;
-            const double y = defl ? 0.0 : recip(d);
-            if (lane == 0) {
-                dm[k] = defl;
-                dk[k] = defl ? 0.0 : d;
-            }
-            if (lane < b) {
-                Ls[k * b + lane] = lane < k || defl ? 0.0 : ra[lane] * y;
-                Zs[k * b + lane] = lane > k || defl ? 0.0 : rz[lane];
-            }
-#pragma unroll
-            for (int x = 0; x < E; ++x) {
-                if (32 * x < bb && ei[x] > k) {
-                    const double l = ra[ei[x]] * y;
-                    if (ec[x] >= ei[x]) a[x] = fma(-l, ra[ec[x]], a[x]);
-                    if (ec[x] <= k && !defl) z[x] = fma(-l, rz[ec[x]], z[x]);
-                    if (ei[x] == k + 1) {
-                        row[(k + 1) & 1][0][ec[x]] = a[x];
-                        row[(k + 1) & 1][1][ec[x]] = z[x];
-                    }
-                }
-            }
-            __syncwarp();
-        }
-        if (lane < b) root[lane] = sqrt(dk[lane]);
-        if (lane == 0) {
+        int cnt, bad;
+        chol_core(b, thresh2, relative, sh, cnt, bad);
+        if (tid == 0) {
             if (ndefl) *ndefl += cnt;
             if (bad && status) atomicOr(status, 1);
         }
@@ -1669,15 +1624,40 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, c
     __syncthreads();
     if (tid < bb) {
         const int i = tid / b, c = tid % b;
-        R[tid] = Ls[tid] * root[i];
-        Rinv[tid] = c >= i && !dm[c] ? Zs[c * b + i] / root[c] : 0.0;
+        R[tid] = chol_R(sh, b, tid);
+        Rinv[tid] = chol_Rinv(sh, b, tid);
         if (Bout) {
             double s = 0.0;
-            for (int l = i; l <= c; ++l) s += Ls[i * b + l] * root[i] * R1[l * b + c];
+            for (int l = i; l <= c; ++l) s += sh.L[i * b + l] * sh.root[i] * R1[l * b + c];
             Bout[tid] = s;
         }
     }
-    if (mask && tid < b) mask[tid] = dm[tid];
+    if (mask && tid < b) mask[tid] = sh.deflated[tid];
+}
+
+// A warp per segment: Cholesky of G + s*b*b with threshold thresh2[s].
+__global__ void __launch_bounds__(32) chol_seg_kernel(int b, const double* __restrict__ G,
+                                                      const double* __restrict__ thresh2, int relative,
+                                                      double* __restrict__ R, double* __restrict__ Rinv,
+                                                      int* __restrict__ ndefl, int* __restrict__ mask,
+                                                      int* __restrict__ status, const int* __restrict__ active) {
+    __shared__ CholShared sh;
+    const int s = blockIdx.x, lane = threadIdx.x, bb = b * b;
+    if (active && !active[s]) return;
+    const int64_t o = (int64_t)s * bb;
+    for (int e = lane; e < bb; e += 32) sh.G[e] = G[o + e];
+    __syncwarp();
+    int cnt, bad;
+    chol_core(b, thresh2 ? thresh2[s] : 0.0, relative, sh, cnt, bad);
+    for (int e = lane; e < bb; e += 32) {
+        R[o + e] = chol_R(sh, b, e);
+        Rinv[o + e] = chol_Rinv(sh, b, e);
+    }
+    if (mask && lane < b) mask[(int64_t)s * b + lane] = sh.deflated[lane];
+    if (lane == 0) {
+        if (ndefl) ndefl[s] += cnt;
+        if (bad && status) atomicOr(status + s, 1);
+    }
 }
 
 }  // namespace
@@ -1966,8 +1946,7 @@ bbl_status apply_seg_typed(int64_t n, int b, int kc, const int* ms, int mss, con
 
 int gram_seg_chunk_rows(int b, int dtype) {
     if (dtype == BBL_FP64) {
-        if (b == 4) return GramRowsShape<double, 4>::R;
-        if (b == 8) return GramRowsShape<double, 8>::R;
+        if (b == 4 || b == 8) return 512;  // the tensor-core form's chunk; within the row kernel's tile
     } else if (dtype == BBL_FP32) {
         if (b == 4) return GramRowsShape<float, 4>::R;
         if (b == 8) return GramRowsShape<float, 8>::R;
@@ -1980,8 +1959,14 @@ bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, cons
                     const int64_t* chunks, int nchunks, const int* seg_chunk_ptr, int nseg, const int* active,
                     double* partial, double* C, cudaStream_t st) {
     constexpr int kC = 4;
-    const int rows_slots = gram_seg_chunk_rows(b, dtype) > 0 ? 1 : 0;
-    if (rows_slots) {
+    // against a whole basis the FP64 products run on the tensor cores; the self
+    // Gram of one block (m_max = b) fills too little of a tile of 16 columns
+    const bool tc = dtype == BBL_FP64 && tc64_seg_supports(b) && m_max >= 32;
+    const int rows_slots = !tc && gram_seg_chunk_rows(b, dtype) > 0 ? 1 : 0;
+    if (tc) {
+        BBL_TRY(gram_tc64_seg(n, b, d_m, static_cast<const double*>(Q), static_cast<const double*>(W), chunks, nchunks,
+                              active, partial, st));
+    } else if (rows_slots) {
         if (dtype == BBL_FP64) {
             auto q = static_cast<const double*>(Q);
             auto w = static_cast<const double*>(W);
@@ -2028,6 +2013,8 @@ bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int
                      cudaStream_t st) {
     if (dtype == BBL_FP64) {
         auto q = static_cast<const double*>(Q);
+        if (sub && kc == b && tc64_seg_supports(b))
+            return update_tc64_seg(n, b, ms, ms_stride, ctas, nctas, active, q, C, cstride, static_cast<double*>(W), st);
         if (sub) return apply_seg_typed<double, true, double, double>(n, b, kc, ms, ms_stride, ctas, nctas, active, q, C, cstride,
                                                                       static_cast<double*>(W), st);
         return apply_seg_typed<double, false, double, double>(n, b, kc, ms, ms_stride, ctas, nctas, active, q, C, cstride,
@@ -2045,8 +2032,7 @@ bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int
 
 bbl_status chol_seg(int b, int nseg, const double* G, const double* thresh2, int relative, double* R, double* Rinv,
                     int* ndefl, int* mask, int* status, const int* active, cudaStream_t st) {
-    chol_seg_kernel<<<(unsigned)ceil_div(nseg, 32), 32, 0, st>>>(b, nseg, G, thresh2, relative, R, Rinv, ndefl, mask,
-                                                                 status, active);
+    chol_seg_kernel<<<(unsigned)nseg, 32, 0, st>>>(b, G, thresh2, relative, R, Rinv, ndefl, mask, status, active);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }

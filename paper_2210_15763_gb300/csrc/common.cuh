@@ -294,6 +294,13 @@ bbl_status gram_tc64(int64_t n, int b, int m, const double* Q, const double* W, 
                      cudaStream_t st);
 bbl_status update_tc64(int64_t n, int b, int m, int kc, const double* Q, const double* C, double* W, bool sub,
                        cudaStream_t st);
+// segmented forms (b that tc64_seg_supports names; block.cu explains the tables)
+bool tc64_seg_supports(int b);
+bbl_status gram_tc64_seg(int64_t n, int b, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
+                         int nchunks, const int* active, double* partial, cudaStream_t st);
+bbl_status update_tc64_seg(int64_t n, int b, const int* ms, int ms_stride, const int64_t* ctas, int nctas,
+                           const int* active, const double* Q, const double* C, int64_t cstride, double* W,
+                           cudaStream_t st);
 // ritz.cu
 bbl_status ritz_dev(int m, int p, int nev, const double* Tband, double* theta, double* S, DevBuf& work,
                     cudaStream_t st, const double* warm = nullptr, int warm_count = 0);

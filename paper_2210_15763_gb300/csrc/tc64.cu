@@ -325,29 +325,149 @@ __device__ __forceinline__ int swizzle(int row, int q) {  // 16-byte chunk q of 
     return B == 16 ? q ^ (2 * (row & 3)) : B == 8 ? q ^ (row & 2) : q;
 }
 
+// Shares of a chunk's steps per tile: with fewer tiles than warps the idle
+// warps take shares (a warp then has one item at most).
+__host__ __device__ inline int gram_parts(int ntiles) {
+    int p = 1;
+    while (ntiles * p * 2 <= kWarps) p *= 2;
+    return p;
+}
+
+// rows [r0, r0 + rows) (at most 512), columns c0 .. c0 + 7 of W: added to slot (m x B).
+// All threads, after a barrier that follows the last use of smem and the zeroing
+// of slot and ew.
 template <int B>
-__global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int rc, int nchunks, int parts,
-                                                          const double* __restrict__ Q, const double* __restrict__ W,
-                                                          double* __restrict__ partial, int* __restrict__ tickets) {
-    extern __shared__ __align__(16) unsigned char tc_smem[];
+__device__ __forceinline__ void gram_chunk(int64_t n, int m, int parts, int64_t r0, int rows, int c0,
+                                           const double* __restrict__ Q, const double* __restrict__ W,
+                                           double* __restrict__ slot, unsigned char* smem, int* ew,
+                                           double (*sums)[128]) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned char* ring = tc_smem + warp * kRing * kStepBytes;
-    uint2* frag = reinterpret_cast<uint2*>(tc_smem + kWarps * kRing * kStepBytes);
-    __shared__ int ew[8];
-    __shared__ int s_chunk;
+    unsigned char* ring = smem + warp * kRing * kStepBytes;
+    uint2* frag = reinterpret_cast<uint2*>(smem + kWarps * kRing * kStepBytes);
     const int g = lane >> 2, t = lane & 3;
-    const int c0 = blockIdx.y * 8;
     const bool col = c0 + g < B;
-    const int ntiles = (m + 15) / 16, items = ntiles * parts;
-    double* slot = partial + (int64_t)blockIdx.x * m * B;
-    for (int e = tid; e < m * B; e += kT)
-        if (e % B >= c0 && e % B < c0 + 8) slot[e] = 0.0;
+    const int items = (m + 15) / 16 * parts;
     // a step of a tile in the ring: block-major, then rows of B entries
     constexpr int CPR = B / 2;                       // 16-byte chunks per row
     constexpr int CPB = 16 * CPR;                    // chunks per block (B = 2, 4, 8, 16: 16 .. 128)
     const int ob = (g / B) * 16 * B * 8;             // line g's block, and line g + 8's
     const int ob8 = ((g + 8) / B) * 16 * B * 8;
     const int og = g % B, og8 = (g + 8) % B;
+    const int steps = (rows + 15) / 16;
+    // the columns' scales, then the digits: a warp per step, a lane's four rows of column c0 + g
+    constexpr int SW = kMaxRows / 16 / kWarps;
+    {
+        double xw[SW][4];
+        int mx = 0;
+#pragma unroll
+        for (int k = 0; k < SW; ++k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = 16 * (warp + k * kWarps) + t + 4 * i;
+                xw[k][i] = (col && r < rows) ? __ldg(W + (r0 + r) * B + c0 + g) : 0.0;
+                mx = max(mx, exp_bits(xw[k][i]));
+            }
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
+        __syncthreads();
+        const int eg = max(ew[g], kEmin);
+#pragma unroll
+        for (int k = 0; k < SW; ++k)
+            if (warp + k * kWarps < steps) store_frag(frag + (warp + k * kWarps) * kDig * 32, lane, xw[k], eg);
+    }
+    __syncthreads();
+    const int per = (steps + parts - 1) / parts;
+    for (int w = warp; w < items; w += kWarps) {
+        const int tile = w / parts, part = w % parts;
+        const int s0 = part * per, s1 = min(steps, s0 + per);
+        if (s0 >= s1) continue;
+        const int j0 = 16 * tile / B, nblk = (m - 16 * tile) / B;  // first block and blocks left
+        const bool whole = nblk * B >= 16;
+        const double* p = Q + ((int64_t)j0 * n + r0) * B;
+        auto issue = [&](int s) {
+            if (s < s1) {
+                unsigned char* buf = ring + (s % kRing) * kStepBytes;
+                const bool full = whole && 16 * s + 16 <= rows;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int e = lane + 32 * i;
+                    const int j = e / CPB, r = (e % CPB) / CPR, q = e % CPR;
+                    void* dst = buf + (j * CPB + r * CPR + swizzle<B>(r, q)) * 16;
+                    const double* src = p + (int64_t)j * n * B + (16 * s + r) * B + 2 * q;
+                    if (full) cp_async16(dst, src);
+                    else cp_async16(dst, (j < nblk && 16 * s + r < rows) ? src : Q, j < nblk && 16 * s + r < rows);
+                }
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
+        Acc acc;
+        acc.clear();
+        LineScale sc;
+        double* mine = sums[warp] + lane;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mine[32 * e] = 0.0;
+        auto flush = [&]() {
+            acc.to_int();
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                mine[32 * e] += unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin));
+            acc.clear();
+        };
+        for (int s = s0; s < s1; ++s) {
+            cp_async_wait<kRing - 2>();
+            __syncwarp();
+            issue(s + kRing - 1);  // into the buffer of step s - 1
+            const unsigned char* buf = ring + (s % kRing) * kStepBytes;
+            double x[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = t + 4 * i;
+                const int k = (i >> 1) * 4 + (i & 1);  // register 0 / 2 of line g, 1 / 3 of line g + 8
+                x[k] = *reinterpret_cast<const double*>(buf + ob + r * B * 8 + swizzle<B>(r, og >> 1) * 16 + (og & 1) * 8);
+                x[k + 2] = *reinterpret_cast<const double*>(buf + ob8 + r * B * 8 + swizzle<B>(r, og8 >> 1) * 16 + (og8 & 1) * 8);
+            }
+            step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
+            if (((s - s0) & 3) == 3) acc.to_int();
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+        flush();
+        if (parts == 1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int a = 16 * tile + g + ((e & 2) ? 8 : 0), c = c0 + 2 * t + (e & 1);
+                // this tile's only writer; an add that returns nothing is not waited for
+                if (a < m && c < B) atomicAdd(slot + (int64_t)a * B + c, mine[32 * e]);
+            }
+        }
+    }
+    if (parts > 1) {  // the shares in order
+        __syncthreads();
+        for (int e = tid; e < items / parts * 128; e += kT) {
+            const int tile = e / 128, q = e % 128, l = q & 31;
+            double v = 0.0;
+            for (int p = 0; p < parts && p * ((steps + parts - 1) / parts) < steps; ++p) v += sums[tile * parts + p][q];
+            const int a = 16 * tile + (l >> 2) + ((q & 64) ? 8 : 0), c = c0 + 2 * (l & 3) + ((q & 32) ? 1 : 0);
+            if (a < m && c < B) slot[(int64_t)a * B + c] += v;
+        }
+    }
+}
+
+template <int B>
+__global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int rc, int nchunks, int parts,
+                                                          const double* __restrict__ Q, const double* __restrict__ W,
+                                                          double* __restrict__ partial, int* __restrict__ tickets) {
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    __shared__ int ew[8];
+    __shared__ double sums[kWarps][128];  // an item's sums
+    __shared__ int s_chunk;
+    const int tid = threadIdx.x, c0 = blockIdx.y * 8;
+    double* slot = partial + (int64_t)blockIdx.x * m * B;
+    for (int e = tid; e < m * B; e += kT)
+        if (e % B >= c0 && e % B < c0 + 8) slot[e] = 0.0;
     for (;;) {
         __syncthreads();
         if (tid == 0) s_chunk = atomicAdd(tickets + blockIdx.y, 1);
@@ -356,92 +476,34 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
         const int chunk = s_chunk;
         if (chunk >= nchunks) break;
         const int64_t r0 = (int64_t)chunk * rc;
-        const int rows = (int)min((int64_t)rc, n - r0);
-        const int steps = (rows + 15) / 16;
-        // the columns' scales, then the digits: a warp per step, a lane's four rows of column c0 + g
-        constexpr int SW = kMaxRows / 16 / kWarps;
-        {
-            double xw[SW][4];
-            int mx = 0;
-#pragma unroll
-            for (int k = 0; k < SW; ++k)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = 16 * (warp + k * kWarps) + t + 4 * i;
-                    xw[k][i] = (col && r < rows) ? __ldg(W + (r0 + r) * B + c0 + g) : 0.0;
-                    mx = max(mx, exp_bits(xw[k][i]));
-                }
-#pragma unroll
-            for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
-            __syncthreads();
-            const int eg = max(ew[g], kEmin);
-#pragma unroll
-            for (int k = 0; k < SW; ++k)
-                if (warp + k * kWarps < steps) store_frag(frag + (warp + k * kWarps) * kDig * 32, lane, xw[k], eg);
-        }
-        __syncthreads();
-        const int per = (steps + parts - 1) / parts;
-        for (int w = warp; w < items; w += kWarps) {
-            const int tile = w / parts, part = w % parts;
-            const int s0 = part * per, s1 = min(steps, s0 + per);
-            if (s0 >= s1) continue;
-            const int j0 = 16 * tile / B, nblk = (m - 16 * tile) / B;  // first block and blocks left
-            const bool whole = nblk * B >= 16;
-            const double* p = Q + ((int64_t)j0 * n + r0) * B;
-            auto issue = [&](int s) {
-                if (s < s1) {
-                    unsigned char* buf = ring + (s % kRing) * kStepBytes;
-                    const bool full = whole && 16 * s + 16 <= rows;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int e = lane + 32 * i;
-                        const int j = e / CPB, r = (e % CPB) / CPR, q = e % CPR;
-                        void* dst = buf + (j * CPB + r * CPR + swizzle<B>(r, q)) * 16;
-                        const double* src = p + (int64_t)j * n * B + (16 * s + r) * B + 2 * q;
-                        if (full) cp_async16(dst, src);
-                        else cp_async16(dst, (j < nblk && 16 * s + r < rows) ? src : Q, j < nblk && 16 * s + r < rows);
-                    }
-                }
-                cp_async_commit();
-            };
-#pragma unroll
-            for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
-            Acc acc;
-            acc.clear();
-            LineScale sc;
-            auto flush = [&]() {
-                acc.to_int();
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int a = 16 * tile + g + ((e & 2) ? 8 : 0), c = c0 + 2 * t + (e & 1);
-                    if (a < m && c < B)
-                        atomicAdd(slot + (int64_t)a * B + c,
-                                  unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin)));
-                }
-                acc.clear();
-            };
-            for (int s = s0; s < s1; ++s) {
-                cp_async_wait<kRing - 2>();
-                __syncwarp();
-                issue(s + kRing - 1);  // into the buffer of step s - 1
-                const unsigned char* buf = ring + (s % kRing) * kStepBytes;
-                double x[8];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = t + 4 * i;
-                    const int k = (i >> 1) * 4 + (i & 1);  // register 0 / 2 of line g, 1 / 3 of line g + 8
-                    x[k] = *reinterpret_cast<const double*>(buf + ob + r * B * 8 + swizzle<B>(r, og >> 1) * 16 + (og & 1) * 8);
-                    x[k + 2] = *reinterpret_cast<const double*>(buf + ob8 + r * B * 8 + swizzle<B>(r, og8 >> 1) * 16 + (og8 & 1) * 8);
-                }
-                step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
-                if (((s - s0) & 3) == 3) acc.to_int();
-            }
-            cp_async_wait<0>();
-            __syncwarp();
-            flush();
-        }
+        gram_chunk<B>(n, m, parts, r0, (int)min((int64_t)rc, n - r0), c0, Q, W, slot, tc_smem, ew, sums);
     }
+}
+
+// Batch of problems stacked row-wise: CTA x takes chunk x, rows [chunks[3x+1],
+// chunks[3x+2]) of segment chunks[3x] (at most 512, never crossing a segment),
+// into its own slot at partial[x * m * B]; m is read from device memory, chunks
+// of inactive segments do nothing.
+template <int B>
+__global__ void __launch_bounds__(kT, 2) gram_tc64_seg_kernel(int64_t n, const int* __restrict__ d_m,
+                                                              const int64_t* __restrict__ chunks,
+                                                              const int* __restrict__ seg_active,
+                                                              const double* __restrict__ Q,
+                                                              const double* __restrict__ W,
+                                                              double* __restrict__ partial) {
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    __shared__ int ew[8];
+    __shared__ double sums[kWarps][128];
+    const int64_t seg = chunks[3 * blockIdx.x];
+    if (seg_active && !seg_active[seg]) return;
+    const int m = *d_m;
+    const int64_t r0 = chunks[3 * blockIdx.x + 1];
+    const int rows = (int)(chunks[3 * blockIdx.x + 2] - r0);
+    double* slot = partial + (int64_t)blockIdx.x * m * B;
+    for (int e = threadIdx.x; e < m * B; e += kT) slot[e] = 0.0;
+    if (threadIdx.x < 8) ew[threadIdx.x] = 0;
+    __syncthreads();
+    gram_chunk<B>(n, m, gram_parts((m + 15) / 16), r0, rows, 0, Q, W, slot, tc_smem, ew, sums);
 }
 
 // -------------------------------------------------------------------- W (-)= Q C
@@ -449,122 +511,149 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
 // and W.  A warp takes 16 rows; the digits of up to kMaxCols rows of C are
 // staged as B fragments (in one go, kept over the CTA's row groups, when they
 // are all of C).
+// One group of rows from row0 on (16 per row tile, kWarps / ks tiles, below
+// row_end); staged: C's digits are in smem from an earlier group.  All threads.
+template <int B, bool SUB>
+__device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, int c0, int64_t row0, int64_t row_end,
+                                             bool& staged, const double* Q, const double* __restrict__ C, double* W,
+                                             unsigned char* smem, int* ew, double (*part)[4][32]) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double2* ring = reinterpret_cast<double2*>(smem + warp * kRing * kStepBytes) + lane;
+    uint2* frag = reinterpret_cast<uint2*>(smem + kWarps * kRing * kStepBytes);
+    const int g = lane >> 2, t = lane & 3;
+    const bool col = c0 + g < kc;
+    const int sub = warp % ks;  // ks warps share a tile of 16 rows, each a share of the steps
+    const int64_t ra = row0 + (warp / ks) * 16 + g, rb = ra + 8;
+    double out[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k0 = 0; k0 < m; k0 += kMaxCols) {
+        const int cols = min(kMaxCols, m - k0), steps = (cols + 15) / 16;
+        if (!staged) {
+            __syncthreads();
+            if (tid < 8) ew[tid] = 0;
+            __syncthreads();
+            int mx = 0;
+            for (int s = warp; s < steps; s += kWarps)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
+                    if (col && a < cols) mx = max(mx, exp_bits(C[(int64_t)(k0 + a) * kc + c0 + g]));
+                }
+#pragma unroll
+            for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
+            __syncthreads();
+            const int eg = max(ew[g], kEmin);
+            for (int s = warp; s < steps; s += kWarps) {
+                double x[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
+                    x[i] = (col && a < cols) ? C[(int64_t)(k0 + a) * kc + c0 + g] : 0.0;
+                }
+                store_frag(frag + s * kDig * 32, lane, x, eg);
+            }
+            __syncthreads();
+            staged = m <= kMaxCols;
+        }
+        // registers 0, 1: columns 2t, 2t+1 of rows g, g+8; 2, 3: columns 2t+8,
+        // 2t+9.  A lane copies its own 16-byte pairs into its ring and reads them back.
+        const int per = (steps + ks - 1) / ks, s0 = sub * per, s1 = min(steps, s0 + per);
+        const bool rows_in = row0 + (warp / ks) * 16 + 16 <= row_end;
+        auto issue = [&](int s) {
+            if (s < s1) {
+                const bool full = rows_in && k0 + 16 * s + 16 <= m;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int a = k0 + 16 * s + 8 * (i >> 1) + 2 * t;
+                    const int64_t r = (i & 1) ? rb : ra;
+                    const double* src = Q + ((int64_t)(a / B) * n + r) * B + a % B;
+                    double2* dst = ring + (s % kRing) * 128 + i * 32;
+                    if (full) cp_async16(dst, src);
+                    else cp_async16(dst, (a < m && r < row_end) ? src : Q, a < m && r < row_end);
+                }
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
+        Acc acc;
+        acc.clear();
+        LineScale sc;
+        auto flush = [&]() {
+            acc.to_int();
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                out[e] += unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin));
+            acc.clear();
+        };
+        for (int s = s0; s < s1; ++s) {
+            cp_async_wait<kRing - 2>();
+            double x[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double2 v = ring[(s % kRing) * 128 + i * 32];
+                x[2 * i] = v.x;
+                x[2 * i + 1] = v.y;
+            }
+            issue(s + kRing - 1);  // into the buffer of step s - 1
+            step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
+            if (((s - s0) & 3) == 3) acc.to_int();
+        }
+        cp_async_wait<0>();
+        if (s0 < s1) flush();
+    }
+    if (ks > 1) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[warp][e][lane] = out[e];
+        __syncthreads();
+        if (sub != 0) return;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            for (int q = 1; q < ks; ++q) out[e] += part[warp + q][e][lane];
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int64_t r = (e & 2) ? rb : ra;
+        const int c = c0 + 2 * t + (e & 1);
+        if (r < row_end && c < kc) {
+            double* w = W + r * kc + c;
+            *w = SUB ? *w - out[e] : out[e];
+        }
+    }
+}
+
 template <int B, bool SUB>
 __global__ void __launch_bounds__(kT, 2) update_tc64_kernel(int64_t n, int m, int kc, int ks, const double* Q,
                                                             const double* __restrict__ C, double* W) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    double2* ring = reinterpret_cast<double2*>(tc_smem + warp * kRing * kStepBytes) + lane;
-    uint2* frag = reinterpret_cast<uint2*>(tc_smem + kWarps * kRing * kStepBytes);
     __shared__ int ew[8];
-    const int g = lane >> 2, t = lane & 3;
-    const int c0 = blockIdx.y * 8;
-    const bool col = c0 + g < kc;
-    // ks warps share a tile of 16 rows, each a share of the steps
     __shared__ double part[kWarps][4][32];
-    const int tiles = kWarps / ks, sub = warp % ks;
-    const int64_t groups = (n + 16 * tiles - 1) / (16 * tiles);
+    const int rows = 16 * (kWarps / ks);
     bool staged = false;
-    for (int64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
-        const int64_t ra = grp * 16 * tiles + (warp / ks) * 16 + g, rb = ra + 8;
-            double out[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int k0 = 0; k0 < m; k0 += kMaxCols) {
-            const int cols = min(kMaxCols, m - k0), steps = (cols + 15) / 16;
-            if (!staged) {
-                __syncthreads();
-                if (tid < 8) ew[tid] = 0;
-                __syncthreads();
-                int mx = 0;
-                for (int s = warp; s < steps; s += kWarps)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
-                        if (col && a < cols) mx = max(mx, exp_bits(C[(int64_t)(k0 + a) * kc + c0 + g]));
-                    }
-#pragma unroll
-                for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                if (t == 0 && mx) atomicMax(&ew[g], mx >> 20);
-                __syncthreads();
-                const int eg = max(ew[g], kEmin);
-                for (int s = warp; s < steps; s += kWarps) {
-                    double x[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
-                        x[i] = (col && a < cols) ? C[(int64_t)(k0 + a) * kc + c0 + g] : 0.0;
-                    }
-                    store_frag(frag + s * kDig * 32, lane, x, eg);
-                }
-                __syncthreads();
-                staged = m <= kMaxCols;
-            }
-            // registers 0, 1: columns 2t, 2t+1 of rows g, g+8; 2, 3: columns 2t+8,
-            // 2t+9.  A lane copies its own 16-byte pairs into its ring and reads them back.
-            const int per = (steps + ks - 1) / ks, s0 = sub * per, s1 = min(steps, s0 + per);
-            const bool rows_in = grp * 16 * tiles + (warp / ks) * 16 + 16 <= n;
-            auto issue = [&](int s) {
-                if (s < s1) {
-                    const bool full = rows_in && k0 + 16 * s + 16 <= m;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int a = k0 + 16 * s + 8 * (i >> 1) + 2 * t;
-                        const int64_t r = (i & 1) ? rb : ra;
-                        const double* src = Q + ((int64_t)(a / B) * n + r) * B + a % B;
-                        double2* dst = ring + (s % kRing) * 128 + i * 32;
-                        if (full) cp_async16(dst, src);
-                        else cp_async16(dst, (a < m && r < n) ? src : Q, a < m && r < n);
-                    }
-                }
-                cp_async_commit();
-            };
-#pragma unroll
-            for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
-            Acc acc;
-            acc.clear();
-            LineScale sc;
-            auto flush = [&]() {
-                acc.to_int();
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    out[e] += unscale(acc.value(e), (e & 2) ? sc.E1 : sc.E0, max(ew[2 * t + (e & 1)], kEmin));
-                acc.clear();
-            };
-            for (int s = s0; s < s1; ++s) {
-                cp_async_wait<kRing - 2>();
-                double x[8];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const double2 v = ring[(s % kRing) * 128 + i * 32];
-                    x[2 * i] = v.x;
-                    x[2 * i + 1] = v.y;
-                }
-                issue(s + kRing - 1);  // into the buffer of step s - 1
-                step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
-                if (((s - s0) & 3) == 3) acc.to_int();
-            }
-            cp_async_wait<0>();
-            if (s0 < s1) flush();
-        }
-        if (ks > 1) {
-            __syncthreads();
-#pragma unroll
-            for (int e = 0; e < 4; ++e) part[warp][e][lane] = out[e];
-            __syncthreads();
-            if (sub != 0) continue;
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                for (int q = 1; q < ks; ++q) out[e] += part[warp + q][e][lane];
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int64_t r = (e & 2) ? rb : ra;
-            const int c = c0 + 2 * t + (e & 1);
-            if (r < n && c < kc) {
-                double* w = W + r * kc + c;
-                *w = SUB ? *w - out[e] : out[e];
-            }
-        }
-    }
+    for (int64_t row0 = (int64_t)blockIdx.x * rows; row0 < n; row0 += (int64_t)gridDim.x * rows)
+        update_group<B, SUB>(n, m, kc, ks, blockIdx.y * 8, row0, n, staged, Q, C, W, tc_smem, ew, part);
+}
+
+// Segmented: CTA x updates rows [ctas[3x+1], ctas[3x+2]) of segment s = ctas[3x]
+// with that segment's coefficients C + s * cstride and m = ms[s * ms_stride]
+// columns; inactive segments skip.
+template <int B>
+__global__ void __launch_bounds__(kT, 2) update_tc64_seg_kernel(int64_t n, const int* __restrict__ ms, int ms_stride,
+                                                                const int64_t* __restrict__ ctas,
+                                                                const int* __restrict__ seg_active, const double* Q,
+                                                                const double* __restrict__ C, int64_t cstride,
+                                                                double* W) {
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    __shared__ int ew[8];
+    __shared__ double part[kWarps][4][32];
+    const int64_t seg = ctas[3 * blockIdx.x];
+    if (seg_active && !seg_active[seg]) return;
+    const int m = ms[seg * ms_stride];
+    const int64_t r1 = ctas[3 * blockIdx.x + 2];
+    bool staged = false;
+    for (int64_t row0 = ctas[3 * blockIdx.x + 1]; row0 < r1; row0 += 16 * kWarps)
+        update_group<B, true>(n, m, B, 1, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew, part);
 }
 
 int sms() {
@@ -575,21 +664,6 @@ int sms() {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
     }
     return n;
-}
-
-// Shares of a chunk's steps per tile: the fewest rounds of steps over the
-// CTA's warps, counting an item's end (its FP64 conversions) as two steps.
-int gram_parts(int ntiles, int steps) {
-    int best = 1;
-    int64_t cost = INT64_MAX;
-    for (int p = 1; p <= kWarps && p <= steps; p <<= 1) {
-        const int64_t c = ceil_div((int64_t)ntiles * p, kWarps) * (ceil_div(steps, p) + 2);
-        if (c < cost) {
-            cost = c;
-            best = p;
-        }
-    }
-    return best;
 }
 
 constexpr int kFragBytes = kDig * 32 * (int)sizeof(uint2);  // a step's B fragments
@@ -604,12 +678,15 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
         attr = true;
     }
     constexpr int NH = (B + 7) / 8;
-    // rows per chunk: at least two chunks per SM where n allows it, at most the staged 512
-    int64_t rc = ceil_div(ceil_div(n, (int64_t)2 * sms()), 64) * 64;
+    // rows per chunk: one chunk per resident CTA where that gives at least 64 rows
+    // (n = 2e4: 80 rows, 250 chunks; with 64 rows a second wave held 9 of 313
+    // chunks), at most the staged 512
+    const int64_t resident = (int64_t)2 * gram_worker_sms();
+    int64_t rc = ceil_div(ceil_div(n, resident), 16) * 16;
     rc = std::min<int64_t>(std::max<int64_t>(rc, 64), kMaxRows);
-    const int parts = gram_parts((m + 15) / 16, (int)rc / 16);
+    const int parts = gram_parts((m + 15) / 16);
     const int64_t chunks = ceil_div(n, rc);
-    const int64_t ctas = std::min<int64_t>(chunks, (int64_t)2 * gram_worker_sms());
+    const int64_t ctas = std::min<int64_t>(chunks, resident);
     const int64_t per = (int64_t)m * B;
     BBL_TRY(partials.grow(sizeof(double) * (size_t)(ctas * per) + 256));
     int* tickets = reinterpret_cast<int*>(partials.as<double>() + ctas * per);
@@ -652,6 +729,54 @@ bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double
 // b = 2 (update) the FMA kernels have no more than two products per entry.
 bool tc64_gram_supports(int b, int m) { return (b == 2 && m >= 32) || ((b == 4 || b == 8 || b == 16) && m >= 16); }
 bool tc64_update_supports(int b, int m) { return (b == 4 || b == 8 || b == 16) && m >= 16; }
+
+namespace {
+
+template <int B>
+bbl_status launch_gram_seg(int64_t n, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
+                           int nchunks, const int* active, double* partial, cudaStream_t st) {
+    constexpr int kSmem = kRingBytes + kMaxRows / 16 * kFragBytes;
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(gram_tc64_seg_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+        attr = true;
+    }
+    gram_tc64_seg_kernel<B><<<(unsigned)nchunks, kT, kSmem, st>>>(n, d_m, chunks, active, Q, W, partial);
+    BBL_LAUNCH_CHECK();
+    return BBL_OK;
+}
+
+template <int B>
+bbl_status launch_update_seg(int64_t n, const int* ms, int ms_stride, const int64_t* ctas, int nctas, const int* active,
+                             const double* Q, const double* C, int64_t cstride, double* W, cudaStream_t st) {
+    constexpr int kSmem = kRingBytes + kMaxCols / 16 * kFragBytes;
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(update_tc64_seg_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+        attr = true;
+    }
+    update_tc64_seg_kernel<B><<<(unsigned)nctas, kT, kSmem, st>>>(n, ms, ms_stride, ctas, active, Q, C, cstride, W);
+    BBL_LAUNCH_CHECK();
+    return BBL_OK;
+}
+
+}  // namespace
+
+// (the chunks of a segmented Gram hold at most 512 rows)
+bool tc64_seg_supports(int b) { return b == 4 || b == 8; }
+
+bbl_status gram_tc64_seg(int64_t n, int b, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
+                         int nchunks, const int* active, double* partial, cudaStream_t st) {
+    if (b == 4) return launch_gram_seg<4>(n, d_m, Q, W, chunks, nchunks, active, partial, st);
+    return launch_gram_seg<8>(n, d_m, Q, W, chunks, nchunks, active, partial, st);
+}
+
+bbl_status update_tc64_seg(int64_t n, int b, const int* ms, int ms_stride, const int64_t* ctas, int nctas,
+                           const int* active, const double* Q, const double* C, int64_t cstride, double* W,
+                           cudaStream_t st) {
+    if (b == 4) return launch_update_seg<4>(n, ms, ms_stride, ctas, nctas, active, Q, C, cstride, W, st);
+    return launch_update_seg<8>(n, ms, ms_stride, ctas, nctas, active, Q, C, cstride, W, st);
+}
 
 bbl_status gram_tc64(int64_t n, int b, int m, const double* Q, const double* W, double* C, DevBuf& partials,
                      cudaStream_t st) {
