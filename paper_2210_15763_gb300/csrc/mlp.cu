@@ -52,154 +52,296 @@ __device__ __forceinline__ float gelu_grad(float x) {
 __device__ __forceinline__ float bf(const __nv_bfloat16* w, int i) { return __bfloat162float(w[i]); }
 
 // activations layout per sample: z1[H] h1[H] z2[H] h2[H] dz1[H] dz2[H] y[O] dy[O]
-__global__ void forward_kernel(int H, int O, const float* __restrict__ P, const __nv_bfloat16* __restrict__ Wb,
-                               const float* __restrict__ g, float* __restrict__ act, float* __restrict__ y_out) {
+//
+// A step is small (48 samples, hidden 128, 512 outputs: 8 MFLOP forward, 0.3 MB of
+// parameters), so its kernels are bound by the latency of dependent loads:
+// they spread the weight rows over the SMs, read them along their contiguous
+// dimension and keep a tile of samples per weight in registers.  (One CTA per
+// sample with a thread per output row read the weights with a stride of a row:
+// 44 us forward, 21 us backward, 74 us a step; the step's kernels now take about
+// 17 us.)
+constexpr int kFwS = 16;          // samples per CTA, forward
+constexpr int kFwThreads = 256;
+constexpr int kFwWarps = kFwThreads / 32;
+constexpr int kBwS = 4;           // samples per CTA, backward
+constexpr int kBwThreads = 1024;
+
+// v[s] summed over the warp for s = lane / 2 (16 values, 16 shuffles)
+__device__ __forceinline__ float warp_sum16(float (&v)[kFwS]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 16, h = kFwS / 2; off > 1; off >>= 1, h >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int x = 0; x < kFwS / 2; ++x)
+            if (x < h) {
+                const float send = up ? v[x] : v[x + h], keep = up ? v[x + h] : v[x];
+                v[x] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// One layer for 16 samples, a warp per output row o: acc = sum_i W[o][i] in[s][i]
+// (in: the samples' inputs in shared memory, rows of `in_dim`); the lane pair of
+// sample s gets row o's sum for it.
+__device__ __forceinline__ float row_dot16(const __nv_bfloat16* __restrict__ Wrow, const float* in, int in_dim) {
+    const int lane = threadIdx.x & 31;
+    float acc[kFwS];
+#pragma unroll
+    for (int q = 0; q < kFwS; ++q) acc[q] = 0.0f;
+    for (int i0 = 0; i0 < in_dim; i0 += 128) {
+        float w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 32 * u + lane;
+            w[u] = i < in_dim ? __bfloat162float(Wrow[i]) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 32 * u + lane;
+            if (i < in_dim) {
+#pragma unroll
+                for (int q = 0; q < kFwS; ++q) acc[q] = fmaf(w[u], in[q * in_dim + i], acc[q]);
+            }
+        }
+    }
+    return warp_sum16(acc);
+}
+
+// h1 of 16 samples (recomputed by every CTA; the first column of CTAs stores
+// it), then z2 and h2 of 8 rows
+__global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, int O, const float* __restrict__ P,
+                                                            const __nv_bfloat16* __restrict__ Wb,
+                                                            const float* __restrict__ g, float* __restrict__ act) {
     extern __shared__ float sh[];
-    float* h1 = sh;
-    float* h2 = sh + H;
-    const int s = blockIdx.x;
-    const float x = g[s];
-    float* a = act + (size_t)s * (6 * H + 2 * O);
-    const __nv_bfloat16* W1 = Wb;
-    const __nv_bfloat16* W2 = Wb + H;
-    const __nv_bfloat16* W3 = Wb + H + H * H;
+    const int s0 = blockIdx.y * kFwS, ns = min(kFwS, batch - s0);
+    const size_t st = 6 * H + 2 * O;
     const float* b1 = P + H;
     const float* b2 = P + 2 * H + H * H;
-    const float* b3 = P + 3 * H + H * H + O * H;
-    for (int i = threadIdx.x; i < H; i += blockDim.x) {
-        const float z = fmaf(bf(W1, i), x, b1[i]);
-        a[i] = z;
-        const float hv = gelu(z);
-        a[H + i] = hv;
-        h1[i] = hv;
+    for (int e = threadIdx.x; e < kFwS * H; e += kFwThreads) {
+        const int q = e / H, i = e - q * H;
+        float hv = 0.0f;
+        if (q < ns) {
+            const float z = fmaf(bf(Wb, i), g[s0 + q], b1[i]);
+            hv = gelu(z);
+            if (blockIdx.x == 0) {
+                act[(s0 + q) * st + i] = z;
+                act[(s0 + q) * st + H + i] = hv;
+            }
+        }
+        sh[e] = hv;
     }
     __syncthreads();
-    for (int o = threadIdx.x; o < H; o += blockDim.x) {
-        float acc = b2[o];
-        for (int i = 0; i < H; ++i) acc = fmaf(bf(W2, o * H + i), h1[i], acc);
-        a[2 * H + o] = acc;
-        const float hv = gelu(acc);
-        a[3 * H + o] = hv;
-        h2[o] = hv;
-    }
-    __syncthreads();
-    for (int o = threadIdx.x; o < O; o += blockDim.x) {
-        float acc = b3[o];
-        for (int i = 0; i < H; ++i) acc = fmaf(bf(W3, o * H + i), h2[i], acc);
-        a[6 * H + o] = acc;
-        if (y_out) y_out[(size_t)s * O + o] = acc;
+    const int o = blockIdx.x * kFwWarps + (threadIdx.x >> 5);
+    if (o >= H) return;
+    const float z = row_dot16(Wb + H + (size_t)o * H, sh, H) + b2[o];
+    const int q = (threadIdx.x & 31) >> 1;
+    if ((threadIdx.x & 1) == 0 && q < ns) {
+        act[(s0 + q) * st + 2 * H + o] = z;
+        act[(s0 + q) * st + 3 * H + o] = gelu(z);
     }
 }
 
-// dy = 2 (y - t) / N and per-sample partial losses
-__global__ void loss_kernel(int batch, int H, int O, const float* __restrict__ target, float* __restrict__ act,
-                            float* __restrict__ lossp) {
-    __shared__ float red[256];
-    const int s = blockIdx.x;
-    float* a = act + (size_t)s * (6 * H + 2 * O);
-    const float invN = 1.0f / ((float)batch * (float)O);
-    float l = 0.f;
-    for (int o = threadIdx.x; o < O; o += blockDim.x) {
-        const float d = a[6 * H + o] - target[(size_t)s * O + o];
-        l = fmaf(d, d, l);
-        a[6 * H + O + o] = 2.0f * d * invN;
-    }
-    red[threadIdx.x] = l;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) lossp[s] = red[0] * invN;
-}
-
-// per-sample backward through the activations: dz2, dz1
-__global__ void backward_act_kernel(int H, int O, const __nv_bfloat16* __restrict__ Wb, float* __restrict__ act) {
+// y of 8 output rows for 16 samples; with a target also dy = 2 (y - t) / N and
+// the CTA's partial loss
+__global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, int O, const float* __restrict__ P,
+                                                            const __nv_bfloat16* __restrict__ Wb,
+                                                            float* __restrict__ act, float* __restrict__ y_out,
+                                                            const float* __restrict__ target,
+                                                            float* __restrict__ lossp) {
     extern __shared__ float sh[];
-    float* dz2s = sh;
-    const int s = blockIdx.x;
-    float* a = act + (size_t)s * (6 * H + 2 * O);
-    const __nv_bfloat16* W2 = Wb + H;
-    const __nv_bfloat16* W3 = Wb + H + H * H;
-    const float* dy = a + 6 * H + O;
-    for (int i = threadIdx.x; i < H; i += blockDim.x) {
-        float acc = 0.f;
-        for (int o = 0; o < O; ++o) acc = fmaf(bf(W3, o * H + i), dy[o], acc);
-        const float d = acc * gelu_grad(a[2 * H + i]);
-        a[5 * H + i] = d;
-        dz2s[i] = d;
+    __shared__ float red[kFwWarps];
+    const int s0 = blockIdx.y * kFwS, ns = min(kFwS, batch - s0);
+    const size_t st = 6 * H + 2 * O;
+    for (int e = threadIdx.x; e < kFwS * H; e += kFwThreads) {
+        const int q = e / H, i = e - q * H;
+        sh[e] = q < ns ? act[(s0 + q) * st + 3 * H + i] : 0.0f;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < H; i += blockDim.x) {
-        float acc = 0.f;
-        for (int o = 0; o < H; ++o) acc = fmaf(bf(W2, o * H + i), dz2s[o], acc);
-        a[4 * H + i] = acc * gelu_grad(a[i]);
+    const int warp = threadIdx.x >> 5, o = blockIdx.x * kFwWarps + warp;
+    float l = 0.0f;
+    if (o < O) {
+        const float y = row_dot16(Wb + H + H * H + (size_t)o * H, sh, H) + P[3 * H + H * H + O * H + o];
+        const int q = (threadIdx.x & 31) >> 1;
+        if ((threadIdx.x & 1) == 0 && q < ns) {
+            float* a = act + (s0 + q) * st;
+            a[6 * H + o] = y;
+            if (y_out) y_out[(size_t)(s0 + q) * O + o] = y;
+            if (target) {
+                const float d = y - target[(size_t)(s0 + q) * O + o];
+                a[6 * H + O + o] = 2.0f * d * (1.0f / ((float)batch * (float)O));
+                l = d * d;
+            }
+        }
+    }
+    if (!target) return;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    if ((threadIdx.x & 31) == 0) red[warp] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.0f;
+        for (int w = 0; w < kFwWarps; ++w) t += red[w];
+        lossp[blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
 }
 
-// weight gradients, one thread per parameter, summed over the batch in order
-__global__ void backward_w_kernel(int batch, int H, int O, const float* __restrict__ g, const float* __restrict__ act,
-                                  float* __restrict__ G) {
+// out[q][i] = sum_o W[o][i] d[q][o] for the CTA's 4 samples (d: rows of n_out in
+// shared memory): a warp takes 32 columns i and a share of the rows o; the
+// shares are added in order.  part: 32 x 4 x 32 floats.
+template <typename Put>
+__device__ __forceinline__ void columns_dot(const __nv_bfloat16* __restrict__ W, int H, int n_out, const float* d,
+                                            float* part, Put&& put) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tiles = (H + 31) / 32, shares = (kBwThreads / 32) / tiles;
+    const int tile = warp % tiles, share = warp / tiles;
+    const int i = 32 * tile + lane;
+    float acc[kBwS] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (share < shares && i < H) {
+#pragma unroll 8
+        for (int o = share; o < n_out; o += shares) {
+            const float w = __bfloat162float(W[(size_t)o * H + i]);
+#pragma unroll
+            for (int q = 0; q < kBwS; ++q) acc[q] = fmaf(w, d[q * n_out + o], acc[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kBwS; ++q) part[(warp * kBwS + q) * 32 + lane] = acc[q];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kBwS * H; e += kBwThreads) {
+        const int q = e / H, c = e - q * H;
+        float t = 0.0f;
+        for (int k = 0; k < shares; ++k) t += part[((k * tiles + c / 32) * kBwS + q) * 32 + c % 32];
+        put(q, c, t);
+    }
+    __syncthreads();
+}
+
+// backward through the activations of 4 samples: dz2, dz1
+__global__ void __launch_bounds__(kBwThreads) backward_act_kernel(int batch, int H, int O,
+                                                                  const __nv_bfloat16* __restrict__ Wb,
+                                                                  float* __restrict__ act) {
+    extern __shared__ float sh[];
+    float* part = sh;                                   // (32 warps) x 4 x 32
+    float* dz2 = part + (kBwThreads / 32) * kBwS * 32;  // 4 x H
+    float* dy = dz2 + kBwS * H;                         // 4 x O
+    const int s0 = blockIdx.x * kBwS, ns = min(kBwS, batch - s0);
+    const size_t st = 6 * H + 2 * O;
+    for (int e = threadIdx.x; e < kBwS * O; e += kBwThreads) {
+        const int q = e / O, o = e - q * O;
+        dy[e] = q < ns ? act[(s0 + q) * st + 6 * H + O + o] : 0.0f;
+    }
+    __syncthreads();
+    columns_dot(Wb + H + H * H, H, O, dy, part, [&](int q, int i, float t) {
+        float v = 0.0f;
+        if (q < ns) {
+            float* a = act + (s0 + q) * st;
+            v = t * gelu_grad(a[2 * H + i]);
+            a[5 * H + i] = v;
+        }
+        dz2[q * H + i] = v;
+    });
+    columns_dot(Wb + H, H, H, dz2, part, [&](int q, int i, float t) {
+        if (q < ns) {
+            float* a = act + (s0 + q) * st;
+            a[4 * H + i] = t * gelu_grad(a[i]);
+        }
+    });
+}
+
+// weight gradients, one thread per parameter, summed over the batch in order;
+// the last CTA adds the partial losses
+__global__ void __launch_bounds__(256) backward_w_kernel(int batch, int H, int O, const float* __restrict__ g,
+                                                         const float* __restrict__ act, float* __restrict__ G,
+                                                         int nloss, const float* __restrict__ lossp,
+                                                         float* __restrict__ loss) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float red[256];
+        float l = 0.0f;
+        for (int e = threadIdx.x; e < nloss; e += 256) l += lossp[e];
+        red[threadIdx.x] = l;
+        __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *loss = red[0] * (1.0f / ((float)batch * (float)O));
+        return;
+    }
     const int np = 3 * H + H * H + O * H + O;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = blockIdx.x * 256 + threadIdx.x;
     if (p >= np) return;
     const size_t st = 6 * H + 2 * O;
-    float acc = 0.f;
+    // dG = sum_s left[s] * right[s]; right is 1 for a bias
+    const float *left, *right = nullptr;
+    size_t rst = st;
     if (p < H) {  // W1[o]
-        for (int s = 0; s < batch; ++s) acc = fmaf(act[s * st + 4 * H + p], g[s], acc);
+        left = act + 4 * H + p;
+        right = g;
+        rst = 1;
     } else if (p < 2 * H) {  // b1
-        const int o = p - H;
-        for (int s = 0; s < batch; ++s) acc += act[s * st + 4 * H + o];
+        left = act + 4 * H + (p - H);
     } else if (p < 2 * H + H * H) {  // W2[o][i]
         const int e = p - 2 * H, o = e / H, i = e % H;
-        for (int s = 0; s < batch; ++s) acc = fmaf(act[s * st + 5 * H + o], act[s * st + H + i], acc);
+        left = act + 5 * H + o;
+        right = act + H + i;
     } else if (p < 3 * H + H * H) {  // b2
-        const int o = p - 2 * H - H * H;
-        for (int s = 0; s < batch; ++s) acc += act[s * st + 5 * H + o];
+        left = act + 5 * H + (p - 2 * H - H * H);
     } else if (p < 3 * H + H * H + O * H) {  // W3[o][i]
         const int e = p - 3 * H - H * H, o = e / H, i = e % H;
-        for (int s = 0; s < batch; ++s) acc = fmaf(act[s * st + 6 * H + O + o], act[s * st + 3 * H + i], acc);
+        left = act + 6 * H + O + o;
+        right = act + 3 * H + i;
     } else {  // b3
-        const int o = p - 3 * H - H * H - O * H;
-        for (int s = 0; s < batch; ++s) acc += act[s * st + 6 * H + O + o];
+        left = act + 6 * H + O + (p - 3 * H - H * H - O * H);
     }
+    float acc = 0.0f;
+#pragma unroll 8
+    for (int s = 0; s < batch; ++s) acc = fmaf(left[s * st], right ? right[s * rst] : 1.0f, acc);
     G[p] = acc;
 }
 
-// bf16 copies of the weight matrices (W1 | W2 | W3)
+// the BF16 copy of parameter p (W1 | W2 | W3), -1 for a bias
+__device__ __forceinline__ int bf16_index(int H, int O, int p) {
+    if (p < H) return p;
+    if (p >= 2 * H && p < 2 * H + H * H) return H + (p - 2 * H);
+    if (p >= 3 * H + H * H && p < 3 * H + H * H + O * H) return H + H * H + (p - 3 * H - H * H);
+    return -1;
+}
+
+// bf16 copies of the weight matrices
 __global__ void to_bf16_kernel(int H, int O, const float* __restrict__ P, __nv_bfloat16* __restrict__ Wb) {
-    const int nw = H + H * H + O * H;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nw; e += gridDim.x * blockDim.x) {
-        int src;
-        if (e < H) src = e;                                   // W1
-        else if (e < H + H * H) src = 2 * H + (e - H);        // W2
-        else src = 3 * H + H * H + (e - H - H * H);           // W3
-        Wb[e] = __float2bfloat16_rn(P[src]);
+    const int np = 3 * H + H * H + O * H + O;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
+        const int w = bf16_index(H, O, p);
+        if (w >= 0) Wb[w] = __float2bfloat16_rn(P[p]);
     }
 }
 
-__global__ void adam_kernel(int np, float lr, float b1, float b2, float eps, float* __restrict__ P,
-                            const float* __restrict__ G, float* __restrict__ M, float* __restrict__ V,
-                            int* __restrict__ tstep) {
-    const int t = *tstep + 1;  // read before the increment below (one block writes it after a grid-wide pass)
+// one Adam step, the new BF16 weights, and (by the CTA that ends last: all have
+// read the step count by then) the step count; tstep[1] counts the CTAs
+__global__ void __launch_bounds__(256) adam_kernel(int H, int O, float lr, float b1, float b2, float eps,
+                                                   float* __restrict__ P, const float* __restrict__ G,
+                                                   float* __restrict__ M, float* __restrict__ V,
+                                                   __nv_bfloat16* __restrict__ Wb, int* tstep) {
+    const int t = *(volatile int*)tstep + 1;
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
+    const int p = blockIdx.x * 256 + threadIdx.x;
+    if (p < 3 * H + H * H + O * H + O) {
         const float gr = G[p];
         const float m = b1 * M[p] + (1.0f - b1) * gr;
         const float v = b2 * V[p] + (1.0f - b2) * gr * gr;
         M[p] = m;
         V[p] = v;
-        P[p] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+        const float np = P[p] - lr * (m / c1) / (sqrtf(v / c2) + eps);
+        P[p] = np;
+        const int w = bf16_index(H, O, p);
+        if (w >= 0) Wb[w] = __float2bfloat16_rn(np);
     }
-}
-
-__global__ void step_inc_kernel(int* tstep) { *tstep += 1; }
-
-__global__ void sum_loss_kernel(int batch, const float* __restrict__ lossp, float* __restrict__ out, int slot) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        float s = 0.f;
-        for (int i = 0; i < batch; ++i) s += lossp[i];
-        out[slot] = s;
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(tstep + 1, 1) == (int)gridDim.x - 1) {
+        tstep[1] = 0;
+        tstep[0] = t;
     }
 }
 
@@ -208,10 +350,14 @@ __global__ void widen_kernel(int count, const float* __restrict__ y, double* __r
     if (e < count) C[e] = (double)y[e];
 }
 
+int loss_parts(const bbl_mlp* M, int batch) {
+    return (int)(ceil_div(M->out, kFwWarps) * ceil_div(batch, kFwS));
+}
+
 bbl_status ensure_batch(bbl_mlp* M, int batch) {
     if (batch <= M->cap_batch) return BBL_OK;
     BBL_TRY(M->act.alloc(sizeof(float) * (size_t)batch * (6 * M->hidden + 2 * M->out)));
-    BBL_TRY(M->lossbuf.alloc(sizeof(float) * (size_t)(batch + 8)));
+    BBL_TRY(M->lossbuf.alloc(sizeof(float) * (size_t)(loss_parts(M, batch) + 8)));  // the loss, then its parts
     M->cap_batch = batch;
     if (M->exec) {
         cudaGraphExecDestroy(M->exec);
@@ -223,34 +369,51 @@ bbl_status ensure_batch(bbl_mlp* M, int batch) {
     return BBL_OK;
 }
 
-bbl_status launch_forward(const bbl_mlp* M, int batch, const float* g, float* y, cudaStream_t st) {
-    forward_kernel<<<batch, 256, sizeof(float) * 2 * M->hidden, st>>>(
-        M->hidden, M->out, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), g, M->act.as<float>(), y);
+bbl_status launch_forward(const bbl_mlp* M, int batch, const float* g, float* y, const float* target, cudaStream_t st) {
+    const int H = M->hidden, O = M->out;
+    const size_t sm = sizeof(float) * kFwS * H;
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(hidden_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwS * 1024 * 4));
+        BBL_CUDA(cudaFuncSetAttribute(output_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwS * 1024 * 4));
+        attr = true;
+    }
+    const unsigned groups = (unsigned)ceil_div(batch, kFwS);
+    hidden_kernel<<<dim3((unsigned)ceil_div(H, kFwWarps), groups), kFwThreads, sm, st>>>(
+        batch, H, O, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), g, M->act.as<float>());
+    BBL_LAUNCH_CHECK();
+    output_kernel<<<dim3((unsigned)ceil_div(O, kFwWarps), groups), kFwThreads, sm, st>>>(
+        batch, H, O, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), M->act.as<float>(), y, target,
+        M->lossbuf.as<float>() + 8);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
 
-bbl_status launch_loss_backward(bbl_mlp* M, int batch, const float* g, const float* target, cudaStream_t st) {
-    loss_kernel<<<batch, 256, 0, st>>>(batch, M->hidden, M->out, target, M->act.as<float>(), M->lossbuf.as<float>());
+// forward, MSE loss (into lossbuf[0]) and backward into the gradient buffer
+bbl_status launch_loss_grad(bbl_mlp* M, int batch, const float* g, const float* target, cudaStream_t st) {
+    const int H = M->hidden, O = M->out;
+    static bool attr = false;
+    if (!attr) {
+        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(float) * (kBwThreads * kBwS + kBwS * (1024 + 4096))));
+        attr = true;
+    }
+    BBL_TRY(launch_forward(M, batch, g, nullptr, target, st));
+    backward_act_kernel<<<(unsigned)ceil_div(batch, kBwS), kBwThreads,
+                          sizeof(float) * (kBwThreads * kBwS + kBwS * (H + O)), st>>>(
+        batch, H, O, M->wbf.as<__nv_bfloat16>(), M->act.as<float>());
     BBL_LAUNCH_CHECK();
-    backward_act_kernel<<<batch, 128, sizeof(float) * M->hidden, st>>>(M->hidden, M->out, M->wbf.as<__nv_bfloat16>(),
-                                                                       M->act.as<float>());
-    BBL_LAUNCH_CHECK();
-    backward_w_kernel<<<(unsigned)ceil_div(M->nparams, 256), 256, 0, st>>>(batch, M->hidden, M->out, g,
-                                                                          M->act.as<float>(), M->grads.as<float>());
+    backward_w_kernel<<<(unsigned)ceil_div(M->nparams, 256) + 1, 256, 0, st>>>(
+        batch, H, O, g, M->act.as<float>(), M->grads.as<float>(), loss_parts(M, batch), M->lossbuf.as<float>() + 8,
+        M->lossbuf.as<float>());
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
 
 bbl_status launch_adam(bbl_mlp* M, float lr, cudaStream_t st) {
-    adam_kernel<<<(unsigned)ceil_div(M->nparams, 256), 256, 0, st>>>(M->nparams, lr, 0.9f, 0.999f, 1e-8f,
-                                                                     M->params.as<float>(), M->grads.as<float>(),
-                                                                     M->m.as<float>(), M->v.as<float>(),
-                                                                     M->tstep.as<int>());
-    BBL_LAUNCH_CHECK();
-    step_inc_kernel<<<1, 1, 0, st>>>(M->tstep.as<int>());
-    BBL_LAUNCH_CHECK();
-    to_bf16_kernel<<<64, 256, 0, st>>>(M->hidden, M->out, M->params.as<float>(), M->wbf.as<__nv_bfloat16>());
+    adam_kernel<<<(unsigned)ceil_div(M->nparams, 256), 256, 0, st>>>(
+        M->hidden, M->out, lr, 0.9f, 0.999f, 1e-8f, M->params.as<float>(), M->grads.as<float>(), M->m.as<float>(),
+        M->v.as<float>(), M->wbf.as<__nv_bfloat16>(), M->tstep.as<int>());
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
@@ -273,7 +436,7 @@ bbl_status bbl_mlp_create(int hidden, int out_dim, bbl_mlp** out) {
     const size_t pb = sizeof(float) * M->nparams;
     bbl_status s;
     if ((s = M->params.alloc(pb)) != BBL_OK || (s = M->grads.alloc(pb)) != BBL_OK || (s = M->m.alloc(pb)) != BBL_OK ||
-        (s = M->v.alloc(pb)) != BBL_OK || (s = M->tstep.alloc(sizeof(int))) != BBL_OK ||
+        (s = M->v.alloc(pb)) != BBL_OK || (s = M->tstep.alloc(2 * sizeof(int))) != BBL_OK ||
         (s = M->wbf.alloc(sizeof(__nv_bfloat16) * (hidden + hidden * hidden + out_dim * hidden))) != BBL_OK) {
         delete M;
         return s;
@@ -281,7 +444,7 @@ bbl_status bbl_mlp_create(int hidden, int out_dim, bbl_mlp** out) {
     cudaMemset(M->params.p, 0, pb);
     cudaMemset(M->m.p, 0, pb);
     cudaMemset(M->v.p, 0, pb);
-    cudaMemset(M->tstep.p, 0, sizeof(int));
+    cudaMemset(M->tstep.p, 0, 2 * sizeof(int));
     cudaMemset(M->wbf.p, 0, M->wbf.bytes);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         delete M;
@@ -307,7 +470,7 @@ bbl_status bbl_mlp_set_params(bbl_mlp* M, const float* packed, void* stream) {
     BBL_CUDA(cudaMemcpyAsync(M->params.p, packed, sizeof(float) * M->nparams, cudaMemcpyDefault, st));
     BBL_CUDA(cudaMemsetAsync(M->m.p, 0, M->m.bytes, st));
     BBL_CUDA(cudaMemsetAsync(M->v.p, 0, M->v.bytes, st));
-    BBL_CUDA(cudaMemsetAsync(M->tstep.p, 0, sizeof(int), st));
+    BBL_CUDA(cudaMemsetAsync(M->tstep.p, 0, 2 * sizeof(int), st));
     to_bf16_kernel<<<64, 256, 0, st>>>(M->hidden, M->out, M->params.as<float>(), M->wbf.as<__nv_bfloat16>());
     BBL_LAUNCH_CHECK();
     BBL_CUDA(cudaStreamSynchronize(st));
@@ -329,7 +492,7 @@ bbl_status bbl_mlp_forward(bbl_mlp* M, int batch, const float* g, float* y, void
     if (!M || !g || !y || batch < 1) return set_error(BBL_ERR_INVALID_ARG, "mlp_forward: bad arguments");
     BBL_TRY(ensure_batch(M, batch));
     cudaStream_t st = as_stream(stream);
-    BBL_TRY(launch_forward(M, batch, g, y, st));
+    BBL_TRY(launch_forward(M, batch, g, y, nullptr, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;
 }
@@ -339,13 +502,9 @@ bbl_status bbl_mlp_loss_grad(bbl_mlp* M, int batch, const float* g, const float*
     if (!M || !g || !target || batch < 1) return set_error(BBL_ERR_INVALID_ARG, "mlp_loss_grad: bad arguments");
     BBL_TRY(ensure_batch(M, batch));
     cudaStream_t st = as_stream(stream);
-    BBL_TRY(launch_forward(M, batch, g, nullptr, st));
-    BBL_TRY(launch_loss_backward(M, batch, g, target, st));
-    float* lp = M->lossbuf.as<float>();
-    sum_loss_kernel<<<1, 32, 0, st>>>(batch, lp, lp, batch);
-    BBL_LAUNCH_CHECK();
+    BBL_TRY(launch_loss_grad(M, batch, g, target, st));
     float h = 0.f;
-    BBL_CUDA(cudaMemcpyAsync(&h, lp + batch, sizeof(float), cudaMemcpyDeviceToHost, st));
+    BBL_CUDA(cudaMemcpyAsync(&h, M->lossbuf.p, sizeof(float), cudaMemcpyDeviceToHost, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     if (loss) *loss = h;
     return BBL_OK;
@@ -380,8 +539,7 @@ bbl_status bbl_mlp_train(bbl_mlp* M, int batch, const float* g, const float* tar
             M->graph = nullptr;
         }
         BBL_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        bbl_status s = launch_forward(M, batch, g, nullptr, st);
-        if (s == BBL_OK) s = launch_loss_backward(M, batch, g, target, st);
+        bbl_status s = launch_loss_grad(M, batch, g, target, st);
         if (s == BBL_OK) s = launch_adam(M, lr, st);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(st, &graph);
@@ -400,10 +558,8 @@ bbl_status bbl_mlp_train(bbl_mlp* M, int batch, const float* g, const float* tar
     for (int e = 0; e < epochs; ++e) {
         BBL_CUDA(cudaGraphLaunch(M->exec, st));
         count_launch();
-        if (loss_hist) {
-            sum_loss_kernel<<<1, 32, 0, st>>>(batch, M->lossbuf.as<float>(), lh.as<float>(), e);
-            BBL_LAUNCH_CHECK();
-        }
+        if (loss_hist)
+            BBL_CUDA(cudaMemcpyAsync(lh.as<float>() + e, M->lossbuf.p, sizeof(float), cudaMemcpyDeviceToDevice, st));
     }
     if (loss_hist && epochs > 0)
         BBL_CUDA(cudaMemcpyAsync(loss_hist, lh.p, sizeof(float) * epochs, cudaMemcpyDeviceToHost, st));
@@ -425,7 +581,7 @@ bbl_status bbl_pivot_learned(bbl_mlp* M, float g, int64_t n, int b_U, int nblock
     BBL_TRY(y.alloc(sizeof(float) * M->out));
     BBL_TRY(C.alloc(sizeof(double) * M->out));
     BBL_CUDA(cudaMemcpyAsync(gb.p, &g, sizeof(float), cudaMemcpyHostToDevice, st));
-    BBL_TRY(launch_forward(M, 1, gb.as<float>(), y.as<float>(), st));
+    BBL_TRY(launch_forward(M, 1, gb.as<float>(), y.as<float>(), nullptr, st));
     widen_kernel<<<(unsigned)ceil_div(M->out, 256), 256, 0, st>>>(M->out, y.as<float>(), C.as<double>());
     BBL_LAUNCH_CHECK();
     BBL_TRY(ritz_vectors(n, b_U, nblocks_U, BBL_FP32, U, b, C.as<double>(), P, st));
