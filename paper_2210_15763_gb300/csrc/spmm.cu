@@ -100,8 +100,9 @@ __device__ __forceinline__ void store_pack(T* p, const T (&v)[N]) {
     }
 }
 
-// CSR, G lanes per row (G a power of two, LPN <= G <= 32).
-template <typename TM, typename TX, int B, int G>
+// CSR, G lanes per row (G a power of two, LPN <= G <= 32), NA running sums per
+// value in a lane.
+template <typename TM, typename TX, int B, int G, int NA = 1>
 __global__ void __launch_bounds__(256) spmm_csr_kernel(int64_t n, const int64_t* __restrict__ rp,
                                                        const int* __restrict__ ci, const TM* __restrict__ va,
                                                        const TX* __restrict__ V, TX* __restrict__ W) {
@@ -116,18 +117,35 @@ __global__ void __launch_bounds__(256) spmm_csr_kernel(int64_t n, const int64_t*
     const int sub = gl % LPN;
     const int slot = gl / LPN;
     const int64_t s = rp[row], e = rp[row + 1];
-    TX acc[VEC];
+    TX part[NA][VEC];
 #pragma unroll
-    for (int q = 0; q < VEC; ++q) acc[q] = TX(0);
-#pragma unroll 4
-    for (int64_t k = s + slot; k < e; k += NPS) {
-        const int c = __ldg(ci + k);
-        const HType<TM, TX> h = (HType<TM, TX>)__ldg(va + k);
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) part[a][q] = TX(0);
+    int64_t k = s + slot;
+    auto term = [&](int64_t i, TX (&sum)[VEC]) {
+        const int c = __ldg(ci + i);
+        const HType<TM, TX> h = (HType<TM, TX>)__ldg(va + i);
         TX v[VEC];
         load_pack<TX, VEC>(V + (int64_t)c * B + sub * VEC, v);
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] = fma(h, v[q], acc[q]);
+        for (int q = 0; q < VEC; ++q) sum[q] = fma(h, v[q], sum[q]);
+    };
+#pragma unroll 4 / NA
+    for (; k + (NA - 1) * NPS < e; k += NA * NPS) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) term(k + a * NPS, part[a]);
     }
+#pragma unroll
+    for (int a = 0; a < NA - 1; ++a)
+        if (k + a * NPS < e) term(k + a * NPS, part[a]);
+#pragma unroll
+    for (int h = 1; h < NA; h <<= 1)
+#pragma unroll
+        for (int a = 0; a + h < NA; a += 2 * h)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) part[a][q] = part[a][q] + part[a + h][q];
+    TX(&acc)[VEC] = part[0];
 #pragma unroll
     for (int off = LPN; off < G; off <<= 1) {
 #pragma unroll
@@ -287,17 +305,22 @@ struct CsrRows {
     int64_t r0;
 };
 
-template <typename TM, typename TX, int B, int G>
+template <typename TM, typename TX, int B, int G, int NA = 1>
 void launch_csr(const CsrRows& R, const TM* val, const TX* V, TX* W, cudaStream_t st) {
     const int64_t threads = R.nr * G;
     const int64_t blocks = ceil_div(threads, 256);
-    spmm_csr_kernel<TM, TX, B, G><<<(unsigned)blocks, 256, 0, st>>>(R.nr, R.rp, R.ci, val, V, W + R.r0 * B);
+    spmm_csr_kernel<TM, TX, B, G, NA><<<(unsigned)blocks, 256, 0, st>>>(R.nr, R.rp, R.ci, val, V, W + R.r0 * B);
 }
 
 template <typename TM, typename TX, int B>
-void launch_csr_g(const CsrRows& R, const TM* val, const TX* V, TX* W, int G, cudaStream_t st) {
+void launch_csr_g(const CsrRows& R, const TM* val, const TX* V, TX* W, int G, int na, cudaStream_t st) {
     constexpr int LPN = VecLayout<TX, B>::LPN;
     if (G < LPN) G = LPN;
+    if constexpr (std::is_same<TX, double>::value && B <= 4) {
+        if (na == 4 && G == 8) { launch_csr<TM, TX, B, 8, 4>(R, val, V, W, st); return; }
+        if (na == 2 && G == 8) { launch_csr<TM, TX, B, 8, 2>(R, val, V, W, st); return; }
+        if (na == 2 && G == 16) { launch_csr<TM, TX, B, 16, 2>(R, val, V, W, st); return; }
+    }
     switch (G) {
         case 1: if constexpr (LPN <= 1) { launch_csr<TM, TX, B, 1>(R, val, V, W, st); return; } break;
         case 2: if constexpr (LPN <= 2) { launch_csr<TM, TX, B, 2>(R, val, V, W, st); return; } break;
@@ -310,7 +333,7 @@ void launch_csr_g(const CsrRows& R, const TM* val, const TX* V, TX* W, int G, cu
 }
 
 // Lanes per row: about the average row length / 2, clamped to [LPN, 32].
-int default_group(const bbl_matrix* A) {
+int spmm_lanes(const bbl_matrix* A) {
     const double avg = A->n ? (double)A->nnz / (double)A->n : 0.0;
     if (avg >= 48) return 32;
     if (avg >= 24) return 16;
@@ -322,7 +345,30 @@ int default_group(const bbl_matrix* A) {
 template <typename TM, typename TX>
 bbl_status spmm_typed(const bbl_matrix* A, int b, const TM* csr_val, const TM* sell_val, const TX* V, TX* W,
                       cudaStream_t st, int G, int64_t r0 = 0, int64_t r1 = -1) {
-    if (G <= 0) G = A->spmm_lanes > 0 ? A->spmm_lanes : default_group(A);
+    int na = 1;  // running sums per lane and value
+    if (G <= 0 && A->spmm_lanes > 0) G = A->spmm_lanes;
+    if (G <= 0) {
+        G = spmm_lanes(A);
+        if (std::is_same<TX, double>::value && b <= 4) {
+            // FP64 arithmetic issues at 1/64 of the FP32 rate, and the tree over a row's
+            // lanes is FP64 additions by all of them (b = 4, 32 lanes: 8 beside 12.5
+            // products per 100-entry row).  So 8 lanes, more only where the GPU would not
+            // be full, each with as many running sums as it replaces lanes: the chains
+            // of additions, and with them the rounding, stay as they were.  With b >= 8
+            // a row has few lanes to add over.  Us before -> now: n = 3e5, 106 per row, b = 1 /
+            // 2 / 4: 179 / 350 / 400 -> 121 / 210 / 328 (8 lanes); 276 per row: 180 / 341 / 496 ->
+            // 178 / 272 / 475; n = 2e4, 99 per row: 16.5 / 28.8 / 31.4 -> 13.1 / 22.4 / 29.3 (16
+            // lanes; 8: 31.2 at b = 4); n = 2e4, 31 per row, b = 4: 16.3 -> 14.4 (8 for 16).  Of
+            // these 475 us at 2 b nnz flop are 0.93 of the measured FP64 rate.
+            const int64_t fill = (int64_t)152 * (A->nnz >= 48 * A->n ? 2048 : 1024);
+            int g = 8;
+            while (g < 32 && A->n * g < fill) g <<= 1;
+            if (g < G) {
+                na = G / g;
+                G = g;
+            }
+        }
+    }
     const bool pow2 = (b == 1 || b == 2 || b == 4 || b == 8 || b == 16);
     const bool ranged = r1 >= 0;  // rows [r0, r1) only, from the CSR copy
     if (r1 < 0) r1 = A->n;
@@ -349,11 +395,11 @@ bbl_status spmm_typed(const bbl_matrix* A, int b, const TM* csr_val, const TM* s
     const CsrRows R{r1 - r0, A->row_ptr.as<int64_t>() + r0, A->col.as<int>(), r0};
     if (R.nr <= 0) return BBL_OK;
     switch (pow2 ? b : 0) {
-        case 1: launch_csr_g<TM, TX, 1>(R, csr_val, V, W, G, st); break;
-        case 2: launch_csr_g<TM, TX, 2>(R, csr_val, V, W, G, st); break;
-        case 4: launch_csr_g<TM, TX, 4>(R, csr_val, V, W, G, st); break;
-        case 8: launch_csr_g<TM, TX, 8>(R, csr_val, V, W, G, st); break;
-        case 16: launch_csr_g<TM, TX, 16>(R, csr_val, V, W, G, st); break;
+        case 1: launch_csr_g<TM, TX, 1>(R, csr_val, V, W, G, na, st); break;
+        case 2: launch_csr_g<TM, TX, 2>(R, csr_val, V, W, G, na, st); break;
+        case 4: launch_csr_g<TM, TX, 4>(R, csr_val, V, W, G, na, st); break;
+        case 8: launch_csr_g<TM, TX, 8>(R, csr_val, V, W, G, na, st); break;
+        case 16: launch_csr_g<TM, TX, 16>(R, csr_val, V, W, G, na, st); break;
         default: {
             const int64_t blocks = ceil_div(R.nr * 32, 256);
             spmm_csr_generic<TM, TX><<<(unsigned)blocks, 256, 0, st>>>(R.nr, b, R.rp, R.ci, csr_val, V, W + r0 * b);
