@@ -93,8 +93,11 @@ __device__ __forceinline__ double pow2(int e) {
     return __hiloint2double((e + 1023) << 20, 0);
 }
 
-// v * 2^e for any e (two exact powers of two)
+// v * 2^e: the exponent field moved by integer arithmetic where v and the
+// result are normal, else by two exact powers of two
 __device__ __forceinline__ double scale_by(double v, int e) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7ff;
+    if (ex > 0 && ex < 0x7ff && ex + e > 0 && ex + e < 0x7ff) return __hiloint2double(hi + e * (1 << 20), __double2loint(v));
     const int h = e / 2;
     return v * pow2(h) * pow2(e - h);
 }
@@ -333,11 +336,13 @@ __host__ __device__ inline int gram_parts(int ntiles) {
     return p;
 }
 
-// rows [r0, r0 + rows) (at most 512), columns c0 .. c0 + 7 of W: added to slot (m x B).
+// Basis tiles tile0 .. tile0 + ntiles - 1 (16 columns each) of rows [r0, r0 +
+// rows) (at most 512) and columns c0 .. c0 + 7 of W: added to slot (m x B).
 // All threads, after a barrier that follows the last use of smem and the zeroing
 // of slot and ew.
 template <int B>
-__device__ __forceinline__ void gram_chunk(int64_t n, int m, int parts, int64_t r0, int rows, int c0,
+__device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntiles, int parts, int64_t r0, int rows,
+                                           int c0,
                                            const double* __restrict__ Q, const double* __restrict__ W,
                                            double* __restrict__ slot, unsigned char* smem, int* ew,
                                            double (*sums)[128]) {
@@ -346,7 +351,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int parts, int64_t 
     uint2* frag = reinterpret_cast<uint2*>(smem + kWarps * kRing * kStepBytes);
     const int g = lane >> 2, t = lane & 3;
     const bool col = c0 + g < B;
-    const int items = (m + 15) / 16 * parts;
+    const int items = ntiles * parts;
     // a step of a tile in the ring: block-major, then rows of B entries
     constexpr int CPR = B / 2;                       // 16-byte chunks per row
     constexpr int CPB = 16 * CPR;                    // chunks per block (B = 2, 4, 8, 16: 16 .. 128)
@@ -379,7 +384,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int parts, int64_t 
     __syncthreads();
     const int per = (steps + parts - 1) / parts;
     for (int w = warp; w < items; w += kWarps) {
-        const int tile = w / parts, part = w % parts;
+        const int tile = tile0 + w / parts, part = w % parts;
         const int s0 = part * per, s1 = min(steps, s0 + per);
         if (s0 >= s1) continue;
         const int j0 = 16 * tile / B, nblk = (m - 16 * tile) / B;  // first block and blocks left
@@ -450,14 +455,15 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int parts, int64_t 
             const int tile = e / 128, q = e % 128, l = q & 31;
             double v = 0.0;
             for (int p = 0; p < parts && p * ((steps + parts - 1) / parts) < steps; ++p) v += sums[tile * parts + p][q];
-            const int a = 16 * tile + (l >> 2) + ((q & 64) ? 8 : 0), c = c0 + 2 * (l & 3) + ((q & 32) ? 1 : 0);
+            const int a = 16 * (tile0 + tile) + (l >> 2) + ((q & 64) ? 8 : 0), c = c0 + 2 * (l & 3) + ((q & 32) ? 1 : 0);
             if (a < m && c < B) slot[(int64_t)a * B + c] += v;
         }
     }
 }
 
 template <int B>
-__global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int rc, int nchunks, int parts,
+__global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int rc, int nchunks, int per_group,
+                                                          int ngroups, int parts,
                                                           const double* __restrict__ Q, const double* __restrict__ W,
                                                           double* __restrict__ partial, int* __restrict__ tickets) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
@@ -475,8 +481,12 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
         __syncthreads();
         const int chunk = s_chunk;
         if (chunk >= nchunks) break;
-        const int64_t r0 = (int64_t)chunk * rc;
-        gram_chunk<B>(n, m, parts, r0, (int)min((int64_t)rc, n - r0), c0, Q, W, slot, tc_smem, ew, sums);
+        // chunk = a range of rc rows and a group of per_group tiles
+        const int range = ngroups > 1 ? chunk / ngroups : chunk;
+        const int t0 = (chunk - range * ngroups) * per_group;
+        const int64_t r0 = (int64_t)range * rc;
+        gram_chunk<B>(n, m, t0, min(per_group, (m + 15) / 16 - t0), parts, r0, (int)min((int64_t)rc, n - r0), c0, Q, W,
+                      slot, tc_smem, ew, sums);
     }
 }
 
@@ -503,7 +513,7 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_seg_kernel(int64_t n, const i
     for (int e = threadIdx.x; e < m * B; e += kT) slot[e] = 0.0;
     if (threadIdx.x < 8) ew[threadIdx.x] = 0;
     __syncthreads();
-    gram_chunk<B>(n, m, gram_parts((m + 15) / 16), r0, rows, 0, Q, W, slot, tc_smem, ew, sums);
+    gram_chunk<B>(n, m, 0, (m + 15) / 16, gram_parts((m + 15) / 16), r0, rows, 0, Q, W, slot, tc_smem, ew, sums);
 }
 
 // -------------------------------------------------------------------- W (-)= Q C
@@ -511,10 +521,11 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_seg_kernel(int64_t n, const i
 // and W.  A warp takes 16 rows; the digits of up to kMaxCols rows of C are
 // staged as B fragments (in one go, kept over the CTA's row groups, when they
 // are all of C).
-// One group of rows from row0 on (16 per row tile, kWarps / ks tiles, below
-// row_end); staged: C's digits are in smem from an earlier group.  All threads.
+// One group of rows from row0 on (16 per row tile, `tiles` of them by ks warps
+// each, below row_end); staged: C's digits are in smem from an earlier group.  All threads.
 template <int B, bool SUB>
-__device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, int c0, int64_t row0, int64_t row_end,
+__device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, int tiles, int c0, int64_t row0,
+                                             int64_t row_end,
                                              bool& staged, const double* Q, const double* __restrict__ C, double* W,
                                              unsigned char* smem, int* ew, double (*part)[4][32]) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -523,7 +534,8 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
     const int g = lane >> 2, t = lane & 3;
     const bool col = c0 + g < kc;
     const int sub = warp % ks;  // ks warps share a tile of 16 rows, each a share of the steps
-    const int64_t ra = row0 + (warp / ks) * 16 + g, rb = ra + 8;
+    // (a warp without a tile works on rows past the end)
+    const int64_t ra = warp / ks < tiles ? row0 + (warp / ks) * 16 + g : row_end, rb = ra + 8;
     double out[4] = {0.0, 0.0, 0.0, 0.0};
     for (int k0 = 0; k0 < m; k0 += kMaxCols) {
         const int cols = min(kMaxCols, m - k0), steps = (cols + 15) / 16;
@@ -558,7 +570,7 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
         // registers 0, 1: columns 2t, 2t+1 of rows g, g+8; 2, 3: columns 2t+8,
         // 2t+9.  A lane copies its own 16-byte pairs into its ring and reads them back.
         const int per = (steps + ks - 1) / ks, s0 = sub * per, s1 = min(steps, s0 + per);
-        const bool rows_in = row0 + (warp / ks) * 16 + 16 <= row_end;
+        const bool rows_in = row0 + (warp / ks) * 16 + 16 <= row_end && warp / ks < tiles;
         auto issue = [&](int s) {
             if (s < s1) {
                 const bool full = rows_in && k0 + 16 * s + 16 <= m;
@@ -624,15 +636,15 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
 }
 
 template <int B, bool SUB>
-__global__ void __launch_bounds__(kT, 2) update_tc64_kernel(int64_t n, int m, int kc, int ks, const double* Q,
+__global__ void __launch_bounds__(kT, 2) update_tc64_kernel(int64_t n, int m, int kc, int ks, int tiles, const double* Q,
                                                             const double* __restrict__ C, double* W) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
     __shared__ int ew[8];
     __shared__ double part[kWarps][4][32];
-    const int rows = 16 * (kWarps / ks);
+    const int rows = 16 * tiles;
     bool staged = false;
     for (int64_t row0 = (int64_t)blockIdx.x * rows; row0 < n; row0 += (int64_t)gridDim.x * rows)
-        update_group<B, SUB>(n, m, kc, ks, blockIdx.y * 8, row0, n, staged, Q, C, W, tc_smem, ew, part);
+        update_group<B, SUB>(n, m, kc, ks, tiles, blockIdx.y * 8, row0, n, staged, Q, C, W, tc_smem, ew, part);
 }
 
 // Segmented: CTA x updates rows [ctas[3x+1], ctas[3x+2]) of segment s = ctas[3x]
@@ -653,7 +665,7 @@ __global__ void __launch_bounds__(kT, 2) update_tc64_seg_kernel(int64_t n, const
     const int64_t r1 = ctas[3 * blockIdx.x + 2];
     bool staged = false;
     for (int64_t row0 = ctas[3 * blockIdx.x + 1]; row0 < r1; row0 += 16 * kWarps)
-        update_group<B, true>(n, m, B, 1, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew, part);
+        update_group<B, true>(n, m, B, 1, kWarps, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew, part);
 }
 
 int sms() {
@@ -678,21 +690,26 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
         attr = true;
     }
     constexpr int NH = (B + 7) / 8;
-    // rows per chunk: one chunk per resident CTA where that gives at least 64 rows
-    // (n = 2e4: 80 rows, 250 chunks; with 64 rows a second wave held 9 of 313
-    // chunks), at most the staged 512
+    // One chunk per resident CTA where that gives at least 64 rows, at most the
+    // staged 512; with fewer than 512 rows the tiles are split into groups of
+    // one per warp, which take more rows each (an item's end, its FP64
+    // conversions, costs as much as three steps).  n = 2e4, b = 4, m = 400: 36.7 us
+    // in one group, 33.4 in four; m = 200: 21.2 and 21.0.
     const int64_t resident = (int64_t)2 * gram_worker_sms();
-    int64_t rc = ceil_div(ceil_div(n, resident), 16) * 16;
-    rc = std::min<int64_t>(std::max<int64_t>(rc, 64), kMaxRows);
-    const int parts = gram_parts((m + 15) / 16);
-    const int64_t chunks = ceil_div(n, rc);
+    const int ntiles = (m + 15) / 16;
+    int64_t groups = (ntiles + kWarps - 1) / kWarps;
+    groups = std::max<int64_t>(std::min<int64_t>(groups, kMaxRows * resident / std::max<int64_t>(n, 1)), 1);
+    const int per_group = (int)ceil_div(ntiles, groups);
+    groups = ceil_div(ntiles, per_group);
+    const int64_t rc = std::min<int64_t>(std::max<int64_t>(ceil_div(ceil_div(n * groups, resident), 16) * 16, 64), kMaxRows);
+    const int64_t chunks = ceil_div(n, rc) * groups;
     const int64_t ctas = std::min<int64_t>(chunks, resident);
     const int64_t per = (int64_t)m * B;
     BBL_TRY(partials.grow(sizeof(double) * (size_t)(ctas * per) + 256));
     int* tickets = reinterpret_cast<int*>(partials.as<double>() + ctas * per);
     BBL_CUDA(cudaMemsetAsync(tickets, 0, sizeof(int) * NH, st));
     gram_tc64_kernel<B><<<dim3((unsigned)ctas, NH), kT, kRingBytes + (size_t)(rc / 16) * kFragBytes, st>>>(
-        n, m, (int)rc, (int)chunks, parts, Q, W, partials.as<double>(), tickets);
+        n, m, (int)rc, (int)chunks, per_group, (int)groups, gram_parts(per_group), Q, W, partials.as<double>(), tickets);
     BBL_LAUNCH_CHECK();
     reduce_partials(per, (int)ctas, partials.as<double>(), C, st);
     BBL_LAUNCH_CHECK();
@@ -707,15 +724,22 @@ bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double
                                       kRingBytes + kMaxCols / 16 * kFragBytes));
         attr = true;
     }
-    // few rows: up to eight warps share a row tile's steps, so that the SMs' 16
-    // warps have work
     const int64_t rtiles = ceil_div(n, 16);
     const int cols = std::min(m, kMaxCols), steps = (cols + 15) / 16;
+    const int64_t ny = (kc + 7) / 8;
+    // few rows: up to eight warps share a row tile's steps, so that the SMs' 16
+    // warps have work
     int ks = 1;
     while (ks < kWarps && rtiles * ks * 2 <= (int64_t)sms() * 2 * kWarps && steps >= ks * 4) ks <<= 1;
-    const int64_t groups = ceil_div(rtiles, kWarps / ks);
+    int tiles = kWarps / ks;
+    // between one and two CTAs per SM: fewer tiles each, so that every SM has two
+    // (n = 2e4, m = 200: 5 tiles, 250 CTAs, 26.2 us; with 8 five of the 152 SMs had
+    // two CTAs, 27.1 us)
+    const int64_t total = ceil_div(rtiles, tiles) * ny;
+    if (ks == 1 && total > sms() && total < (int64_t)2 * sms()) tiles = (int)ceil_div(rtiles * ny, (int64_t)2 * sms());
+    const int64_t groups = ceil_div(rtiles, tiles);
     const dim3 grid((unsigned)std::min<int64_t>(groups, (int64_t)sms() * 8), (unsigned)((kc + 7) / 8));
-    update_tc64_kernel<B, SUB><<<grid, kT, kRingBytes + (size_t)steps * kFragBytes, st>>>(n, m, kc, ks, Q, C, W);
+    update_tc64_kernel<B, SUB><<<grid, kT, kRingBytes + (size_t)steps * kFragBytes, st>>>(n, m, kc, ks, tiles, Q, C, W);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
