@@ -184,6 +184,10 @@ uint64_t bbl_kernel_launches(void);
  * instead of being freed (an allocation plus free of 16 GB costs about 10 ms);
  * a later request reuses an idle buffer of at least its size and at most
  * 1/16 more (repeated solves of one size reuse theirs exactly).
+ * The scratch of the single calls (bbl_block_gram, bbl_block_reorth,
+ * bbl_cholqr2, bbl_ritz_banded, the pivot checks, the FP16 first pass) is kept
+ * the same way, rounded up to a power of two: buffers of at most 64 MiB, at
+ * most 16 of them and 256 MiB per device.
  * Reuse is ordered by an event on the stream that last used the memory, so
  * calls on different streams may share the cache.  A call whose allocation
  * fails frees the idle buffers and tries once more before reporting
@@ -323,7 +327,7 @@ bbl_status bbl_block_gram_f16(int64_t n, int nblocks, const void* basis16, const
  * (in Lanczos these carry the large coefficients A_j and B_{j-1}).  The
  * update sums over the basis in FP32; the Gram sums a CTA's rows in FP32 and
  * the CTAs in FP64.  basis and W 16-byte aligned (BBL_ERR_INVALID_ARG
- * otherwise).  The call allocates its workspace and synchronises `stream`. */
+ * otherwise).  The call takes its workspace from the cache and synchronises `stream`. */
 bbl_status bbl_block_update_gram(int64_t n, int nblocks, const float* basis, const double* C1, float* W, double* C2,
                                  void* stream);
 
@@ -346,7 +350,7 @@ bbl_status bbl_block_update_gram(int64_t n, int nblocks, const float* basis, con
  * Gram-Schmidt pass removes.  The newest blocks are FP32 FMA products with
  * C rounded to FP32, added to the same FP32 sum, which is then subtracted
  * from W.  basis16, basis and W 16-byte aligned (BBL_ERR_INVALID_ARG
- * otherwise).  The call allocates its workspace and synchronises `stream`. */
+ * otherwise).  The call takes its workspace from the cache and synchronises `stream`. */
 bbl_status bbl_block_update_f16old(int64_t n, int nblocks, int nnew, const void* basis16, const float* basis,
                                    const double* C, float* W, void* stream);
 

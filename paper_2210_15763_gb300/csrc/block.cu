@@ -2056,7 +2056,7 @@ bbl_status bbl_block_reorth(int64_t n, int b, int nblocks, bbl_dtype dtype, cons
     if (dtype != BBL_FP64 && dtype != BBL_FP32) return set_error(BBL_ERR_INVALID_ARG, "block_reorth: bad dtype");
     if (!aligned16(basis) || !aligned16(W)) return set_error(BBL_ERR_INVALID_ARG, "block_reorth: pointers must be 16-byte aligned");
     cudaStream_t st = as_stream(stream);
-    DevBuf partials, cbuf;
+    DevBuf partials(st), cbuf(st);
     const int m = nblocks * b;
     double* C = coeff;
     if (!C) {
@@ -2080,7 +2080,7 @@ bbl_status bbl_cholqr2(int64_t n, int b, bbl_dtype dtype, void* W, double* B, do
     if (!aligned16(W)) return set_error(BBL_ERR_INVALID_ARG, "cholqr2: W must be 16-byte aligned");
     if (defl_abs < 0) return set_error(BBL_ERR_INVALID_ARG, "cholqr2: defl_abs < 0");
     cudaStream_t st = as_stream(stream);
-    DevBuf partials, small, cnt;
+    DevBuf partials(st), small(st), cnt(st);
     BBL_TRY(cnt.alloc(sizeof(int)));
     BBL_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int), st));
     BBL_TRY(small.alloc(sizeof(double) * 8 * kMaxB * kMaxB + sizeof(int) * 4 * kMaxB));
@@ -2246,7 +2246,7 @@ extern "C" bbl_status bbl_pivot_overlap(int64_t n, int b, const double* P, int k
     if (n < 1 || b < 1 || b > kMaxB || k < 1 || k > kMaxB || !P || !X || !overlap)
         return set_error(BBL_ERR_INVALID_ARG, "pivot_overlap: bad arguments (b, k in 1..%d)", kMaxB);
     cudaStream_t st = as_stream(stream);
-    DevBuf Q, Xd, partials, small, cnt, part, C;
+    DevBuf Q(st), Xd(st), partials(st), small(st), cnt(st), part(st), C(st);
     BBL_TRY(Q.alloc(sizeof(double) * n * b));
     BBL_CUDA(cudaMemcpyAsync(Q.p, P, sizeof(double) * n * b, cudaMemcpyDefault, st));
     const double* Xp = X;
@@ -2261,7 +2261,7 @@ extern "C" bbl_status bbl_pivot_overlap(int64_t n, int b, const double* P, int k
     BBL_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int), st));
     BBL_TRY(small.alloc(sizeof(double) * 8 * kMaxB * kMaxB + sizeof(int) * 4 * kMaxB));
     BBL_CUDA(cudaMemsetAsync(small.p, 0, small.bytes, st));
-    DevBuf Bm;
+    DevBuf Bm(st);
     BBL_TRY(Bm.alloc(sizeof(double) * kMaxB * kMaxB));
     BBL_TRY(cholqr2_dev(n, b, BBL_FP64, Q.p, Bm.as<double>(), -1e-20, cnt.as<int>(), nullptr, partials, small, st));
     const int grid = (int)std::min<int64_t>(152 * 4, ceil_div(n, kOvRows));

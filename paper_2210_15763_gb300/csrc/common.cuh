@@ -68,18 +68,33 @@ bool is_device_pointer(const void* p);
 bool pool_free_idle_current_device();
 
 // ------------------------------------------------------------------ device buffers
-// Owning device allocation; frees on destruction.
+struct DevBuf;
+bool kept_alloc(DevBuf& b, size_t nbytes, bbl_status* status);
+void kept_release(DevBuf& b);
+
+// Owning device allocation; frees on destruction.  Constructed with a
+// stream, its allocations of up to kKeptBuf bytes come from, and go back to, a
+// per-device list of idle scratch buffers: for a call whose kernels all run on
+// that stream.  Reuse is ordered by an event on it, as for PoolBuf.
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
+    bool kept = false;           // constructed with a stream
+    bool listed = false;         // p goes back to the list
+    int dev = 0;
+    cudaStream_t st = nullptr;
+    cudaEvent_t ready = nullptr;
     DevBuf() = default;
+    explicit DevBuf(cudaStream_t stream) : kept(true), st(stream) {}
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
     ~DevBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (listed) kept_release(*this);
+        else if (p) cudaFree(p);
         p = nullptr;
         bytes = 0;
+        listed = false;
     }
     // workspace growth: at least doubles, so that a buffer sized by a
     // growing basis is reallocated (cudaFree synchronises the device) a
@@ -91,6 +106,10 @@ struct DevBuf {
     bbl_status alloc(size_t nbytes) {
         release();
         if (nbytes == 0) nbytes = 16;
+        if (kept) {
+            bbl_status s = BBL_OK;
+            if (kept_alloc(*this, nbytes, &s)) return s;
+        }
         cudaError_t e = cudaMalloc(&p, nbytes);
         if (e == cudaErrorMemoryAllocation && pool_free_idle_current_device()) {  // cached bases back, once more
             (void)cudaGetLastError();

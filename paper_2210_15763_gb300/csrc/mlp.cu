@@ -576,7 +576,7 @@ bbl_status bbl_pivot_learned(bbl_mlp* M, float g, int64_t n, int b_U, int nblock
         return set_error(BBL_ERR_INVALID_ARG, "pivot_learned: shapes do not match the network output");
     cudaStream_t st = as_stream(stream);
     BBL_TRY(ensure_batch(M, 1));
-    DevBuf gb, y, C;
+    DevBuf gb(st), y(st), C(st);
     BBL_TRY(gb.alloc(sizeof(float)));
     BBL_TRY(y.alloc(sizeof(float) * M->out));
     BBL_TRY(C.alloc(sizeof(double) * M->out));

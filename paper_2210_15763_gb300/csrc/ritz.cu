@@ -1409,7 +1409,7 @@ extern "C" bbl_status bbl_ritz_banded(int m, int p, int nev, const double* Tband
         return set_error(BBL_ERR_INVALID_ARG, "ritz_banded: bad arguments (m=%d p=%d nev=%d)", m, p, nev);
     if (m > 16384) return set_error(BBL_ERR_UNSUPPORTED, "ritz_banded: m=%d above 16384", m);
     cudaStream_t st = as_stream(stream);
-    DevBuf work;
+    DevBuf work(st);
     BBL_TRY(ritz_dev(m, p, nev, Tband, theta, S, work, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;

@@ -1047,7 +1047,7 @@ extern "C" bbl_status bbl_pivot_rr_residual(const bbl_matrix* A, int b, const do
         return set_error(BBL_ERR_INVALID_ARG, "pivot_rr_residual: bad arguments");
     cudaStream_t st = as_stream(stream);
     const int64_t n = A->n;
-    DevBuf Q, W, G, Tb, th, S, X, Y, partials, small, rwork, scratch;
+    DevBuf Q(st), W(st), G(st), Tb(st), th(st), S(st), X(st), Y(st), partials(st), small(st), rwork(st), scratch(st);
     BBL_TRY(Q.alloc(sizeof(double) * n * b));
     BBL_TRY(W.alloc(sizeof(double) * n * b));
     BBL_TRY(X.alloc(sizeof(double) * n * b));
@@ -1093,7 +1093,7 @@ extern "C" bbl_status bbl_block_gram_f16(int64_t n, int nblocks, const void* bas
     if (!aligned16(basis16) || !aligned16(W))
         return set_error(BBL_ERR_INVALID_ARG, "block_gram_f16: pointers must be 16-byte aligned");
     cudaStream_t st = as_stream(stream);
-    DevBuf partials;
+    DevBuf partials(st);
     BBL_TRY(gram_half(n, nblocks, basis16, W, C, partials, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;
@@ -1111,7 +1111,7 @@ extern "C" bbl_status bbl_block_update_gram(int64_t n, int nblocks, const float*
     if (!update_gram_tc_supports(nblocks))
         return set_error(BBL_ERR_UNSUPPORTED, "block_update_gram: %d blocks (at most 128)", nblocks);
     cudaStream_t st = as_stream(stream);
-    DevBuf work;
+    DevBuf work(st);
     BBL_TRY(update_gram_tc(n, nblocks, basis, C1, W, C2, work, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;
@@ -1127,7 +1127,7 @@ extern "C" bbl_status bbl_block_update_f16old(int64_t n, int nblocks, int nnew, 
     if (!aligned16(basis16) || !aligned16(basis) || !aligned16(W))
         return set_error(BBL_ERR_INVALID_ARG, "block_update_f16old: pointers must be 16-byte aligned");
     cudaStream_t st = as_stream(stream);
-    DevBuf work;
+    DevBuf work(st);
     BBL_TRY(update_half_old(n, nblocks, nnew, basis16, basis, C, W, work, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;
@@ -1142,7 +1142,7 @@ extern "C" bbl_status bbl_block_gram(int64_t n, int b, int nblocks, bbl_dtype dt
     if (dtype != BBL_FP64 && dtype != BBL_FP32) return set_error(BBL_ERR_INVALID_ARG, "block_gram: bad dtype");
     if (!aligned16(basis) || !aligned16(W)) return set_error(BBL_ERR_INVALID_ARG, "block_gram: pointers must be 16-byte aligned");
     cudaStream_t st = as_stream(stream);
-    DevBuf partials;
+    DevBuf partials(st);
     BBL_TRY(gram(n, b, nblocks, dtype, basis, W, C, partials, st));
     BBL_CUDA(cudaStreamSynchronize(st));
     return BBL_OK;
