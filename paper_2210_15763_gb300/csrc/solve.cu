@@ -61,9 +61,15 @@ __global__ void df32_hi_kernel(int64_t count, const df32* __restrict__ in, float
         out[e] = in[e].hi;
 }
 
-// B_j (upper triangular) into block (j+1, j) of T
-__global__ void fill_B_kernel(int j, int b, int rows_alloc, const double* __restrict__ Bj, double* __restrict__ Tb) {
+// B_j (upper triangular) into block (j+1, j) of T, and the count of deflated
+// columns to page-locked host memory: a copy by the copy engine of these four
+// bytes held the stream up for 10 to 20 us per block (the engine's start, and
+// the next kernel's wait for it; n = 2e4, FP64, 111 blocks: 25.4 -> 24.0 ms per
+// solve with the Ritz reports below).
+__global__ void fill_B_kernel(int j, int b, int rows_alloc, const double* __restrict__ Bj, double* __restrict__ Tb,
+                              const int* __restrict__ ndefl, int* __restrict__ h_ndefl) {
     const int e = threadIdx.x;
+    if (e == 0) *h_ndefl = *ndefl;
     if (e >= b * b) return;
     const int r = e / b, c = e % b;
     if (c < r) return;
@@ -73,8 +79,10 @@ __global__ void fill_B_kernel(int j, int b, int rows_alloc, const double* __rest
 }
 
 // est_i = || B_j S[m-b .. m-1, i] ||_2 with B_j read from rows m..m+b-1 of
-// the band (upper triangular: B_j[r][c] at d = b + r - c, c >= r)
+// the band (upper triangular: B_j[r][c] at d = b + r - c, c >= r); est and a
+// copy of theta go to page-locked host memory
 __global__ void estimate_kernel(int m, int b, int k, const double* __restrict__ Tb, const double* __restrict__ S,
+                                const double* __restrict__ theta, double* __restrict__ h_theta,
                                 double* __restrict__ est) {
     const int i = threadIdx.x;
     if (i >= k) return;
@@ -85,6 +93,7 @@ __global__ void estimate_kernel(int m, int b, int k, const double* __restrict__ 
         s2 += t * t;
     }
     est[i] = sqrt(s2);
+    h_theta[i] = theta[i];
 }
 
 // Z[:, c] -> W[:, c] for masked columns
@@ -606,10 +615,9 @@ bbl_status lanczos_stage(const bbl_matrix* A, int nev, int b, const double* pivo
     cudaEvent_t* ev_r0 = guard.e + 2;     // [2] Ritz start
     cudaEvent_t* ev_r1 = guard.e + 4;     // [2] Ritz done (report in host memory)
     cudaEvent_t ev_defl = guard.e[6];     // deflation count of the last CholQR2 in host memory
-    DevBuf theta2, S2, est2;
+    DevBuf theta2, S2;
     BBL_TRY(theta2.alloc(sizeof(double) * 2 * 64));
     BBL_TRY(S2.alloc(sizeof(double) * 2 * (size_t)m_max * nev));
-    BBL_TRY(est2.alloc(sizeof(double) * 2 * 64));
     DevBuf rwork2;
     BBL_TRY(rwork2.alloc(ritz_workspace_bytes(m_max, b, nev) + 1024));
     DevBuf* rw[2] = {&rwork, &rwork2};
@@ -630,16 +638,13 @@ bbl_status lanczos_stage(const bbl_matrix* A, int nev, int b, const double* pivo
         BBL_CUDA(cudaEventRecord(ev_r0[slot], side));
         double* th = theta2.as<double>() + 64 * slot;
         double* Sd = S2.as<double>() + (size_t)slot * m_max * nev;
-        double* es = est2.as<double>() + 64 * slot;
         // warm start from the previous Ritz solve on this stream (other slot)
         const double* warm = warm_k > 0 ? theta2.as<double>() + 64 * (slot ^ 1) : nullptr;
         BBL_TRY(ritz_dev(m, b, k, Tb.as<double>(), th, Sd, *rw[slot], side, warm, warm_k));
         warm_k = k;
         // B_jj sits in rows (jj+1)b.. of the band: the estimate reads it there
-        estimate_kernel<<<1, 64, 0, side>>>(m, b, k, Tb.as<double>(), Sd, es);
+        estimate_kernel<<<1, 64, 0, side>>>(m, b, k, Tb.as<double>(), Sd, th, h_theta + 32 * slot, h_est + 32 * slot);
         BBL_LAUNCH_CHECK();
-        BBL_CUDA(cudaMemcpyAsync(h_theta + 32 * slot, th, sizeof(double) * k, cudaMemcpyDeviceToHost, side));
-        BBL_CUDA(cudaMemcpyAsync(h_est + 32 * slot, es, sizeof(double) * k, cudaMemcpyDeviceToHost, side));
         BBL_CUDA(cudaEventRecord(ev_r1[slot], side));
         return BBL_OK;
     };
@@ -786,11 +791,10 @@ bbl_status lanczos_stage(const bbl_matrix* A, int nev, int b, const double* pivo
         BBL_LAUNCH_CHECK();
         BBL_CUDA(cudaEventRecord(tm.ev[2], st));
         BBL_TRY(cholqr2_dev(n, b, dtype, Wn, bj.as<double>(), thresh2, d_ndefl, d_mask, partials, small, st));
-        fill_B_kernel<<<1, 256, 0, st>>>(j, b, t_rows, bj.as<double>(), Tb.as<double>());
+        fill_B_kernel<<<1, 256, 0, st>>>(j, b, t_rows, bj.as<double>(), Tb.as<double>(), d_ndefl, h_ndefl);
         BBL_LAUNCH_CHECK();
         BBL_CUDA(cudaEventRecord(tm.ev[3], st));
         BBL_CUDA(cudaEventRecord(ev_main[tb & 1], st));
-        BBL_CUDA(cudaMemcpyAsync(h_ndefl, d_ndefl, sizeof(int), cudaMemcpyDeviceToHost, st));
         BBL_CUDA(cudaEventRecord(ev_defl, st));
         out.gram_bytes += half1 ? (double)n * (j + 1) * b * 2.0 + (double)n * b * 4.0
                                 : ((double)n * (j + 1) * b + (double)n * b) * (double)s;

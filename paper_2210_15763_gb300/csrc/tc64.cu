@@ -476,10 +476,10 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
         if (e % B >= c0 && e % B < c0 + 8) slot[e] = 0.0;
     for (;;) {
         __syncthreads();
-        if (tid == 0) s_chunk = atomicAdd(tickets + blockIdx.y, 1);
+        if (tid == 0 && tickets) s_chunk = atomicAdd(tickets + blockIdx.y, 1);
         if (tid < 8) ew[tid] = 0;
         __syncthreads();
-        const int chunk = s_chunk;
+        const int chunk = tickets ? s_chunk : blockIdx.x;  // no tickets: one chunk per CTA
         if (chunk >= nchunks) break;
         // chunk = a range of rc rows and a group of per_group tiles
         const int range = ngroups > 1 ? chunk / ngroups : chunk;
@@ -487,6 +487,7 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
         const int64_t r0 = (int64_t)range * rc;
         gram_chunk<B>(n, m, t0, min(per_group, (m + 15) / 16 - t0), parts, r0, (int)min((int64_t)rc, n - r0), c0, Q, W,
                       slot, tc_smem, ew, sums);
+        if (!tickets) break;
     }
 }
 
@@ -706,8 +707,11 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
     const int64_t ctas = std::min<int64_t>(chunks, resident);
     const int64_t per = (int64_t)m * B;
     BBL_TRY(partials.grow(sizeof(double) * (size_t)(ctas * per) + 256));
-    int* tickets = reinterpret_cast<int*>(partials.as<double>() + ctas * per);
-    BBL_CUDA(cudaMemsetAsync(tickets, 0, sizeof(int) * NH, st));
+    int* tickets = nullptr;
+    if (chunks > ctas) {
+        tickets = reinterpret_cast<int*>(partials.as<double>() + ctas * per);
+        BBL_CUDA(cudaMemsetAsync(tickets, 0, sizeof(int) * NH, st));
+    }
     gram_tc64_kernel<B><<<dim3((unsigned)ctas, NH), kT, kRingBytes + (size_t)(rc / 16) * kFragBytes, st>>>(
         n, m, (int)rc, (int)chunks, per_group, (int)groups, gram_parts(per_group), Q, W, partials.as<double>(), tickets);
     BBL_LAUNCH_CHECK();
