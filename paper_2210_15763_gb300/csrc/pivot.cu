@@ -4,8 +4,8 @@
 // a truncated model space and projected into the full space.  For matrices
 // without a physics basis the truncated space is the set S of the trunc_dim
 // rows with the smallest diagonal entries (ties: lower index first):
-//   1. threshold search on the order-preserving 64-bit key of H_ii
-//      (bisection over the key range, one counting pass per bit);
+//   1. the k-th smallest of the order-preserving 64-bit keys of H_ii (radix
+//      selection: one histogram pass per 8 bits);
 //   2. stable compaction of S and of the position map pos[i] (device);
 //   3. extraction of the principal submatrix H[S,S] as CSR (device);
 //   4. its lowest b eigenpairs by this library's own block Lanczos (FP64);
@@ -23,14 +23,62 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-__global__ void count_below_kernel(int64_t n, const double* __restrict__ d, unsigned long long t,
-                                   unsigned long long* __restrict__ cnt) {
-    unsigned long long c = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += (order_key(d[i]) < t);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(cnt, c);
+// Radix selection of the k-th smallest key: the pass over bits shift ..
+// shift + 7 counts the keys that agree with the prefix found so far by these
+// bits; the last CTA to finish takes the digit that holds the k-th and clears
+// the counters for the next pass.  (A bisection by counting passes read its
+// count on the host 65 times, about 25 us each.  A mixed-precision solve with its
+// pivot at n = 5e5: 131.1 -> 125.9 ms with the reports that the solver's kernels
+// write to host memory.)
+struct KthState {
+    unsigned long long prefix;   // the bits found
+    unsigned long long rank;     // of the k-th among the keys that agree with them, from 1
+    unsigned done;               // CTAs finished in this pass
+    unsigned long long count[256];
+};
+
+__global__ void __launch_bounds__(256) kth_pass_kernel(int64_t n, const double* __restrict__ d, int shift,
+                                                       KthState* __restrict__ st) {
+    __shared__ unsigned long long hist[256];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    hist[tid] = 0;
+    __syncthreads();
+    const unsigned long long prefix = st->prefix;
+    const unsigned long long high = shift < 56 ? ~0ull << (shift + 8) : 0ull;
+    // equal digits in a row (the high ones nearly always) are added at once
+    int bin = 0;
+    unsigned long long run = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + tid; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned long long k = order_key(d[i]);
+        if ((k ^ prefix) & high) continue;
+        const int q = (int)(k >> shift) & 255;
+        if (q != bin) {
+            if (run) atomicAdd(&hist[bin], run);
+            bin = q;
+            run = 0;
+        }
+        ++run;
+    }
+    if (run) atomicAdd(&hist[bin], run);
+    __syncthreads();
+    if (hist[tid]) atomicAdd(&st->count[tid], hist[tid]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    hist[tid] = atomicExch(&st->count[tid], 0ull);
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long r = st->rank;
+        int q = 0;
+        while (q < 255 && r > hist[q]) r -= hist[q++];
+        st->prefix = prefix | (unsigned long long)q << shift;
+        st->rank = r;
+        st->done = 0;
+    }
 }
 
 // flags: 1 if key < t, or key == t and among the first `need_eq` equal keys
@@ -193,30 +241,22 @@ extern "C" bbl_status bbl_pivot_bootstrap(const bbl_matrix* A, int64_t trunc_dim
     const int64_t n = A->n;
     const int64_t k = std::min(trunc_dim, n);
     const unsigned grid = 152 * 8;
-    // 1. threshold: smallest key t with count(key < t) >= k  ->  kth key = t - 1
-    DevBuf cnt;
-    BBL_TRY(cnt.alloc(sizeof(unsigned long long)));
-    auto count_below = [&](unsigned long long t, unsigned long long* out) -> bbl_status {
-        BBL_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), st));
-        count_below_kernel<<<grid, 256, 0, st>>>(n, A->diag.as<double>(), t, cnt.as<unsigned long long>());
+    // 1. the k-th smallest key: count(key < kth) < k <= count(key <= kth)
+    DevBuf sel_state;
+    BBL_TRY(sel_state.alloc(sizeof(KthState)));
+    KthState* kst = sel_state.as<KthState>();
+    unsigned long long found[2] = {0, (unsigned long long)k};  // prefix, rank
+    BBL_CUDA(cudaMemsetAsync(sel_state.p, 0, sizeof(KthState), st));
+    BBL_CUDA(cudaMemcpyAsync(kst, found, sizeof(found), cudaMemcpyHostToDevice, st));
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        kth_pass_kernel<<<grid, 256, 0, st>>>(n, A->diag.as<double>(), shift, kst);
         BBL_LAUNCH_CHECK();
-        BBL_CUDA(cudaMemcpyAsync(out, cnt.p, sizeof(*out), cudaMemcpyDeviceToHost, st));
-        BBL_CUDA(cudaStreamSynchronize(st));
-        return BBL_OK;
-    };
-    // binary search for the k-th smallest key value kth: count(key < kth) < k <= count(key <= kth)
-    unsigned long long lo = 0, hi = ~0ull;  // invariant: count(< lo) < k, count(< hi) >= k (or hi = max)
-    while (hi - lo > 1) {
-        const unsigned long long mid = lo + (hi - lo) / 2;
-        unsigned long long c = 0;
-        BBL_TRY(count_below(mid, &c));
-        if (c >= (unsigned long long)k) hi = mid;
-        else lo = mid;
     }
-    const unsigned long long kth = lo;  // count(< kth) < k and count(< kth + 1) >= k
-    unsigned long long nless = 0;
-    BBL_TRY(count_below(kth, &nless));
-    const int64_t need_eq = k - (int64_t)nless;
+    BBL_CUDA(cudaMemcpyAsync(found, kst, sizeof(found), cudaMemcpyDeviceToHost, st));
+    BBL_CUDA(cudaStreamSynchronize(st));
+    const unsigned long long kth = found[0];
+    if (kth == ~0ull) return set_error(BBL_ERR_NUMERICAL, "pivot_bootstrap: fewer than %lld usable diagonal entries", (long long)k);
+    const int64_t need_eq = (int64_t)found[1];  // of the keys equal to kth, the first need_eq belong to S
     // 2. flags, ranks, compaction
     DevBuf flt, feq, req, sel, spos, Sidx, pos;
     BBL_TRY(flt.alloc(sizeof(int) * n));
