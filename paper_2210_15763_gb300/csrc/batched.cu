@@ -31,9 +31,9 @@ bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, cons
 bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int dtype, const void* Q, const double* C,
                      int64_t cstride, void* W, bool sub, bool f64_out, const int64_t* ctas, int nctas, const int* active,
                      cudaStream_t st);
-bbl_status chol_seg(int b, int nseg, const double* G, const double* thresh2, int relative, double* R, double* Rinv,
-                    int* ndefl, int* mask, int* status, const int* active, cudaStream_t st);
-bbl_status trmul_seg(int b, int nseg, const double* R2, const double* R1, double* B, const int* active, cudaStream_t st);
+bbl_status chol_seg(int b, int dtype, int nseg, const double* partial, const int* seg_chunk_ptr, const double* thresh2,
+                    int relative, double* R, double* Rinv, int* ndefl, int* mask, int* status, const int* active,
+                    cudaStream_t st);
 size_t ritz_batch_workspace_bytes(int m_max, int p, int nev, int nseg);
 int gram_seg_chunk_rows(int b, int dtype);
 bbl_status ritz_dev_batched(int m_max, int p, int nev, int nseg, const double* Tb, int64_t sT, double* theta,
@@ -106,40 +106,40 @@ __global__ void copy_slot_kernel(int64_t count, const int* __restrict__ d_j, int
     }
 }
 
-// A_j = sym(C1[s][j-block]) and B_j into segment s's band (rows_alloc rows, b+1 columns)
-__global__ void fill_AB_seg_kernel(int b, int m_max, int rows_alloc, const int* __restrict__ d_j,
-                                   const int* __restrict__ active, const double* __restrict__ C1,
-                                   const double* __restrict__ Bj, double* __restrict__ Tb, int which) {
+// Per active segment: A_j = sym(C1[s][j-block]) and B_j = R2 R1 into its band
+// (rows_alloc rows, b+1 columns).  For all segments: which test convergence at
+// block j: with every > 0 each every-th block, else (adaptive) from block
+// next_chk[s] on; always on a breakdown and at the last block.  (One kernel: the
+// four small ones took 2 us each in every block.)
+__global__ void __launch_bounds__(256) fill_AB_seg_kernel(int b, int m_max, int rows_alloc, int J_max, int every,
+                                                          const int* __restrict__ d_j, const int* __restrict__ active,
+                                                          const double* __restrict__ C1, const double* __restrict__ R1,
+                                                          const double* __restrict__ R2, double* __restrict__ Tb,
+                                                          const int* __restrict__ ndefl,
+                                                          const int* __restrict__ next_chk, int* __restrict__ due) {
     const int s = blockIdx.x;
-    if (active && !active[s]) return;
     const int j = *d_j;
     const int e = threadIdx.x;
-    if (e >= b * b) return;
+    if (e == 0) {
+        const bool sched = every > 0 ? ((j + 1) % every == 0) : (j >= next_chk[s]);
+        due[s] = (active[s] && (sched || ndefl[s] > 0 || j + 1 >= J_max)) ? 1 : 0;
+    }
+    if (!active[s] || e >= b * b) return;
     const int r = e / b, c = e % b;
     double* T = Tb + (int64_t)s * rows_alloc * (b + 1);
-    if (which == 0) {
-        if (c > r) return;
+    if (c <= r) {
         const double* C = C1 + (int64_t)s * m_max * b;
         const int jb = j * b;
         T[(int64_t)(jb + r) * (b + 1) + (r - c)] = 0.5 * (C[(int64_t)(jb + r) * b + c] + C[(int64_t)(jb + c) * b + r]);
-    } else {
-        if (c < r) return;
-        const int row = (j + 1) * b + r;
-        if (row < rows_alloc) T[(int64_t)row * (b + 1) + (b + r - c)] = Bj[(int64_t)s * b * b + r * b + c];
     }
-}
-
-// which segments test convergence at block j: with every > 0 each every-th
-// block, else (adaptive) from block next_chk[s] on; always on a breakdown
-// and at the last block
-__global__ void due_seg_kernel(int nseg, int J_max, int every, const int* __restrict__ d_j,
-                               const int* __restrict__ active, const int* __restrict__ ndefl,
-                               const int* __restrict__ next_chk, int* __restrict__ due) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nseg) return;
-    const int j = *d_j;
-    const bool sched = every > 0 ? ((j + 1) % every == 0) : (j >= next_chk[s]);
-    due[s] = (active[s] && (sched || ndefl[s] > 0 || j + 1 >= J_max)) ? 1 : 0;
+    const int row = (j + 1) * b + r;
+    if (c >= r && row < rows_alloc) {
+        const double* U = R2 + (int64_t)s * b * b;
+        const double* V = R1 + (int64_t)s * b * b;
+        double acc = 0.0;
+        for (int l = 0; l < b; ++l) acc += U[r * b + l] * V[l * b + c];
+        T[(int64_t)row * (b + 1) + (b + r - c)] = acc;
+    }
 }
 
 // per due segment: estimates, convergence / deflation decisions, and the
@@ -383,7 +383,7 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
     const int nchunks = (int)(chunks.size() / 3), nctas = (int)(ctas.size() / 3);
     // ---- device buffers ----
     PoolBuf basis;
-    DevBuf d_chunks, d_ctas, d_chunk_ptr, Vfix, Wfix, C1, C2, G, R1, R1i, R2, R2i, Bj, partial, Tb, theta, width,
+    DevBuf d_chunks, d_ctas, d_chunk_ptr, Vfix, Wfix, C1, C2, R1, R1i, R2, R2i, partial, Tb, theta, width,
         S, est, ws, tmp, ints, thr, X, Y, rpart, piv, lprev;
     BBL_TRY(d_chunks.alloc(sizeof(int64_t) * chunks.size()));
     BBL_TRY(d_ctas.alloc(sizeof(int64_t) * ctas.size()));
@@ -394,12 +394,10 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
     BBL_TRY(C1.alloc(sizeof(double) * (size_t)nseg * m_max * b));
     BBL_TRY(C2.alloc(sizeof(double) * (size_t)nseg * m_max * b));
     const size_t bb = sizeof(double) * (size_t)nseg * b * b;
-    BBL_TRY(G.alloc(bb));
     BBL_TRY(R1.alloc(bb));
     BBL_TRY(R1i.alloc(bb));
     BBL_TRY(R2.alloc(bb));
     BBL_TRY(R2i.alloc(bb));
-    BBL_TRY(Bj.alloc(bb));
     // per chunk: up to 8 slots of m x b when m < 8b (row shares), else one
     BBL_TRY(partial.alloc(sizeof(double) * (size_t)nchunks * std::max(m_max, 8 * b) * b));
     BBL_TRY(Tb.alloc(sizeof(double) * (size_t)nseg * rows_alloc * (b + 1)));
@@ -464,21 +462,20 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
     const int64_t* CH = d_chunks.as<int64_t>();
     const int64_t* CT = d_ctas.as<int64_t>();
     const int* CP = d_chunk_ptr.as<int>();
-    auto cholqr2_seg = [&](void* Wb, bool with_B, const int* act, int* nd) -> bbl_status {
+    auto cholqr2_seg = [&](void* Wb, const int* act, int* nd) -> bbl_status {
         // m = b for the self Gram: d_b holds b
-        BBL_TRY(gram_seg(n, b, b, d_b, dtype, Wb, Wb, CH, nchunks, CP, nseg, act, partial.as<double>(), G.as<double>(),
+        BBL_TRY(gram_seg(n, b, b, d_b, dtype, Wb, Wb, CH, nchunks, CP, nseg, act, partial.as<double>(), nullptr,
                          st));
-        BBL_TRY(chol_seg(b, nseg, G.as<double>(), thr.as<double>(), 0, R1.as<double>(), R1i.as<double>(), nd, mask,
-                         nullptr, act, st));
+        BBL_TRY(chol_seg(b, dtype, nseg, partial.as<double>(), CP, thr.as<double>(), 0, R1.as<double>(),
+                         R1i.as<double>(), nd, mask, nullptr, act, st));
         BBL_TRY(apply_seg(n, b, b, d_b, 0, dtype, Wb, R1i.as<double>(), (int64_t)b * b, Wb, false, false, CT, nctas, act,
                           st));
-        BBL_TRY(gram_seg(n, b, b, d_b, dtype, Wb, Wb, CH, nchunks, CP, nseg, act, partial.as<double>(), G.as<double>(),
+        BBL_TRY(gram_seg(n, b, b, d_b, dtype, Wb, Wb, CH, nchunks, CP, nseg, act, partial.as<double>(), nullptr,
                          st));
-        BBL_TRY(chol_seg(b, nseg, G.as<double>(), thr.as<double>() + nseg, 0, R2.as<double>(), R2i.as<double>(), nullptr,
-                         nullptr, nullptr, act, st));
+        BBL_TRY(chol_seg(b, dtype, nseg, partial.as<double>(), CP, thr.as<double>() + nseg, 0, R2.as<double>(),
+                         R2i.as<double>(), nullptr, nullptr, nullptr, act, st));
         BBL_TRY(apply_seg(n, b, b, d_b, 0, dtype, Wb, R2i.as<double>(), (int64_t)b * b, Wb, false, false, CT, nctas, act,
                           st));
-        if (with_B) BBL_TRY(trmul_seg(b, nseg, R2.as<double>(), R1.as<double>(), Bj.as<double>(), act, st));
         return BBL_OK;
     };
     // orthonormalise the pivot (relative threshold), store as block 0
@@ -488,15 +485,15 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
         BBL_TRY(thr0.alloc(sizeof(double) * nseg));
         BBL_CUDA(cudaMemcpyAsync(thr0.p, th.data(), sizeof(double) * nseg, cudaMemcpyHostToDevice, st));
         BBL_TRY(gram_seg(n, b, b, d_b, dtype, Vfix.p, Vfix.p, CH, nchunks, CP, nseg, active, partial.as<double>(),
-                         G.as<double>(), st));
-        BBL_TRY(chol_seg(b, nseg, G.as<double>(), thr0.as<double>(), 1, R1.as<double>(), R1i.as<double>(), nullptr,
-                         nullptr, nullptr, active, st));
+                         nullptr, st));
+        BBL_TRY(chol_seg(b, dtype, nseg, partial.as<double>(), CP, thr0.as<double>(), 1, R1.as<double>(),
+                         R1i.as<double>(), nullptr, nullptr, nullptr, active, st));
         BBL_TRY(apply_seg(n, b, b, d_b, 0, dtype, Vfix.p, R1i.as<double>(), (int64_t)b * b, Vfix.p, false, false, CT,
                           nctas, active, st));
         BBL_TRY(gram_seg(n, b, b, d_b, dtype, Vfix.p, Vfix.p, CH, nchunks, CP, nseg, active, partial.as<double>(),
-                         G.as<double>(), st));
-        BBL_TRY(chol_seg(b, nseg, G.as<double>(), thr.as<double>() + nseg, 0, R2.as<double>(), R2i.as<double>(), nullptr,
-                         nullptr, nullptr, active, st));
+                         nullptr, st));
+        BBL_TRY(chol_seg(b, dtype, nseg, partial.as<double>(), CP, thr.as<double>() + nseg, 0, R2.as<double>(),
+                         R2i.as<double>(), nullptr, nullptr, nullptr, active, st));
         BBL_TRY(apply_seg(n, b, b, d_b, 0, dtype, Vfix.p, R2i.as<double>(), (int64_t)b * b, Vfix.p, false, false, CT,
                           nctas, active, st));
         BBL_CUDA(cudaMemcpyAsync(bp, Vfix.p, (size_t)n * b * sz, cudaMemcpyDeviceToDevice, st));
@@ -525,16 +522,14 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
                          C1.as<double>(), st));
         BBL_TRY(apply_seg(n, b, b, d_m, 0, dtype, basis.p, C1.as<double>(), (int64_t)m_max * b, Wfix.p, true, false, CT,
                           nctas, active, st));
-        fill_AB_seg_kernel<<<nseg, 256, 0, st>>>(b, m_max, rows_alloc, d_j, active, C1.as<double>(), Bj.as<double>(),
-                                                  Tb.as<double>(), 0);
-        BBL_LAUNCH_CHECK();
         BBL_TRY(gram_seg(n, b, m_max, d_m, dtype, basis.p, Wfix.p, CH, nchunks, CP, nseg, active, partial.as<double>(),
                          C2.as<double>(), st));
         BBL_TRY(apply_seg(n, b, b, d_m, 0, dtype, basis.p, C2.as<double>(), (int64_t)m_max * b, Wfix.p, true, false, CT,
                           nctas, active, st));
-        BBL_TRY(cholqr2_seg(Wfix.p, true, active, ndefl));
-        fill_AB_seg_kernel<<<nseg, 256, 0, st>>>(b, m_max, rows_alloc, d_j, active, C1.as<double>(), Bj.as<double>(),
-                                                  Tb.as<double>(), 1);
+        BBL_TRY(cholqr2_seg(Wfix.p, active, ndefl));
+        fill_AB_seg_kernel<<<nseg, 256, 0, st>>>(b, m_max, rows_alloc, J_max, std::max(0, o.check_every), d_j, active,
+                                                  C1.as<double>(), R1.as<double>(), R2.as<double>(), Tb.as<double>(),
+                                                  ndefl, next_chk, due);
         BBL_LAUNCH_CHECK();
         if (dtype == BBL_FP64)
             copy_slot_kernel<double><<<cg, 256, 0, st>>>(n * b, d_j, 1, Wfix.as<double>(), basis.as<double>(),
@@ -542,9 +537,6 @@ bbl_status batch_stage(bbl_batch* Bt, int nev, int b, const bbl_options& o, int 
         else
             copy_slot_kernel<float><<<cg, 256, 0, st>>>(n * b, d_j, 1, Wfix.as<float>(), basis.as<float>(),
                                                         Vfix.as<float>());
-        BBL_LAUNCH_CHECK();
-        due_seg_kernel<<<(unsigned)ceil_div(nseg, 256), 256, 0, st>>>(nseg, J_max, std::max(0, o.check_every), d_j,
-                                                                       active, ndefl, next_chk, due);
         BBL_LAUNCH_CHECK();
         BBL_TRY(ritz_dev_batched(m_max, b, nev, nseg, Tb.as<double>(), (int64_t)rows_alloc * (b + 1), theta.as<double>(),
                                  nev, width.as<double>(), S.as<double>(), (int64_t)m_max * nev, ws.as<double>(),

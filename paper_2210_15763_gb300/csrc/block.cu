@@ -1480,18 +1480,6 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
 // -------------------------------------------------------------------- Cholesky of the b x b Gram
 // status bits: 1 = non-finite Gram.  mask[i] = 1 for deflated columns.
 
-__global__ void trmul_seg_kernel(int b, int nseg, const double* __restrict__ R2, const double* __restrict__ R1,
-                                 double* __restrict__ B, const int* __restrict__ active) {
-    const int s = blockIdx.y;
-    const int e = threadIdx.x;
-    if (s >= nseg || e >= b * b || (active && !active[s])) return;
-    const int64_t o = (int64_t)s * b * b;
-    const int i = e / b, k = e % b;
-    double acc = 0.0;
-    for (int l = 0; l < b; ++l) acc += R2[o + i * b + l] * R1[o + l * b + k];
-    B[o + e] = acc;
-}
-
 // 1 / d of a normal finite d, to about one unit in the last place: an FP32
 // seed on the mantissa and two Newton steps (four FP64 instructions in a chain;
 // an FP64 instruction occupies its scheduler for 64 cycles here, and the
@@ -1592,6 +1580,21 @@ __device__ __forceinline__ double chol_Rinv(const CholShared& sh, int b, int e) 
     return c >= i && !sh.deflated[c] ? sh.Z[c * b + i] / sh.root[c] : 0.0;
 }
 
+// sh.G = the sum of nparts partial b x b Grams, by all kCholThreads threads
+__device__ __forceinline__ void chol_gram(int b, int nparts, const double* __restrict__ partial, double* red,
+                                          CholShared& sh) {
+    const int tid = threadIdx.x, bb = b * b;
+    const int groups = kCholThreads / bb, e = tid % bb, g = tid / bb;  // groups of bb threads add the parts
+    red[tid] = g < groups ? sum_parts(bb, nparts, partial, e, g, groups) : 0.0;
+    __syncthreads();
+    if (tid < bb) {
+        double s = red[tid];
+        for (int q = 1; q < groups; ++q) s += red[tid + q * bb];
+        sh.G[tid] = s;
+    }
+    __syncthreads();
+}
+
 // The Cholesky step of CholQR2 by one CTA: G = the sum of nparts partial b x b
 // Grams, R = chol(G) with deflation and R^{-1}, and, with Bout, B = R R1.
 __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, const double* __restrict__ partial,
@@ -1602,17 +1605,7 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, c
     __shared__ CholShared sh;
     __shared__ double red[kCholThreads];
     const int tid = threadIdx.x, bb = b * b;
-    {  // groups of bb threads add the parts
-        const int groups = kCholThreads / bb, e = tid % bb, g = tid / bb;
-        red[tid] = g < groups ? sum_parts(bb, nparts, partial, e, g, groups) : 0.0;
-        __syncthreads();
-        if (tid < bb) {
-            double s = red[tid];
-            for (int q = 1; q < groups; ++q) s += red[tid + q * bb];
-            sh.G[tid] = s;
-        }
-        __syncthreads();
-    }
+    chol_gram(b, nparts, partial, red, sh);
     if (tid < 32) {
         int cnt, bad;
         chol_core(b, thresh2, relative, sh, cnt, bad);
@@ -1635,18 +1628,24 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, c
     if (mask && tid < b) mask[tid] = sh.deflated[tid];
 }
 
-// A warp per segment: Cholesky of G + s*b*b with threshold thresh2[s].
-__global__ void __launch_bounds__(32) chol_seg_kernel(int b, const double* __restrict__ G,
-                                                      const double* __restrict__ thresh2, int relative,
-                                                      double* __restrict__ R, double* __restrict__ Rinv,
-                                                      int* __restrict__ ndefl, int* __restrict__ mask,
-                                                      int* __restrict__ status, const int* __restrict__ active) {
+// A CTA per segment: G = the sum of the segment's partial Grams (slots of b x b,
+// `per` for each of its chunks), then its Cholesky by one warp with threshold
+// thresh2[s].
+__global__ void __launch_bounds__(kCholThreads) chol_seg_kernel(int b, const double* __restrict__ partial,
+                                                                const int* __restrict__ seg_chunk_ptr, int per,
+                                                                const double* __restrict__ thresh2, int relative,
+                                                                double* __restrict__ R, double* __restrict__ Rinv,
+                                                                int* __restrict__ ndefl, int* __restrict__ mask,
+                                                                int* __restrict__ status,
+                                                                const int* __restrict__ active) {
     __shared__ CholShared sh;
-    const int s = blockIdx.x, lane = threadIdx.x, bb = b * b;
+    __shared__ double red[kCholThreads];
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid, bb = b * b;
     if (active && !active[s]) return;
     const int64_t o = (int64_t)s * bb;
-    for (int e = lane; e < bb; e += 32) sh.G[e] = G[o + e];
-    __syncwarp();
+    const int p0 = seg_chunk_ptr[s] * per, p1 = seg_chunk_ptr[s + 1] * per;
+    chol_gram(b, p1 - p0, partial + (int64_t)p0 * bb, red, sh);
+    if (tid >= 32) return;
     int cnt, bad;
     chol_core(b, thresh2 ? thresh2[s] : 0.0, relative, sh, cnt, bad);
     for (int e = lane; e < bb; e += 32) {
@@ -1849,20 +1848,33 @@ bbl_status cholqr2_dev(int64_t n, int b, int dtype, void* W, double* B, double d
 namespace {
 
 // C[s] = sum of segment s's partial slots (rows_slots: the row-contiguous
-// kernel's wpb slots per chunk, else one), in chunk order
-__global__ void reduce_seg_kernel(int m_max, int b, const int* __restrict__ d_m, const int* __restrict__ seg_chunk_ptr,
-                                  const int* __restrict__ active, const double* __restrict__ partial,
-                                  double* __restrict__ C, int rows_slots) {
+// kernel's wpb slots per chunk, else one): 32 entries per CTA, the slots split
+// over 8 groups of threads and combined in a fixed order.  (One thread per entry
+// adding all slots in turn took 11.6 us for the 40 slots of an FP64 segment of 2e4
+// rows and 4.9 us in FP32.)
+__global__ void __launch_bounds__(256) reduce_seg_kernel(int m_max, int b, const int* __restrict__ d_m,
+                                                         const int* __restrict__ seg_chunk_ptr,
+                                                         const int* __restrict__ active,
+                                                         const double* __restrict__ partial, double* __restrict__ C,
+                                                         int rows_slots) {
+    __shared__ double red[8][32];
     const int s = blockIdx.y;
     if (active && !active[s]) return;
     const int m = d_m ? *d_m : m_max;
     const int per = rows_slots ? gram_rows_wpb(m / b) : 1;
     const int64_t count = (int64_t)m * b;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= count) return;
-    double acc = 0.0;
-    for (int c = seg_chunk_ptr[s] * per; c < seg_chunk_ptr[s + 1] * per; ++c) acc += partial[(int64_t)c * count + e];
-    C[(int64_t)s * m_max * b + e] = acc;
+    const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t e = (int64_t)blockIdx.x * 32 + x;
+    if (e - x >= count) return;  // the whole CTA
+    const int p0 = seg_chunk_ptr[s] * per, p1 = seg_chunk_ptr[s + 1] * per;
+    red[g][x] = e < count ? sum_parts(count, p1 - p0, partial + (int64_t)p0 * count, e, g, 8) : 0.0;
+    __syncthreads();
+    if (g == 0 && e < count) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = red[q][x];
+        C[(int64_t)s * m_max * b + e] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
 }
 
 template <typename T, int B>
@@ -2002,7 +2014,8 @@ bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, cons
             default: return set_error(BBL_ERR_UNSUPPORTED, "batched: b=%d", b);
         }
     }
-    dim3 g((unsigned)ceil_div((int64_t)m_max * b, 256), (unsigned)nseg);
+    if (!C) return BBL_OK;  // the caller takes the partial sums
+    dim3 g((unsigned)ceil_div((int64_t)m_max * b, 32), (unsigned)nseg);
     reduce_seg_kernel<<<g, 256, 0, st>>>(m_max, b, d_m, seg_chunk_ptr, active, partial, C, rows_slots);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
@@ -2030,15 +2043,13 @@ bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int
                                                        static_cast<float*>(W), st);
 }
 
-bbl_status chol_seg(int b, int nseg, const double* G, const double* thresh2, int relative, double* R, double* Rinv,
-                    int* ndefl, int* mask, int* status, const int* active, cudaStream_t st) {
-    chol_seg_kernel<<<(unsigned)nseg, 32, 0, st>>>(b, G, thresh2, relative, R, Rinv, ndefl, mask, status, active);
-    BBL_LAUNCH_CHECK();
-    return BBL_OK;
-}
-
-bbl_status trmul_seg(int b, int nseg, const double* R2, const double* R1, double* B, const int* active, cudaStream_t st) {
-    trmul_seg_kernel<<<dim3(1, nseg), 256, 0, st>>>(b, nseg, R2, R1, B, active);
+// partial: of gram_seg with m_max = b and no C
+bbl_status chol_seg(int b, int dtype, int nseg, const double* partial, const int* seg_chunk_ptr, const double* thresh2,
+                    int relative, double* R, double* Rinv, int* ndefl, int* mask, int* status, const int* active,
+                    cudaStream_t st) {
+    const int per = gram_seg_chunk_rows(b, dtype) > 0 ? gram_rows_wpb(1) : 1;
+    chol_seg_kernel<<<(unsigned)nseg, kCholThreads, 0, st>>>(b, partial, seg_chunk_ptr, per, thresh2, relative, R, Rinv,
+                                                             ndefl, mask, status, active);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }

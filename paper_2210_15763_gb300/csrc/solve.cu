@@ -41,41 +41,33 @@ __global__ void convert_kernel(int64_t count, const TI* __restrict__ in, TO* __r
         out[e] = (TO)in[e];
 }
 
-// A_j = sym(C1[j-block] + C2[j-block]) into the lower band of T: both
-// Gram-Schmidt passes' own-block coefficients
-__global__ void fill_A2_kernel(int j, int b, const double* __restrict__ C1, const double* __restrict__ C2,
-                               double* __restrict__ Tb) {
-    const int e = threadIdx.x;
-    if (e >= b * b) return;
-    const int r = e / b, c = e % b;
-    if (c > r) return;
-    const int jb = j * b;
-    const int64_t rc = (int64_t)(jb + r) * b + c, cr = (int64_t)(jb + c) * b + r;
-    const double v = 0.5 * ((C1[rc] + C2[rc]) + (C1[cr] + C2[cr]));
-    Tb[(int64_t)(jb + r) * (b + 1) + (r - c)] = v;
-}
-
 // the high FP32 parts of float-float values
 __global__ void df32_hi_kernel(int64_t count, const df32* __restrict__ in, float* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
         out[e] = in[e].hi;
 }
 
-// B_j (upper triangular) into block (j+1, j) of T, and the count of deflated
-// columns to page-locked host memory: a copy by the copy engine of these four
-// bytes held the stream up for 10 to 20 us per block (the engine's start, and
-// the next kernel's wait for it; n = 2e4, FP64, 111 blocks: 25.4 -> 24.0 ms per
-// solve with the Ritz reports below).
-__global__ void fill_B_kernel(int j, int b, int rows_alloc, const double* __restrict__ Bj, double* __restrict__ Tb,
-                              const int* __restrict__ ndefl, int* __restrict__ h_ndefl) {
+// A_j = sym(C1[j-block] + C2[j-block]) (both Gram-Schmidt passes' own-block
+// coefficients) into the lower band of T, B_j (upper triangular) into its block
+// (j+1, j), and the count of deflated columns to page-locked host memory: a copy
+// by the copy engine of these four bytes held the stream up for 10 to 20 us per
+// block (the engine's start, and the next kernel's wait for it; n = 2e4, FP64, 111
+// blocks: 25.4 -> 24.0 ms per solve with the Ritz reports below).
+__global__ void __launch_bounds__(256) fill_AB_kernel(int j, int b, int rows_alloc, const double* __restrict__ C1,
+                                                      const double* __restrict__ C2, const double* __restrict__ Bj,
+                                                      double* __restrict__ Tb, const int* __restrict__ ndefl,
+                                                      int* __restrict__ h_ndefl) {
     const int e = threadIdx.x;
     if (e == 0) *h_ndefl = *ndefl;
     if (e >= b * b) return;
     const int r = e / b, c = e % b;
-    if (c < r) return;
+    if (c <= r) {
+        const int jb = j * b;
+        const int64_t rc = (int64_t)(jb + r) * b + c, cr = (int64_t)(jb + c) * b + r;
+        Tb[(int64_t)(jb + r) * (b + 1) + (r - c)] = 0.5 * ((C1[rc] + C2[rc]) + (C1[cr] + C2[cr]));
+    }
     const int row = (j + 1) * b + r;
-    if (row >= rows_alloc) return;
-    Tb[(int64_t)row * (b + 1) + (b + r - c)] = Bj[r * b + c];
+    if (c >= r && row < rows_alloc) Tb[(int64_t)row * (b + 1) + (b + r - c)] = Bj[r * b + c];
 }
 
 // est_i = || B_j S[m-b .. m-1, i] ||_2 with B_j read from rows m..m+b-1 of
@@ -784,14 +776,12 @@ bbl_status lanczos_stage(const bbl_matrix* A, int nev, int b, const double* pivo
             BBL_TRY(narrow_update(j + 1, C2, Wn));
         else
             BBL_TRY(update(n, b, j + 1, dtype, basis.p, C2, Wn, st));
+        BBL_CUDA(cudaEventRecord(tm.ev[2], st));
+        BBL_TRY(cholqr2_dev(n, b, dtype, Wn, bj.as<double>(), thresh2, d_ndefl, d_mask, partials, small, st));
         // A_j = sym(C1 + C2)[j-block]: the second pass's own-block coefficients
         // are the rounding (or, from a cheaper first pass, the approximation)
         // the first left in A_j
-        fill_A2_kernel<<<1, 256, 0, st>>>(j, b, C1, C2, Tb.as<double>());
-        BBL_LAUNCH_CHECK();
-        BBL_CUDA(cudaEventRecord(tm.ev[2], st));
-        BBL_TRY(cholqr2_dev(n, b, dtype, Wn, bj.as<double>(), thresh2, d_ndefl, d_mask, partials, small, st));
-        fill_B_kernel<<<1, 256, 0, st>>>(j, b, t_rows, bj.as<double>(), Tb.as<double>(), d_ndefl, h_ndefl);
+        fill_AB_kernel<<<1, 256, 0, st>>>(j, b, t_rows, C1, C2, bj.as<double>(), Tb.as<double>(), d_ndefl, h_ndefl);
         BBL_LAUNCH_CHECK();
         BBL_CUDA(cudaEventRecord(tm.ev[3], st));
         BBL_CUDA(cudaEventRecord(ev_main[tb & 1], st));
