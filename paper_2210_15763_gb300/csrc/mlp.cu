@@ -188,44 +188,63 @@ __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, in
 }
 
 // out[q][i] = sum_o W[o][i] d[q][o] for the CTA's 4 samples (d: rows of n_out in
-// shared memory): a warp takes 32 columns i and a share of the rows o; the
-// shares are added in order.  part: 32 x 4 x 32 floats.
-template <typename Put>
+// shared memory): a warp takes 32 V columns i, V per lane (4, one 8-byte load,
+// where H is a multiple of 4), and a share of the rows o; the shares are added in
+// order.  A few CTAs walk all of W, so the chain of loads per warp is what counts:
+// hidden 128, 512 outputs, 48 samples: V = 1 (8 shares) 18.1 us, V = 4 (32) 10.6.  part: 32 warps x
+// 4 x 32 V floats.
+template <int V, typename Put>
 __device__ __forceinline__ void columns_dot(const __nv_bfloat16* __restrict__ W, int H, int n_out, const float* d,
                                             float* part, Put&& put) {
+    constexpr int TW = 32 * V;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = (H + 31) / 32, shares = (kBwThreads / 32) / tiles;
+    const int tiles = (H + TW - 1) / TW, shares = (kBwThreads / 32) / tiles;
     const int tile = warp % tiles, share = warp / tiles;
-    const int i = 32 * tile + lane;
-    float acc[kBwS] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const int i = TW * tile + V * lane;
+    float acc[kBwS][V] = {};
     if (share < shares && i < H) {
 #pragma unroll 8
         for (int o = share; o < n_out; o += shares) {
-            const float w = __bfloat162float(W[(size_t)o * H + i]);
+            float w[V];
+            if constexpr (V == 4) {
+                const uint2 x = __ldg(reinterpret_cast<const uint2*>(W + (size_t)o * H + i));
+                w[0] = __uint_as_float(x.x << 16);
+                w[1] = __uint_as_float(x.x & 0xffff0000u);
+                w[2] = __uint_as_float(x.y << 16);
+                w[3] = __uint_as_float(x.y & 0xffff0000u);
+            } else {
+                w[0] = __bfloat162float(W[(size_t)o * H + i]);
+            }
 #pragma unroll
-            for (int q = 0; q < kBwS; ++q) acc[q] = fmaf(w, d[q * n_out + o], acc[q]);
+            for (int q = 0; q < kBwS; ++q)
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[q][v] = fmaf(w[v], d[q * n_out + o], acc[q][v]);
         }
     }
 #pragma unroll
-    for (int q = 0; q < kBwS; ++q) part[(warp * kBwS + q) * 32 + lane] = acc[q];
+    for (int q = 0; q < kBwS; ++q)
+#pragma unroll
+        for (int v = 0; v < V; ++v) part[(warp * kBwS + q) * TW + V * lane + v] = acc[q][v];
     __syncthreads();
     for (int e = threadIdx.x; e < kBwS * H; e += kBwThreads) {
         const int q = e / H, c = e - q * H;
         float t = 0.0f;
-        for (int k = 0; k < shares; ++k) t += part[((k * tiles + c / 32) * kBwS + q) * 32 + c % 32];
+#pragma unroll 8
+        for (int k = 0; k < shares; ++k) t += part[((k * tiles + c / TW) * kBwS + q) * TW + c % TW];
         put(q, c, t);
     }
     __syncthreads();
 }
 
 // backward through the activations of 4 samples: dz2, dz1
+template <int V>
 __global__ void __launch_bounds__(kBwThreads) backward_act_kernel(int batch, int H, int O,
                                                                   const __nv_bfloat16* __restrict__ Wb,
                                                                   float* __restrict__ act) {
     extern __shared__ float sh[];
-    float* part = sh;                                   // (32 warps) x 4 x 32
-    float* dz2 = part + (kBwThreads / 32) * kBwS * 32;  // 4 x H
-    float* dy = dz2 + kBwS * H;                         // 4 x O
+    float* part = sh;                           // (32 warps) x 4 x 32 V
+    float* dz2 = part + kBwThreads * kBwS * V;  // 4 x H
+    float* dy = dz2 + kBwS * H;                 // 4 x O
     const int s0 = blockIdx.x * kBwS, ns = min(kBwS, batch - s0);
     const size_t st = 6 * H + 2 * O;
     for (int e = threadIdx.x; e < kBwS * O; e += kBwThreads) {
@@ -233,7 +252,7 @@ __global__ void __launch_bounds__(kBwThreads) backward_act_kernel(int batch, int
         dy[e] = q < ns ? act[(s0 + q) * st + 6 * H + O + o] : 0.0f;
     }
     __syncthreads();
-    columns_dot(Wb + H + H * H, H, O, dy, part, [&](int q, int i, float t) {
+    columns_dot<V>(Wb + H + H * H, H, O, dy, part, [&](int q, int i, float t) {
         float v = 0.0f;
         if (q < ns) {
             float* a = act + (s0 + q) * st;
@@ -242,7 +261,7 @@ __global__ void __launch_bounds__(kBwThreads) backward_act_kernel(int batch, int
         }
         dz2[q * H + i] = v;
     });
-    columns_dot(Wb + H, H, H, dz2, part, [&](int q, int i, float t) {
+    columns_dot<V>(Wb + H, H, H, dz2, part, [&](int q, int i, float t) {
         if (q < ns) {
             float* a = act + (s0 + q) * st;
             a[4 * H + i] = t * gelu_grad(a[i]);
@@ -392,15 +411,19 @@ bbl_status launch_forward(const bbl_mlp* M, int batch, const float* g, float* y,
 // forward, MSE loss (into lossbuf[0]) and backward into the gradient buffer
 bbl_status launch_loss_grad(bbl_mlp* M, int batch, const float* g, const float* target, cudaStream_t st) {
     const int H = M->hidden, O = M->out;
+    const int V = H % 4 == 0 ? 4 : 1;
+    const auto backward_act = V == 4 ? backward_act_kernel<4> : backward_act_kernel<1>;
     static bool attr = false;
     if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(float) * (kBwThreads * kBwS + kBwS * (1024 + 4096))));
+        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(float) * (kBwThreads * kBwS * 4 + kBwS * (1024 + 4096))));
         attr = true;
     }
     BBL_TRY(launch_forward(M, batch, g, nullptr, target, st));
-    backward_act_kernel<<<(unsigned)ceil_div(batch, kBwS), kBwThreads,
-                          sizeof(float) * (kBwThreads * kBwS + kBwS * (H + O)), st>>>(
+    backward_act<<<(unsigned)ceil_div(batch, kBwS), kBwThreads,
+                   sizeof(float) * (kBwThreads * kBwS * V + kBwS * (H + O)), st>>>(
         batch, H, O, M->wbf.as<__nv_bfloat16>(), M->act.as<float>());
     BBL_LAUNCH_CHECK();
     backward_w_kernel<<<(unsigned)ceil_div(M->nparams, 256) + 1, 256, 0, st>>>(
