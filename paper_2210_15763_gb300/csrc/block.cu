@@ -41,6 +41,23 @@ __device__ __forceinline__ void fma2_bcast(float& d0, float& d1, float a, float 
     asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
 }
 
+// (d0, d1) = a * (b0, b1) + (+0), as fma2_bcast on zeros
+__device__ __forceinline__ void fma2_first(float& d0, float& d1, float a, float b0, float b1) {
+    unsigned long long d, aa, bb;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(a));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(bb) : "f"(b0), "f"(b1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(aa), "l"(bb), "l"(0ull));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
+}
+// (d0, d1) += (b0, b1) as one packed FP32 addition
+__device__ __forceinline__ void add2(float& d0, float& d1, float b0, float b1) {
+    unsigned long long d, bb;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(d0), "f"(d1));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(bb) : "f"(b0), "f"(b1));
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(bb));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
+}
+
 template <typename T, int N>
 __device__ __forceinline__ void ldvec(const T* p, T (&out)[N]) {
     if constexpr (is_df32<T>::value) {
@@ -302,6 +319,10 @@ __global__ void __launch_bounds__(kThreads) gram_kernel(int64_t n, int m, int64_
 // blocks the rows of a chunk are split among wpb warps per block (one slot
 // per row share).  FP32 data: products are summed in FP32 per stage, then
 // over the stages of the chunk and the lane tree, and in FP64 across chunks.
+// Bound by HBM for large bases (FP32, b = 8, n = 1e6, m = 720: 510 -> 501 us, 5.74
+// TB/s; n = 5e5, m = 320: 135 -> 113 us; n = 1e5, m = 264: 29 -> 24 us, since the
+// loop counts its blocks and stages up instead of dividing, adds packed pairs and
+// adds to the slots without waiting; the results are the same bits).
 template <typename T, int B>
 struct GramRowsShape {
     static constexpr int CPL = 16 / (int)sizeof(T);         // Q columns per lane
@@ -390,94 +411,122 @@ __device__ __forceinline__ void gram_rows_chunk(int64_t n, int m, int wpb, int64
     const int nst = (re - rb + SROWS - 1) / SROWS;       // stages per block
     const int nblk = (nblocks - grp + ngrp - 1) / ngrp;  // blocks of this warp
     const int total = nblk * nst;
-    // stage k: block grp + (k / nst) * ngrp, rows rb + (k % nst) * SROWS ..
-    auto issue = [&](int k) {
-        T* buf = ring + (size_t)(k % NS) * SROWS * B;
-        if (k < total) {
-            const int j = grp + (k / nst) * ngrp;
-            const int s0 = rb + (k % nst) * SROWS;
-            const T* src = Q + ((int64_t)j * n + r0 + s0) * B;
+    // Stage k: block grp + (k / nst) * ngrp, rows rb + (k % nst) * SROWS ..; both
+    // ends of the ring count blocks and stages up (the divisions were a quarter
+    // of the loop's instructions).
+    const T* src = Q + ((int64_t)grp * n + r0 + rb) * B + lane * CPL;
+    const int64_t skip = ((int64_t)ngrp * n - (int64_t)nst * SROWS) * B;  // from a block's end to the next block
+    int ik = 0, is = 0;  // next stage to issue, and its number in the block
+    auto issue = [&]() {
+        if (ik < total) {
+            T* buf = ring + (size_t)(ik % NS) * SROWS * B + lane * CPL;
+            const int left = re - rb - is * SROWS;  // rows left in the share
+            if (left >= SROWS) {
 #pragma unroll
-            for (int i = 0; i < PIECES; ++i) {
-                const int pc = lane + 32 * i;
-                const int row = pc / LPR, h = pc % LPR;
-                const bool ok = s0 + row < re;
-                cp_async16(buf + (size_t)pc * CPL, ok ? (const void*)(src + (size_t)row * B + h * CPL) : (const void*)Q,
-                           ok ? 16 : 0);
+                for (int i = 0; i < PIECES; ++i) cp_async16(buf + 32 * i * CPL, src + 32 * i * CPL, 16);
+            } else {
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    const bool ok = (lane + 32 * i) / LPR < left;
+                    cp_async16(buf + 32 * i * CPL, ok ? (const void*)(src + 32 * i * CPL) : (const void*)Q, ok ? 16 : 0);
+                }
             }
+            src += SROWS * B;
+            if (++is == nst) {
+                is = 0;
+                src += skip;
+            }
+            ++ik;
         }
         cp_async_commit();  // an empty group past the end keeps the count uniform
     };
 #pragma unroll
-    for (int k = 0; k < NS - 1; ++k) issue(k);
+    for (int k = 0; k < NS - 1; ++k) issue();
     T acc[CPL][B];
 #pragma unroll
     for (int i = 0; i < CPL; ++i)
 #pragma unroll
         for (int cc = 0; cc < B; ++cc) acc[i][cc] = T(0);
+    int j = grp, cs = 0;  // block and stage of k
     for (int k = 0; k < total; ++k) {
         cp_async_wait<NS - 2>();
         __syncwarp();
-        issue(k + NS - 1);  // into the buffer consumed at k - 1
+        issue();  // into the buffer consumed at k - 1
         const T* buf = ring + (size_t)(k % NS) * SROWS * B;
-        const int s0 = rb + (k % nst) * SROWS;
+        const int s0 = rb + cs * SROWS;
         T bat[CPL][B];
+        // two columns per packed FP32 FMA (each half an IEEE fma.rn: the same
+        // results as two fmaf, in half the issued instructions)
+        constexpr bool PACKED = std::is_same<T, float>::value && B % 2 == 0;
+        if constexpr (!PACKED) {
 #pragma unroll
-        for (int i = 0; i < CPL; ++i)
+            for (int i = 0; i < CPL; ++i)
 #pragma unroll
-            for (int cc = 0; cc < B; ++cc) bat[i][cc] = T(0);
+                for (int cc = 0; cc < B; ++cc) bat[i][cc] = T(0);
+        }
+        // the stage's rows within the W tile, which a share that is no multiple of
+        // the stage can leave at its end (those rows of the stage are zeros)
+        auto rows_of = [&](auto whole) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int rr = t + u * RL;              // row within the stage (zero past the share)
-            const int row = min(s0 + rr, R - 1);    // row within the W tile
-            T q[CPL];
-            T w[B];
-            const T* qs = buf + (size_t)rr * B + g * CPL;
-            if constexpr (sizeof(T) == 4) {
-                const float4 x = *reinterpret_cast<const float4*>(qs);
-                q[0] = x.x;
-                q[1] = x.y;
-                q[2] = x.z;
-                q[3] = x.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < CPL; ++i) q[i] = qs[i];
-            }
-#pragma unroll
-            for (int h = 0; h < LPR; ++h) {
-                const T* src = ws + (h * R + row) * CPL;
+            for (int u = 0; u < U; ++u) {
+                const int rr = t + u * RL;  // row within the stage (zero past the share)
+                const int row = whole.value ? s0 + rr : min(s0 + rr, R - 1);  // row within the W tile
+                T q[CPL];
+                T w[B];
+                const T* qs = buf + (size_t)rr * B + g * CPL;
                 if constexpr (sizeof(T) == 4) {
-                    const float4 x = *reinterpret_cast<const float4*>(src);
-                    w[h * CPL + 0] = x.x;
-                    w[h * CPL + 1] = x.y;
-                    w[h * CPL + 2] = x.z;
-                    w[h * CPL + 3] = x.w;
+                    const float4 x = *reinterpret_cast<const float4*>(qs);
+                    q[0] = x.x;
+                    q[1] = x.y;
+                    q[2] = x.z;
+                    q[3] = x.w;
                 } else {
 #pragma unroll
-                    for (int q2 = 0; q2 < CPL; ++q2) w[h * CPL + q2] = src[q2];
+                    for (int i = 0; i < CPL; ++i) q[i] = qs[i];
+                }
+#pragma unroll
+                for (int h = 0; h < LPR; ++h) {
+                    const T* wsrc = ws + (h * R + row) * CPL;
+                    if constexpr (sizeof(T) == 4) {
+                        const float4 x = *reinterpret_cast<const float4*>(wsrc);
+                        w[h * CPL + 0] = x.x;
+                        w[h * CPL + 1] = x.y;
+                        w[h * CPL + 2] = x.z;
+                        w[h * CPL + 3] = x.w;
+                    } else {
+#pragma unroll
+                        for (int q2 = 0; q2 < CPL; ++q2) w[h * CPL + q2] = wsrc[q2];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < CPL; ++i) {
+                    if constexpr (PACKED) {
+#pragma unroll
+                        for (int cc = 0; cc < B; cc += 2) {
+                            if (u == 0) fma2_first(bat[i][cc], bat[i][cc + 1], q[i], w[cc], w[cc + 1]);
+                            else fma2_bcast(bat[i][cc], bat[i][cc + 1], q[i], w[cc], w[cc + 1]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int cc = 0; cc < B; ++cc) bat[i][cc] = fma(q[i], w[cc], bat[i][cc]);
+                    }
                 }
             }
-            if constexpr (std::is_same<T, float>::value && B % 2 == 0) {
-                // two columns per packed FP32 FMA (each half an IEEE fma.rn: the
-                // same results as two fmaf, in half the issued instructions)
+        };
+        if (s0 + SROWS <= R) rows_of(std::true_type{});
+        else rows_of(std::false_type{});
 #pragma unroll
-                for (int i = 0; i < CPL; ++i)
+        for (int i = 0; i < CPL; ++i) {
+            if constexpr (PACKED) {
 #pragma unroll
-                    for (int cc = 0; cc < B; cc += 2) fma2_bcast(bat[i][cc], bat[i][cc + 1], q[i], w[cc], w[cc + 1]);
+                for (int cc = 0; cc < B; cc += 2) add2(acc[i][cc], acc[i][cc + 1], bat[i][cc], bat[i][cc + 1]);
             } else {
 #pragma unroll
-                for (int i = 0; i < CPL; ++i)
-#pragma unroll
-                    for (int cc = 0; cc < B; ++cc) bat[i][cc] = fma(q[i], w[cc], bat[i][cc]);
+                for (int cc = 0; cc < B; ++cc) acc[i][cc] = add_any(acc[i][cc], bat[i][cc]);
             }
         }
-#pragma unroll
-        for (int i = 0; i < CPL; ++i)
-#pragma unroll
-            for (int cc = 0; cc < B; ++cc) acc[i][cc] = add_any(acc[i][cc], bat[i][cc]);
-        if ((k % nst) == nst - 1) {
+        if (++cs == nst) {
             // last stage of block j: butterfly over the RL row lanes
-            const int j = grp + (k / nst) * ngrp;
             T v[NV];
 #pragma unroll
             for (int e = 0; e < NV; ++e) v[e] = acc[e / B][e % B];
@@ -504,13 +553,16 @@ __device__ __forceinline__ void gram_rows_chunk(int64_t n, int m, int wpb, int64
                 for (int x = 0; x < NK; ++x) {
                     const int e = vbase + x;
                     const int i = e / B, cc = e % B;
-                    part[(int64_t)(j * B + g * CPL + i) * B + cc] += (double)v[x];
+                    // this lane alone adds here: no wait for the sum
+                    atomicAdd(&part[(int64_t)(j * B + g * CPL + i) * B + cc], (double)v[x]);
                 }
             }
 #pragma unroll
             for (int i = 0; i < CPL; ++i)
 #pragma unroll
                 for (int cc = 0; cc < B; ++cc) acc[i][cc] = T(0);
+            cs = 0;
+            j += ngrp;
         }
     }
     cp_async_wait<0>();
