@@ -1000,7 +1000,8 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const unsigned (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, int nchunks,
+template <bool GROUPED>
+__global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, int nitems, int groups,
                                                              const __half* __restrict__ Q, const float* __restrict__ W,
                                                              double* __restrict__ partial, int* __restrict__ ticket) {
     constexpr int B = 8;
@@ -1015,14 +1016,19 @@ __global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, i
     const int g = lane >> 2, tig = lane & 3;
     double* part = partial + (int64_t)blockIdx.x * m * B;
     for (int e = threadIdx.x; e < m * B; e += kThreads) part[e] = 0.0;
-    const int mypairs = warp < npairs ? (npairs - warp + kHmWarps - 1) / kHmWarps : 0;
+    const int per_group = GROUPED ? (npairs + groups - 1) / groups : npairs;  // pairs of an item
     constexpr int NST = kHalfRows / 16 / kHmSK;  // stages per pair per chunk
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_chunk = atomicAdd(ticket, 1);
         __syncthreads();
-        const int c = s_chunk;
-        if (c >= nchunks) break;
+        const int item = s_chunk;
+        if (item >= nitems) break;
+        // an item is a chunk and a group of its pairs
+        const int c = GROUPED ? item / groups : item;
+        const int p0 = GROUPED ? (item - c * groups) * per_group + warp : warp;
+        const int p1 = GROUPED ? min(npairs, p0 - warp + per_group) : npairs;
+        const int mypairs = p0 < p1 ? (p1 - p0 + kHmWarps - 1) / kHmWarps : 0;
         const int64_t r0 = (int64_t)c * kHalfRows;
         const int rows = (int)min((int64_t)kHalfRows, n - r0);
         // the chunk's largest |W| -> power-of-two scale
@@ -1043,11 +1049,11 @@ __global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, i
             ws[e] = __float2half_rn(e < rows * B ? W[r0 * B + e] * scale : 0.f);
         __syncthreads();
         const int total = mypairs * NST;
-        // ring stage k: pair warp + (k / NST) * kHmWarps, rows (k % NST) * 16 * kHmSK ..
+        // ring stage k: pair p0 + (k / NST) * kHmWarps, rows (k % NST) * 16 * kHmSK ..
         // lane L copies row (L & 15) of block 2p + (L >> 4) for each tile u
         auto issue = [&](int k) {
             if (k < total) {
-                const int p = warp + (k / NST) * kHmWarps;
+                const int p = p0 + (k / NST) * kHmWarps;
                 const int j = 2 * p + (lane >> 4);
                 __half* buf = ring[warp][k % kHmNS];
 #pragma unroll
@@ -1081,7 +1087,7 @@ __global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, i
             }
             if ((k % NST) == NST - 1) {
                 // the pair's sums over this chunk: rows g (block 2p) and g + 8 (block 2p + 1), columns 2 tig, 2 tig + 1
-                const int p = warp + (k / NST) * kHmWarps;
+                const int p = p0 + (k / NST) * kHmWarps;
                 const int j0 = 2 * p, j1 = 2 * p + 1;
                 double* o0 = part + ((int64_t)j0 * B + g) * B + 2 * tig;
                 o0[0] += (double)acc[0] * unscale;
@@ -1102,18 +1108,26 @@ bbl_status launch_gram_half(int64_t n, int m, const __half* Q, const float* W, d
                             cudaStream_t st) {
     static int occ = 0;
     if (occ == 0) {
-        BBL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gram_half_kernel, kThreads, 0));
+        BBL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gram_half_kernel<false>, kThreads, 0));
         if (occ < 1) occ = 1;
     }
     const int64_t slots_max = (int64_t)std::max(1, sm_count() - kRitzReserveSMs) * occ;
     const int nch = (int)std::max<int64_t>(1, ceil_div(n, kHalfRows));
-    const int64_t workers = std::min<int64_t>(slots_max, nch);
+    // fewer chunks than SMs: a chunk's pairs are split into groups of at least one
+    // pair per warp (n = 1e5, 60 blocks: 48.4 us, in three groups 32.9; with more
+    // chunks than that the groups' partial sums cost more)
+    const int npairs = (m / 8 + 1) / 2;
+    int64_t groups = 1;
+    if (nch < sm_count()) groups = std::max<int64_t>(1, std::min<int64_t>(ceil_div(slots_max, nch), npairs / kHmWarps));
+    const int64_t workers = std::min<int64_t>(slots_max, nch * groups);
     const int64_t per = (int64_t)m * 8;
     const size_t need = sizeof(double) * (size_t)(workers * per) + 256;
     BBL_TRY(partials.grow(need));
     int* ticket = reinterpret_cast<int*>(partials.as<char>() + sizeof(double) * (size_t)(workers * per));
     BBL_CUDA(cudaMemsetAsync(ticket, 0, sizeof(int), st));
-    gram_half_kernel<<<(unsigned)workers, kThreads, 0, st>>>(n, m, nch, Q, W, partials.as<double>(), ticket);
+    const auto kernel = groups > 1 ? gram_half_kernel<true> : gram_half_kernel<false>;
+    kernel<<<(unsigned)workers, kThreads, 0, st>>>(n, m, (int)(nch * groups), (int)groups, Q, W, partials.as<double>(),
+                                                   ticket);
     BBL_LAUNCH_CHECK();
     launch_reduce(per, (int)workers, partials.as<double>(), C, st);
     BBL_LAUNCH_CHECK();
@@ -1368,6 +1382,7 @@ __global__ void __launch_bounds__(256) half_old_prep_kernel(int jsplit, const do
 // One warp per 16-row tile.  A fragments of the older blocks come straight
 // from global memory (each 4-byte load of a warp covers 8 rows x 16 bytes
 // of one block: one 128-byte line).
+template <int U, bool AHEAD>
 __global__ void __launch_bounds__(256) apply_half_old_kernel(int64_t n, int nblocks, int jsplit,
                                                              const __half* __restrict__ Q16,
                                                              const float* __restrict__ Q,
@@ -1383,28 +1398,47 @@ __global__ void __launch_bounds__(256) apply_half_old_kernel(int64_t n, int nblo
     const unsigned* Q16w = reinterpret_cast<const unsigned*>(Q16);  // two halves per word
     float d[4] = {0.f, 0.f, 0.f, 0.f};
     const int npo = (jsplit + 1) >> 1;
-    // groups of kHoU block pairs: every load of a group is issued before its products
-    constexpr int kHoU = 8;
-    for (int q0 = 0; q0 < npo; q0 += kHoU) {
-        unsigned a[kHoU][4];
-        unsigned b[kHoU][2];
+    // groups of U block pairs; AHEAD: two in turn, a group's loads issued before the
+    // products of the group before it, else all loads of a group before its products
+    struct Group {
+        unsigned a[U][4], b[U][2];
+    };
+    auto load = [&](int q0, Group& x) {
 #pragma unroll
-        for (int u = 0; u < kHoU; ++u) {
+        for (int u = 0; u < U; ++u) {
             const int q = q0 + u;
             const bool on = q < npo;
             const int j0 = on ? 2 * q : 0;
             const int j1 = (on && 2 * q + 1 < nblocks) ? 2 * q + 1 : j0;  // past the basis: b1 is zero
-            a[u][0] = (on && oka) ? __ldg(Q16w + (((int64_t)j0 * n + ra) * 8 + 2 * t) / 2) : 0u;
-            a[u][1] = (on && okb) ? __ldg(Q16w + (((int64_t)j0 * n + rb) * 8 + 2 * t) / 2) : 0u;
-            a[u][2] = (on && oka) ? __ldg(Q16w + (((int64_t)j1 * n + ra) * 8 + 2 * t) / 2) : 0u;
-            a[u][3] = (on && okb) ? __ldg(Q16w + (((int64_t)j1 * n + rb) * 8 + 2 * t) / 2) : 0u;
+            x.a[u][0] = (on && oka) ? __ldg(Q16w + (((int64_t)j0 * n + ra) * 8 + 2 * t) / 2) : 0u;
+            x.a[u][1] = (on && okb) ? __ldg(Q16w + (((int64_t)j0 * n + rb) * 8 + 2 * t) / 2) : 0u;
+            x.a[u][2] = (on && oka) ? __ldg(Q16w + (((int64_t)j1 * n + ra) * 8 + 2 * t) / 2) : 0u;
+            x.a[u][3] = (on && okb) ? __ldg(Q16w + (((int64_t)j1 * n + rb) * 8 + 2 * t) / 2) : 0u;
             const uint2 f = on ? __ldg(frag + q * 32 + lane) : make_uint2(0u, 0u);
-            b[u][0] = f.x;
-            b[u][1] = f.y;
+            x.b[u][0] = f.x;
+            x.b[u][1] = f.y;
         }
+    };
+    auto products = [&](int q0, const Group& x) {
 #pragma unroll
-        for (int u = 0; u < kHoU; ++u)
-            if (q0 + u < npo) mma_16816(d, a[u], b[u]);
+        for (int u = 0; u < U; ++u)
+            if (q0 + u < npo) mma_16816(d, x.a[u], x.b[u]);
+    };
+    Group g0;
+    if constexpr (AHEAD) {
+        Group g1;
+        if (npo > 0) load(0, g0);
+        for (int q0 = 0; q0 < npo; q0 += 2 * U) {
+            if (q0 + U < npo) load(q0 + U, g1);
+            products(q0, g0);
+            if (q0 + 2 * U < npo) load(q0 + 2 * U, g0);
+            products(q0 + U, g1);
+        }
+    } else {
+        for (int q0 = 0; q0 < npo; q0 += U) {
+            load(q0, g0);
+            products(q0, g0);
+        }
     }
     const float inv = npo > 0 ? __ldg(scale) : 0.f;
     // acc[row][col]: rows ra / rb, columns 2t, 2t + 1
@@ -1771,8 +1805,14 @@ bbl_status update_half_old(int64_t n, int nblocks, int nnew, const void* Q16, co
         BBL_LAUNCH_CHECK();
     }
     const int64_t warps = ceil_div(n, (int64_t)16);
-    apply_half_old_kernel<<<(unsigned)ceil_div(warps * 32, 256), 256, 0, st>>>(
-        n, nblocks, jsplit, static_cast<const __half*>(Q16), Q, C, frag, scale, W);
+    // With 48 warps per SM and more, few registers and two pairs ahead: n = 1e6, 90
+    // blocks 275 -> 261 us, n = 5e5, 45 blocks 89 -> 80 (3 ahead 278 and 89, 4 ahead 305
+    // and 104: the registers cost more warps than the loads in flight bring).  With
+    // fewer, eight pairs at once: n = 9000, 90 blocks 10.1 us, two ahead 11.1; n = 6e4
+    // 25.0 and 26.3; n = 1e5, 60 blocks 27.0 and 27.3.
+    const auto kernel = warps >= (int64_t)sm_count() * 48 ? apply_half_old_kernel<2, true> : apply_half_old_kernel<8, false>;
+    kernel<<<(unsigned)ceil_div(warps * 32, 256), 256, 0, st>>>(n, nblocks, jsplit, static_cast<const __half*>(Q16), Q, C,
+                                                                frag, scale, W);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
