@@ -393,11 +393,15 @@ bbl_status bbl_cholqr2(int64_t n, int b, bbl_dtype dtype, void* W, double* B, do
  * Tband[i*(p+1) + d] = T[i][i-d] (d = 0..p; entries with i-d < 0 ignored).
  *   theta  device FP64 [nev] ascending;  S device FP64 m x nev row-major,
  *   unit columns (sign: first largest-magnitude entry positive).
- * Method: Sylvester-inertia bisection (LDL^T of T - sigma I) then inverse
- * iteration (banded LU with partial pivoting) and Rayleigh quotients; the
- * vectors of clustered eigenvalues are orthonormalised together.  For
- * p in {1, 2, 4, 8} the recurrences run in FP32 and float-float (~48-bit)
- * arithmetic; normalisation and Rayleigh quotients are FP64.
+ * Method: where the FP32 band fits in shared memory (m up to about 6000 at p =
+ * 8) the spectrum is sliced by eigenvalue counts at many shifts, and each pair
+ * is found by FP32 block cyclic reduction of T - sigma I with corrections from
+ * FP64 residuals; a pair that this does not certify, and longer bands, by
+ * Sylvester-inertia bisection (LDL^T of T - sigma I), inverse
+ * iteration (banded LU with partial pivoting) and Rayleigh quotients.  The
+ * vectors of clustered eigenvalues are orthonormalised together.  For p in
+ * {1, 2, 4, 8} the second route's recurrences run in FP32 and float-float
+ * (~48-bit) arithmetic; normalisation and Rayleigh quotients are FP64.
  * 1 <= nev <= min(m, 32), p <= 16, m <= 16384.                                   */
 bbl_status bbl_ritz_banded(int m, int p, int nev, const double* Tband, double* theta, double* S,
                            void* stream);
