@@ -1590,7 +1590,7 @@ constexpr int kCholParts = 128;  // most partial Grams one CTA adds itself (two 
 // by one thread per segment, this one about 8.)
 struct CholShared {
     double G[kMaxB * kMaxB];
-    double L[kMaxB * kMaxB];      // row k: L[.][k]
+    double L[kMaxB * kMaxB];      // row k: D[k] L[.][k]
     double Z[kMaxB * kMaxB];      // row k of L^{-1}
     double row[2][2][kMaxB];      // row k of the Schur complement and of L^{-1}
     double d[kMaxB], root[kMaxB]; // D (0 for deflated columns) and its square roots
@@ -1638,7 +1638,7 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
             sh.d[k] = defl ? 0.0 : d;
         }
         if (lane < b) {
-            sh.L[k * b + lane] = lane < k || defl ? 0.0 : ra[lane] * y;
+            sh.L[k * b + lane] = lane < k || defl ? 0.0 : ra[lane];
             sh.Z[k * b + lane] = lane > k || defl ? 0.0 : rz[lane];
         }
 #pragma unroll
@@ -1660,7 +1660,12 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
 }
 
 // entry e of R = D^{1/2} L^T and of R^{-1}: zero rows (columns) for deflated columns
-__device__ __forceinline__ double chol_R(const CholShared& sh, int b, int e) { return sh.L[e] * sh.root[e / b]; }
+// (one division each: L scaled by the root, after the reciprocal, rounds twice more)
+__device__ __forceinline__ double chol_R(const CholShared& sh, int b, int e) {
+    const int i = e / b, c = e - i * b;
+    if (c <= i || sh.deflated[i]) return c == i ? sh.root[i] : 0.0;
+    return sh.L[e] / sh.root[i];
+}
 __device__ __forceinline__ double chol_Rinv(const CholShared& sh, int b, int e) {
     const int i = e / b, c = e % b;
     return c >= i && !sh.deflated[c] ? sh.Z[c * b + i] / sh.root[c] : 0.0;
@@ -1702,14 +1707,15 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(int b, int nparts, c
     }
     __syncthreads();
     if (tid < bb) {
-        const int i = tid / b, c = tid % b;
-        R[tid] = chol_R(sh, b, tid);
+        red[tid] = R[tid] = chol_R(sh, b, tid);
         Rinv[tid] = chol_Rinv(sh, b, tid);
-        if (Bout) {
-            double s = 0.0;
-            for (int l = i; l <= c; ++l) s += sh.L[i * b + l] * sh.root[i] * R1[l * b + c];
-            Bout[tid] = s;
-        }
+    }
+    __syncthreads();
+    if (Bout && tid < bb) {
+        const int i = tid / b, c = tid % b;
+        double s = 0.0;
+        for (int l = i; l <= c; ++l) s += red[i * b + l] * R1[l * b + c];
+        Bout[tid] = s;
     }
     if (mask && tid < b) mask[tid] = sh.deflated[tid];
 }
