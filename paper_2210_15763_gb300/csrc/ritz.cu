@@ -1064,23 +1064,29 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
     if (tid == 0) s_scale_bits = 0;
     __syncthreads();
     // scale = max |theta|, at least the largest diagonal magnitude (non-negative
-    // doubles order as their bits)
+    // doubles order as their bits), NaN left out
     {
         unsigned long long sc = 0;
-        for (int r = tid; r < m; r += 256)
-            sc = max(sc, (unsigned long long)__double_as_longlong(Tb[(int64_t)r * (p + 1)]) & 0x7fffffffffffffffull);
-        if (tid < nev) sc = max(sc, (unsigned long long)__double_as_longlong(theta[tid]) & 0x7fffffffffffffffull);
+        auto take = [&](double v) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+            if (b <= 0x7ff0000000000000ull) sc = max(sc, b);
+        };
+        for (int r = tid; r < m; r += 256) take(Tb[(int64_t)r * (p + 1)]);
+        if (tid < nev) take(theta[tid]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sc = max(sc, __shfl_xor_sync(0xffffffffu, sc, o));
         if ((tid & 31) == 0) atomicMax(&s_scale_bits, sc);
     }
-    // rank of each value (ties by index)
+    // rank of each value: a total order, so that every rank is taken once (NaN
+    // last, ties and NaN among themselves by index)
     if (tid < nev) {
         const double v = theta[tid];
         int rank = 0;
         for (int k = 0; k < nev; ++k) {
             const double o = theta[k];
-            rank += (o < v || (o == v && k < tid)) ? 1 : 0;
+            const bool before = isnan(v) ? !isnan(o) : o < v;
+            const bool same = isnan(v) ? isnan(o) : o == v;
+            rank += (before || (same && k < tid)) ? 1 : 0;
         }
         th[rank] = v;
         order[rank] = tid;
@@ -1091,7 +1097,7 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
         int g = 0, ok = 1;
         start[0] = 0;
         for (int k = 1; k < nev; ++k) {
-            if (th[k] - th[k - 1] > 1e-3 * s_scale) start[++g] = k;
+            if (!(th[k] - th[k - 1] <= 1e-3 * s_scale)) start[++g] = k;  // a NaN stands alone
             ok = ok && order[k] > order[k - 1];
         }
         start[++g] = nev;
