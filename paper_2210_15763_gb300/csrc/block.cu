@@ -2056,7 +2056,7 @@ bbl_status apply_seg_typed(int64_t n, int b, int kc, const int* ms, int mss, con
 
 int gram_seg_chunk_rows(int b, int dtype) {
     if (dtype == BBL_FP64) {
-        if (b == 4 || b == 8) return 512;  // the tensor-core form's chunk; within the row kernel's tile
+        if (b == 4 || b == 8) return tc64_seg_chunk_rows();  // within the row kernel's tile
     } else if (dtype == BBL_FP32) {
         if (b == 4) return GramRowsShape<float, 4>::R;
         if (b == 8) return GramRowsShape<float, 8>::R;

@@ -315,6 +315,7 @@ bbl_status update_tc64(int64_t n, int b, int m, int kc, const double* Q, const d
                        cudaStream_t st);
 // segmented forms (b that tc64_seg_supports names; block.cu explains the tables)
 bool tc64_seg_supports(int b);
+int tc64_seg_chunk_rows();  // rows of a chunk at most
 bbl_status gram_tc64_seg(int64_t n, int b, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
                          int nchunks, const int* active, double* partial, cudaStream_t st);
 bbl_status update_tc64_seg(int64_t n, int b, const int* ms, int ms_stride, const int64_t* ctas, int nctas,

@@ -4,25 +4,43 @@
 //
 // GB300's FP64 pipes (1.06 TFLOP/s measured) bind C = Q^T W and W -= Q C at
 // 16 operations per 8-byte basis element (b = 8): 12 times the time HBM needs.
-// Here an FP64 number becomes an integer of 56 bits relative to a power of
-// two near its row's (or column's) largest entry, cut into seven digits of 8
+// Here an FP64 number becomes an integer of 64 bits relative to a power of
+// two near its row's (or column's) largest entry, cut into eight digits of 8
 // bits; a digit with its sign is an FP16 number, and a product of two digit
 // matrices is exact in the tensor cores' FP32 sums as long as these stay
 // below 2^24.  Digit products i, j of one order o = i + j share an
-// accumulator: 34 products give the orders 0..7.  Orders 0..3 are exact:
-// after 64 terms (at most 64 (1023 * 128 + 2 * 255 * 128 + 255 * 256) < 2^24) they move to
-// 32-bit integers; orders 4..7 weigh 2^-32 and less, where FP32 rounding is
-// below 2^-56.  The basis is cut in sign and magnitude (the first digit has
-// two spare bits, so a line may outgrow its first entries fourfold); the
-// other operand, cut once per CTA, into balanced digits -128..127 of the
-// rounded value, so that the dropped orders (below 2^-62 of the largest
-// products) have random signs instead of the products' own.
+// accumulator: 36 products give the orders 0..7.  Orders 0..4 move to 64-bit
+// integers after every 64 terms (at most 64 (1023 * 128 + 3 * 255 * 128 + 255 * 256) <
+// 1.13 * 2^24, and above 2^24 only where the first digits are large); orders 5..7
+// weigh 2^-40 and less, where FP32 rounding is below 2^-62.  The basis is cut in
+// sign and magnitude (the first digit has two spare bits, so a line may outgrow
+// its first entries fourfold); the other operand, cut once per CTA, into balanced
+// digits -128..127 of the rounded value, so that the dropped orders (below 2^-62 of
+// the largest products) have random signs instead of the products' own.
+//
+// What the cut loses is measured against a line's largest entry, and a sum whose
+// own terms are all far below that (a basis column with one large entry opposite
+// a zero, a row that is tiny where the coefficients are large) would lose bits that
+// FP64 sums keep.  So each sum certifies itself: one more product, of the two
+// leading digits' magnitudes, gives Sigma = sum |q||w| in units of 2^96 of the
+// (56-bit) integers' product, to two digits.  What is dropped and truncated is at most 2^50 per term,
+// and about 2^46.5 with a random sign: 2^51 over 512 terms.  From Sigma = 64 = 2^102 on that is
+// 4 x 2^-53 of sum |q||w| over 512 terms (2 N x 2^-53 for N terms if all signs
+// agree; the bound of an FP64 sum in sequence is N x 2^-53).  A sum below, or with
+// an operand that is not finite, is formed again by FP64 FMA, which also treats
+// infinities and numbers below the digits' range as FP64 does.  In a Lanczos run
+// that is about one sum in 10^5.  The largest error of any sum, relative to its
+// sum of magnitudes, on orthonormal bases (n = 2e4, b = 4, 360 columns; n = 2e5, b = 8,
+// 400): Gram 9.1e-17 and 1.1e-16, update 5.8e-17 and 7.4e-17; FP64 FMA kernels
+// 1.3e-16 and 1.8e-16, 1.9e-16 and 2.8e-16; 56-bit integers without the check
+// 9.2e-17 and 1.2e-16, 6.1e-16 and 6.1e-16.
 //
 // Digits are cut by integer instructions in registers from a ring of
-// asynchronous copies.  At n = 2e5, b = 8, 50 blocks (640 MB, 94 us at the copy
-// rate) the Gram takes 0.25 ms and the update 0.24 ms; the FP64 FMA kernels
-// took 1.67 and 1.20 ms.  What bounds them now is instruction issue (integer
-// pipe 51-55 %, tensor pipe 33 % active, DRAM a third of the copy rate).
+// asynchronous copies.  At n = 6e5, b = 8, 90 blocks (3.5 GB, 0.51 ms at the copy
+// rate) the Gram takes 1.25 ms and the update 1.21 ms (with 56 bits and no check
+// 1.09 and 1.12).  What bounds them is the latency of the cutting at four warps per
+// scheduler (integer pipe about half, tensor pipe a third active, DRAM a third of
+// the copy rate).
 #include <algorithm>
 #include <cstdint>
 
@@ -35,11 +53,12 @@ namespace {
 
 constexpr int kT = 256;            // threads per CTA
 constexpr int kWarps = kT / 32;
-constexpr int kDig = 7;            // digits of 8 bits
-constexpr int kOrd = 8;            // orders summed (of the products' 13)
-constexpr int kExact = 4;          // orders kept exactly
+constexpr int kDig = 8;            // digits of 8 bits
+constexpr int kOrd = 8;            // orders summed (of the products' 15)
+constexpr int kExact = 5;          // orders kept exactly
+constexpr float kCertified = 64.0f;   // a sum's Sigma from which the digits' error is that of FP64 sums
 constexpr int kOver = 2;           // bits by which an entry may exceed its line's scale (the first digit's spare bits)
-constexpr int kMaxRows = 512;      // Gram: rows per CTA
+constexpr int kMaxRows = 448;      // Gram: rows per CTA (two CTAs per SM by their shared memory)
 constexpr int kMaxCols = 512;      // update: coefficient rows staged at once
 constexpr int kEmin = 100;         // smallest exponent field used for a scale
 constexpr int kRing = 3;           // steps of a warp in its shared-memory ring
@@ -47,32 +66,38 @@ constexpr int kStepBytes = 2048;   // 16 x 16 basis entries
 
 struct Acc {
     float f[kOrd][4];   // order sums
-    int h[kExact][4];   // exact sums of the first orders
-    __device__ __forceinline__ void clear() {
+    long long h[4];     // exact sums of the first orders, in units of order 4
+    float c[4];         // Sigma, in units of the present scales
+    __device__ __forceinline__ Acc() {
+        clear();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[e] = 0.0f;
+    }
+    __device__ __forceinline__ void clear() {  // the sums, not Sigma
 #pragma unroll
         for (int o = 0; o < kOrd; ++o)
 #pragma unroll
             for (int e = 0; e < 4; ++e) f[o][e] = 0.0f;
 #pragma unroll
-        for (int o = 0; o < kExact; ++o)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) h[o][e] = 0;
+        for (int e = 0; e < 4; ++e) h[e] = 0;
     }
     __device__ __forceinline__ void to_int() {
 #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i1 = __float2int_rn(f[1][e]), i2 = __float2int_rn(f[2][e]), i3 = __float2int_rn(f[3][e]);
+            const long long up = (long long)i1 * (1 << 24) + h[e];
+            const long long low = (long long)i3 * (1 << 8) + ((long long)i2 * (1 << 16) + __float2int_rn(f[4][e]));
+            h[e] = up + low + (long long)__float2int_rn(f[0][e]) * (1ll << 32);
+        }
+#pragma unroll
         for (int o = 0; o < kExact; ++o)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                h[o][e] += __float2int_rn(f[o][e]);
-                f[o][e] = 0.0f;
-            }
+            for (int e = 0; e < 4; ++e) f[o][e] = 0.0f;
     }
-    // the sum over the orders in units of order 3 (call to_int before)
+    // the sum over the orders in units of order 4 (call to_int before)
     __device__ __forceinline__ double value(int e) const {
-        const long long H = ((long long)h[0][e] << 24) + ((long long)h[1][e] << 16) + ((long long)h[2][e] << 8) +
-                            (long long)h[3][e];
-        const float L = fmaf(f[4][e], 0x1p-8f, fmaf(f[5][e], 0x1p-16f, fmaf(f[6][e], 0x1p-24f, f[7][e] * 0x1p-32f)));
-        return (double)H + (double)L;
+        const float L = fmaf(fmaf(f[7][e], 0x1p-8f, f[6][e]), 0x1p-8f, f[5][e]);
+        return fma((double)L, 0x1p-8, (double)h[e]);
     }
 };
 
@@ -125,49 +150,62 @@ __device__ __forceinline__ void aligned_mantissa(double v, unsigned& yl, unsigne
 }
 
 // The magnitude of v relative to the exponent field E: floor(|v| 2^(55 - (E
-// - 1023))), below 2^56 if v's exponent field is at most E; s = shift_word
-// with bits 5..10 clear.
-__device__ __forceinline__ uint2 magnitude(double v, unsigned s) {
+// - 1023))), below 2^56 if v's exponent field is at most E, in .x, .y, and the
+// next eight bits in the top of .z; s = shift_word with bits 5..10 clear.
+__device__ __forceinline__ uint3 magnitude(double v, unsigned s) {
     unsigned yl, yh;
     aligned_mantissa(v, yl, yh);
-    return make_uint2(__funnelshift_r(yl, yh, s), __funnelshift_r(yh, 0u, s));
+    return make_uint3(__funnelshift_r(yl, yh, s), __funnelshift_r(yh, 0u, s), __funnelshift_r(0u, yl, s));
 }
 
 // the same for any s with v at most kOver bits above the scale
-__device__ __forceinline__ uint2 magnitude_any(double v, unsigned s) {
+__device__ __forceinline__ uint3 magnitude_any(double v, unsigned s) {
     unsigned yl, yh;
     aligned_mantissa(v, yl, yh);
     s &= 0x7ffu;
-    if (s >= 64) return make_uint2(0u, 0u);
-    if (s >= 32) return make_uint2(yh >> (s - 32), 0u);
-    return make_uint2(__funnelshift_r(yl, yh, s), yh >> s);
+    if (s >= 96) return make_uint3(0u, 0u, 0u);
+    if (s >= 64) return make_uint3(0u, 0u, yh >> (s - 64));
+    if (s >= 32) return make_uint3(yh >> (s - 32), 0u, __funnelshift_r(yl, yh, s - 32));
+    return make_uint3(__funnelshift_r(yl, yh, s), yh >> s, __funnelshift_r(0u, yl, s));
 }
 
+__device__ __forceinline__ unsigned fma_f16x2(unsigned a, unsigned b, unsigned c) {
+    unsigned r;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
 // Two magnitudes and the high words that carry their signs: digit i
-// (0 = most significant) of both as a pair of signed FP16 numbers.
+// (0 = most significant) of both as a pair of signed FP16 numbers.  The integer
+// ALU is the busiest pipe, and per pair of digits this takes one and a half byte
+// permutations (one interleaves two entries' bytes, one each puts two of them
+// below the exponent of 1024) and one FMA.
 struct Pair {
-    uint2 u, v;
-    unsigned sg, off;  // +-1 and -+1024 as FP16 pairs
+    unsigned w0, w12, w34, w56;  // interleaved: 1024 + digit 0; digits 2, 1; 4, 3; 6, 5
+    unsigned last;               // digit 7
+    unsigned sg, off;            // +-1 and -+1024 as FP16 pairs
     template <bool ANY>
     __device__ __forceinline__ void set(double a, double b, unsigned sa, unsigned sb) {
-        u = ANY ? magnitude_any(a, sa) : magnitude(a, sa);
-        v = ANY ? magnitude_any(b, sb) : magnitude(b, sb);
+        const uint3 x = ANY ? magnitude_any(a, sa) : magnitude(a, sa);
+        const uint3 y = ANY ? magnitude_any(b, sb) : magnitude(b, sb);
         const unsigned s = __byte_perm((unsigned)__double2hiint(a), (unsigned)__double2hiint(b), 0x7430) & 0x80008000u;
         sg = s | 0x3c003c00u;
         off = s ^ 0xe400e400u;
+        w0 = __byte_perm(x.y, y.y, 0x7632) | 0x64006400u;  // the bits from 48 on: up to ten
+        w12 = __byte_perm(x.y, y.y, 0x5140);
+        w34 = __byte_perm(x.x, y.x, 0x7362);
+        w56 = __byte_perm(x.x, y.x, 0x5140);
+        last = fma_f16x2((__byte_perm(x.z, y.z, 0x7733) & 0x00ff00ffu) | 0x64006400u, sg, off);
     }
     template <int I>
     __device__ __forceinline__ unsigned digit() const {
-        unsigned x;  // 1024 + digit
-        if constexpr (I == 0) {
-            x = __byte_perm(u.y, v.y, 0x7632) | 0x64006400u;  // the bits from 48 on: up to ten
-        } else {
-            constexpr int byte = I < 3 ? 2 - I : 6 - I;
-            constexpr unsigned sel = (unsigned)(byte | (byte << 4) | ((4 + byte) << 8) | ((4 + byte) << 12));
-            x = (__byte_perm(I < 3 ? u.y : u.x, I < 3 ? v.y : v.x, sel) & 0x00ff00ffu) | 0x64006400u;
-        }
+        if constexpr (I == 7) return last;
+        if constexpr (I == 0) return fma_f16x2(w0, sg, off);
+        const unsigned w = I < 3 ? w12 : I < 5 ? w34 : w56;
+        return fma_f16x2(__byte_perm(w, 0x64646464u, I % 2 ? 0x4342 : 0x4140), sg, off);
+    }
+    __device__ __forceinline__ unsigned lead() const {  // digit 0 without its sign
         unsigned r;
-        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(sg), "r"(off));
+        asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w0), "r"(0xe400e400u));
         return r;
     }
 };
@@ -184,6 +222,9 @@ __device__ __forceinline__ void mma_step(Acc& acc, const Pair (&p)[4], const uin
     uint2 b[kDig];
 #pragma unroll
     for (int j = 0; j < kDig; ++j) b[j] = frag[j * 32 + lane];
+    mma_digit<7>(acc, p, b);
+    const unsigned a[4] = {p[0].lead(), p[1].lead(), p[2].lead(), p[3].lead()};
+    mma_f16(acc.c, a, make_uint2(b[0].x & 0x7fff7fffu, b[0].y & 0x7fff7fffu));
     mma_digit<0>(acc, p, b);
     mma_digit<1>(acc, p, b);
     mma_digit<2>(acc, p, b);
@@ -193,36 +234,60 @@ __device__ __forceinline__ void mma_step(Acc& acc, const Pair (&p)[4], const uin
     mma_digit<6>(acc, p, b);
 }
 
-// round(v 2^(55 - (E - 1023))) plus 128 in each of the low six bytes and 384 in
-// the bits above: balanced digits -128 .. 127 (the first -256 .. 256) in
-// unsigned fields; E at least v's exponent field.
+// r = round(|v| 2^(63 - (E - 1023))) with v's sign in balanced digits -128 .. 127
+// (the first -256 .. 256, the last -128 .. 128); E at least v's exponent field.  The
+// first seven come in unsigned fields: plus 128 in each of the low six bytes of q
+// and 384 in the bits above.
 constexpr unsigned long long kBalance = 0x0180808080808080ull;
-__device__ __forceinline__ unsigned long long balanced(double v, int E) {
-    if (exp_bits(v) == 0) return kBalance;  // zero (or denormal)
-    const uint2 q = magnitude_any(v, shift_word(E - 1, v));
-    const unsigned long long r = ((((unsigned long long)q.y << 32) | q.x) + 1) >> 1;
-    return (v < 0.0 ? 0ull - r : r) + kBalance;
+struct Balanced {
+    unsigned long long q;
+    int last;
+};
+__device__ __forceinline__ Balanced balanced(double v, int E) {
+    const unsigned hi = (unsigned)__double2hiint(v);
+    const int ex = (int)(hi >> 20) & 0x7ff;
+    if (ex == 0) return {kBalance, 0};  // zero (or denormal)
+    // the mantissa with its leading bit at 63, then rounded to the place
+    const unsigned lo = (unsigned)__double2loint(v);
+    unsigned long long r =
+        ((unsigned long long)__funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 11) << 32) | (lo << 11);
+    const int d = E - ex;
+    if (d > 0) r = ((r >> min(d - 1, 63)) + 1) >> 1;
+    if (d > 64) r = 0;
+    const unsigned long long h = (r + 128) >> 8;  // (no carry out: eleven bits below the mantissa are zero)
+    const int last = (int)(signed char)(r & 255u);
+    const bool neg = (hi >> 31) != 0;
+    return {neg ? kBalance - h : kBalance + h, neg ? -last : last};
 }
 
 // B's digits of one lane: terms x[0], x[1] and x[2], x[3] of its column,
 // exponent field E of the column's scale
 __device__ __forceinline__ void store_frag(uint2* __restrict__ frag, int lane, const double (&x)[4], int E) {
-    unsigned long long q[4];
+    Balanced q[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) q[i] = balanced(x[i], E);
 #pragma unroll
     for (int j = 0; j < kDig; ++j) {
-        const int sh = 8 * (kDig - 1 - j);
+        const int sh = 8 * (kDig - 2 - j);
+        const unsigned mask = j == 0 ? 0x3ffu : 0xffu;
         unsigned w[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const unsigned mask = j == 0 ? 0x3ffu : 0xffu;
-            const unsigned lo = (unsigned)(q[2 * h] >> sh) & mask, hi = (unsigned)(q[2 * h + 1] >> sh) & mask;
+            const Balanced &p0 = q[2 * h], &p1 = q[2 * h + 1];
+            const unsigned lo = j < 7 ? (unsigned)(p0.q >> max(sh, 0)) & mask : (unsigned)(p0.last + 128);
+            const unsigned hi = j < 7 ? (unsigned)(p1.q >> max(sh, 0)) & mask : (unsigned)(p1.last + 128);
             const unsigned b = 0x64006400u | lo | (hi << 16);  // 1024 + 128 (or 384) + digit
             asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w[h]) : "r"(b), "r"(j == 0 ? 0xe580e580u : 0xe480e480u));
         }
         frag[j * 32 + lane] = make_uint2(w[0], w[1]);
     }
+}
+
+// the field by which a column's entry counts towards its scale: its exponent, 1
+// for a denormal number (0 stands for a column of zeros)
+__device__ __forceinline__ int scale_field(double v) {
+    const int e = exp_bits(v);
+    return e == 0 && v != 0.0 ? 1 << 20 : e;
 }
 
 // The A operand's scales: a lane's registers 0 and 2 belong to line g (a basis
@@ -231,22 +296,34 @@ __device__ __forceinline__ void store_frag(uint2* __restrict__ frag, int lane, c
 // x: the lane's eight entries, pairs (0,1) (2,3) (4,5) (6,7) of registers 0..3.
 struct LineScale {
     int E0 = 0, E1 = 0;
+    unsigned nz0 = 0, nz1 = 0;  // not zero: the lane has seen entries that are not zero
     // shift words of the entries; for the whole warp: 0 if all are at most 31,
     // bit 0 if some are larger, bit 1 if an entry exceeds its scale by more than
     // kOver bits
-    __device__ __forceinline__ unsigned shifts(const double (&x)[8], unsigned (&s)[8]) const {
+    __device__ __forceinline__ unsigned shifts(const double (&x)[8], unsigned (&s)[8]) {
         unsigned bits = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             s[k] = shift_word((k & 2) ? E1 : E0, x[k]);
             bits |= s[k] & 0x7e0u;
         }
-        if (!__any_sync(0xffffffffu, bits)) return 0;
+        if (!__any_sync(0xffffffffu, bits)) {
+            nz0 = nz1 = 1u;
+            return 0;
+        }
         bool over = false;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             over = over || (int)(((unsigned)__double2hiint(x[k]) >> 20) & 0x7ffu) > ((k & 2) ? E1 : E0) + kOver;
         return __any_sync(0xffffffffu, over) ? 3 : 1;
+    }
+    __device__ __forceinline__ void seen(const double (&x)[8]) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const unsigned any = ((unsigned)__double2hiint(x[k]) << 1) | (unsigned)__double2loint(x[k]);
+            if (k & 2) nz1 |= any;
+            else nz0 |= any;
+        }
     }
     __device__ __forceinline__ void raise(const double (&x)[8]) {
         int m0 = max(max(exp_bits(x[0]), exp_bits(x[1])), max(exp_bits(x[4]), exp_bits(x[5])));
@@ -264,28 +341,112 @@ struct LineScale {
     static __device__ __forceinline__ int limit(int E) { return E >= 0x7ff ? 0x7ff : max(kEmin, min(E, 0x7fd)); }
 };
 
+// 2^-d, d >= 0 (0 from d = 127 on)
+__device__ __forceinline__ float down2(int d) { return d < 127 ? __int_as_float((127 - d) << 23) : 0.0f; }
+
 // One step of 16 terms; flush() moves the accumulators to the sums at the old
-// scales (nothing before the first step).
+// scales (nothing before the first step).  settle: 64 terms since the last move to
+// integers, which is done here, between the cutting and the products: right after
+// the products it waits for the tensor cores (n = 6e5, b = 8, m = 720: update 1251 us,
+// here 1213).
 template <typename Flush>
 __device__ __forceinline__ void step(Acc& acc, LineScale& sc, const double (&x)[8], const uint2* __restrict__ frag,
-                                     int lane, bool first, Flush&& flush) {
+                                     int lane, bool settle, Flush&& flush) {
     unsigned s[8];
     Pair p[4];
+    const bool first = sc.E0 == 0;
     const unsigned how = first ? 3u : sc.shifts(x, s);
-    if (how == 0) {
+    if (how == 0) {  // no entry is zero
 #pragma unroll
         for (int r = 0; r < 4; ++r) p[r].template set<false>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
     } else {
         if (how & 2) {
             if (!first) flush();
+            const int e0 = sc.E0, e1 = sc.E1;
             sc.raise(x);
+            const float d0 = down2(sc.E0 - e0), d1 = down2(sc.E1 - e1);
+            acc.c[0] *= d0;
+            acc.c[1] *= d0;
+            acc.c[2] *= d1;
+            acc.c[3] *= d1;
 #pragma unroll
             for (int k = 0; k < 8; ++k) s[k] = shift_word((k & 2) ? sc.E1 : sc.E0, x[k]);
         }
+        sc.seen(x);
 #pragma unroll
         for (int r = 0; r < 4; ++r) p[r].template set<true>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
     }
+    if (settle) acc.to_int();
     mma_step(acc, p, frag, lane);
+}
+
+// the fields of the lane's lines as the sums 0, 1 and 2, 3 see them, 0 for a line of zeros
+__device__ __forceinline__ void line_fields(const LineScale& sc, int (&E)[2]) {
+    unsigned n0 = sc.nz0, n1 = sc.nz1;
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        n0 |= __shfl_xor_sync(0xffffffffu, n0, o);
+        n1 |= __shfl_xor_sync(0xffffffffu, n1, o);
+    }
+    E[0] = n0 ? sc.E0 : 0;
+    E[1] = n1 ? sc.E1 : 0;
+}
+
+// Which of the lane's four sums (bit e) the digits do not certify: a line and a
+// column that are not zero (fields not 0) with too small a Sigma, or one that is
+// not finite.
+__device__ __forceinline__ unsigned uncertified(const float (&c)[4], const int (&E)[2], int field0, int field1) {
+    unsigned bad = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int line = E[e >> 1], field = (e & 1) ? field1 : field0;
+        if ((line != 0 && field != 0 && !(c[e] >= kCertified)) || line >= 0x7ff || field >= 0x7ff) bad |= 1u << e;
+    }
+    return bad;
+}
+
+// The sums (bits of bad: sum e of this lane is that of line g + 8 (e / 2) and column 2t
+// + e % 2) formed again in FP64: term(line, column, k) gives a's and b's entry of
+// term k < terms.  A few sums are shared by the warp's lanes one after the other
+// (about 20 FP64 instructions each for 450 terms); of many, each lane forms its own.
+template <typename Term, typename Put>
+__device__ __forceinline__ void again(unsigned bad, int terms, Term&& term, Put&& put) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    if (__reduce_add_sync(0xffffffffu, __popc(bad)) > 48) {
+        double sum[4] = {0.0, 0.0, 0.0, 0.0};
+        if (bad) {
+            for (int k = 0; k < terms; ++k) {
+                double a[2], b[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) term(g + 8 * h, 2 * t + h, k, a[h], b[h]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sum[e] = fma(a[e >> 1], b[e & 1], sum[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (bad >> e & 1) put(e, sum[e]);
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        for (unsigned left = __ballot_sync(0xffffffffu, bad >> e & 1); left; left &= left - 1) {
+            const int who = __ffs(left) - 1;
+            double sum = 0.0;
+            for (int k0 = lane; k0 < terms; k0 += 128) {  // four terms' loads at once
+                double a[4], b[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    a[u] = b[u] = 0.0;
+                    if (k0 + 32 * u < terms) term((who >> 2) + 8 * (e >> 1), 2 * (who & 3) + (e & 1), k0 + 32 * u, a[u], b[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sum = fma(a[u], b[u], sum);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == who) put(e, sum);
+        }
 }
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool ok) {
@@ -304,12 +465,12 @@ __device__ __forceinline__ void cp_async_wait() {
 
 __device__ __forceinline__ double not_a_number() { return __longlong_as_double(0x7ff8000000000000ll); }
 
-// v: the sum over orders in units of order 3 (2^72); the scales of A and B are
+// v: the sum over orders in units of order 4 (2^64); the scales of A and B are
 // 2^(EA - 1078) and 2^(EB - 1078).  An entry that is not finite has the field
 // 0x7ff: its line's (column's) sums are NaN.
 __device__ __forceinline__ double unscale(double v, int ea, int eb) {
     if (ea >= 0x7ff || eb >= 0x7ff) return not_a_number();
-    return scale_by(v, 72 + ea + eb - 2156);
+    return scale_by(v, 64 + ea + eb - 2156);
 }
 
 // -------------------------------------------------------------------- C = Q^T W
@@ -337,7 +498,7 @@ __host__ __device__ inline int gram_parts(int ntiles) {
 }
 
 // Basis tiles tile0 .. tile0 + ntiles - 1 (16 columns each) of rows [r0, r0 +
-// rows) (at most 512) and columns c0 .. c0 + 7 of W: added to slot (m x B).
+// rows) (at most kMaxRows) and columns c0 .. c0 + 7 of W: added to slot (m x B).
 // All threads, after a barrier that follows the last use of smem and the zeroing
 // of slot and ew.
 template <int B>
@@ -360,7 +521,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
     const int og = g % B, og8 = (g + 8) % B;
     const int steps = (rows + 15) / 16;
     // the columns' scales, then the digits: a warp per step, a lane's four rows of column c0 + g
-    constexpr int SW = kMaxRows / 16 / kWarps;
+    constexpr int SW = (kMaxRows / 16 + kWarps - 1) / kWarps;
     {
         double xw[SW][4];
         int mx = 0;
@@ -370,7 +531,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
             for (int i = 0; i < 4; ++i) {
                 const int r = 16 * (warp + k * kWarps) + t + 4 * i;
                 xw[k][i] = (col && r < rows) ? __ldg(W + (r0 + r) * B + c0 + g) : 0.0;
-                mx = max(mx, exp_bits(xw[k][i]));
+                mx = max(mx, scale_field(xw[k][i]));
             }
 #pragma unroll
         for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -409,7 +570,6 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
 #pragma unroll
         for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
         Acc acc;
-        acc.clear();
         LineScale sc;
         double* mine = sums[warp] + lane;
 #pragma unroll
@@ -434,12 +594,25 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
                 x[k] = *reinterpret_cast<const double*>(buf + ob + r * B * 8 + swizzle<B>(r, og >> 1) * 16 + (og & 1) * 8);
                 x[k + 2] = *reinterpret_cast<const double*>(buf + ob8 + r * B * 8 + swizzle<B>(r, og8 >> 1) * 16 + (og8 & 1) * 8);
             }
-            step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
-            if (((s - s0) & 3) == 3) acc.to_int();
+            step(acc, sc, x, frag + s * kDig * 32, lane, s != s0 && ((s - s0) & 3) == 0, flush);
         }
         cp_async_wait<0>();
         __syncwarp();
         flush();
+        int E[2];
+        line_fields(sc, E);
+        const unsigned bad = uncertified(acc.c, E, ew[2 * t], ew[2 * t + 1]);
+        if (__any_sync(0xffffffffu, bad)) {
+            // (lines past the last basis column and columns past W's are zeros, which are certified)
+            again(bad, min(16 * s1, rows) - 16 * s0,
+                  [&](int line, int c, int k, double& a, double& b) {
+                      const int64_t r = r0 + 16 * s0 + k;
+                      const int j = 16 * tile + line;
+                      a = j < m ? Q[((int64_t)(j / B) * n + r) * B + j % B] : 0.0;
+                      b = c0 + c < B ? W[r * B + c0 + c] : 0.0;
+                  },
+                  [&](int e, double v) { mine[32 * e] = v; });
+        }
         if (parts == 1) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -492,7 +665,7 @@ __global__ void __launch_bounds__(kT, 2) gram_tc64_kernel(int64_t n, int m, int 
 }
 
 // Batch of problems stacked row-wise: CTA x takes chunk x, rows [chunks[3x+1],
-// chunks[3x+2]) of segment chunks[3x] (at most 512, never crossing a segment),
+// chunks[3x+2]) of segment chunks[3x] (at most kMaxRows, never crossing a segment),
 // into its own slot at partial[x * m * B]; m is read from device memory, chunks
 // of inactive segments do nothing.
 template <int B>
@@ -528,7 +701,7 @@ template <int B, bool SUB>
 __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, int tiles, int c0, int64_t row0,
                                              int64_t row_end,
                                              bool& staged, const double* Q, const double* __restrict__ C, double* W,
-                                             unsigned char* smem, int* ew, double (*part)[4][32]) {
+                                             unsigned char* smem, int* ew) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     double2* ring = reinterpret_cast<double2*>(smem + warp * kRing * kStepBytes) + lane;
     uint2* frag = reinterpret_cast<uint2*>(smem + kWarps * kRing * kStepBytes);
@@ -536,20 +709,25 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
     const bool col = c0 + g < kc;
     const int sub = warp % ks;  // ks warps share a tile of 16 rows, each a share of the steps
     // (a warp without a tile works on rows past the end)
-    const int64_t ra = warp / ks < tiles ? row0 + (warp / ks) * 16 + g : row_end, rb = ra + 8;
+    const int64_t rt = warp / ks < tiles ? row0 + (warp / ks) * 16 : row_end, ra = rt + g, rb = ra + 8;
     double out[4] = {0.0, 0.0, 0.0, 0.0};
+    Acc acc;
+    LineScale sc;
     for (int k0 = 0; k0 < m; k0 += kMaxCols) {
         const int cols = min(kMaxCols, m - k0), steps = (cols + 15) / 16;
         if (!staged) {
+            // the columns' scales grow from one staged piece of C to the next, as the lines' do
             __syncthreads();
-            if (tid < 8) ew[tid] = 0;
+            const int f0 = max(ew[2 * t], kEmin), f1 = max(ew[2 * t + 1], kEmin);
+            __syncthreads();
+            if (k0 == 0 && tid < 8) ew[tid] = 0;
             __syncthreads();
             int mx = 0;
             for (int s = warp; s < steps; s += kWarps)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int a = 16 * s + 2 * t + (i & 1) + 8 * (i >> 1);
-                    if (col && a < cols) mx = max(mx, exp_bits(C[(int64_t)(k0 + a) * kc + c0 + g]));
+                    if (col && a < cols) mx = max(mx, scale_field(C[(int64_t)(k0 + a) * kc + c0 + g]));
                 }
 #pragma unroll
             for (int o = 1; o <= 2; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -566,6 +744,11 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
                 store_frag(frag + s * kDig * 32, lane, x, eg);
             }
             __syncthreads();
+            const float d0 = down2(max(ew[2 * t] - f0, 0)), d1 = down2(max(ew[2 * t + 1] - f1, 0));
+            acc.c[0] *= d0;
+            acc.c[2] *= d0;
+            acc.c[1] *= d1;
+            acc.c[3] *= d1;
             staged = m <= kMaxCols;
         }
         // registers 0, 1: columns 2t, 2t+1 of rows g, g+8; 2, 3: columns 2t+8,
@@ -589,9 +772,6 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
         };
 #pragma unroll
         for (int k = 0; k < kRing - 1; ++k) issue(s0 + k);
-        Acc acc;
-        acc.clear();
-        LineScale sc;
         auto flush = [&]() {
             acc.to_int();
 #pragma unroll
@@ -609,21 +789,74 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
                 x[2 * i + 1] = v.y;
             }
             issue(s + kRing - 1);  // into the buffer of step s - 1
-            step(acc, sc, x, frag + s * kDig * 32, lane, s == s0, flush);
-            if (((s - s0) & 3) == 3) acc.to_int();
+            step(acc, sc, x, frag + s * kDig * 32, lane, s != s0 && ((s - s0) & 3) == 0, flush);
         }
         cp_async_wait<0>();
         if (s0 < s1) flush();
     }
-    if (ks > 1) {
+    int E[2];
+    line_fields(sc, E);
+    if (ks > 1) {  // the shares' sums, Sigmas and fields through the rings, which nobody uses any more
+        struct Share {
+            double out[4];
+            float c[4];
+            int E[2];
+        };
+        Share* shares = reinterpret_cast<Share*>(smem);
         __syncthreads();
+        Share& own = shares[tid];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) part[warp][e][lane] = out[e];
+        for (int e = 0; e < 4; ++e) {
+            own.out[e] = out[e];
+            own.c[e] = acc.c[e];
+        }
+        own.E[0] = E[0];
+        own.E[1] = E[1];
+        __syncthreads();
+        if (sub == 0) {
+            for (int q = 1; q < ks; ++q) {
+                const Share& o = shares[tid + 32 * q];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int top = max(E[h], o.E[h]);
+                    const float a = down2(top - E[h]), b = down2(top - o.E[h]);
+                    E[h] = top;
+#pragma unroll
+                    for (int e = 2 * h; e < 2 * h + 2; ++e) {
+                        acc.c[e] = acc.c[e] * a + o.c[e] * b;
+                        out[e] += o.out[e];
+                    }
+                }
+            }
+        }
         __syncthreads();
         if (sub != 0) return;
+    }
+    unsigned bad = uncertified(acc.c, E, ew[2 * t], ew[2 * t + 1]);
+    if (__any_sync(0xffffffffu, bad)) {
+        if (SUB) {  // the difference rounds by |W| as well, which counts towards Sigma
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            for (int q = 1; q < ks; ++q) out[e] += part[warp + q][e][lane];
+            for (int e = 0; e < 4; ++e) {
+                const int64_t r = (e & 2) ? rb : ra;
+                const int c = 2 * t + (e & 1), line = E[e >> 1], field = max(ew[c], kEmin);
+                if ((bad >> e & 1) && line < 0x7ff && field < 0x7ff && r < row_end && c0 + c < kc &&
+                    acc.c[e] + scale_by(fabs(W[r * kc + c0 + c]), 2156 - 96 - line - field) >= kCertified)
+                    bad &= ~(1u << e);
+            }
+        }
+        // (rows past the end and columns past C's are zeros, which are certified
+        // unless the other operand is not finite)
+        again(bad, m,
+              [&](int line, int c, int k, double& a, double& b) {
+                  const int64_t r = rt + line;
+                  a = r < row_end ? Q[((int64_t)(k / B) * n + r) * B + k % B] : 0.0;
+                  b = c0 + c < kc ? C[(int64_t)k * kc + c0 + c] : 0.0;
+              },
+              [&](int e, double v) {
+#pragma unroll
+                  for (int q = 0; q < 4; ++q)
+                      if (q == e) out[q] = v;
+              });
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -641,11 +874,10 @@ __global__ void __launch_bounds__(kT, 2) update_tc64_kernel(int64_t n, int m, in
                                                             const double* __restrict__ C, double* W) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
     __shared__ int ew[8];
-    __shared__ double part[kWarps][4][32];
     const int rows = 16 * tiles;
     bool staged = false;
     for (int64_t row0 = (int64_t)blockIdx.x * rows; row0 < n; row0 += (int64_t)gridDim.x * rows)
-        update_group<B, SUB>(n, m, kc, ks, tiles, blockIdx.y * 8, row0, n, staged, Q, C, W, tc_smem, ew, part);
+        update_group<B, SUB>(n, m, kc, ks, tiles, blockIdx.y * 8, row0, n, staged, Q, C, W, tc_smem, ew);
 }
 
 // Segmented: CTA x updates rows [ctas[3x+1], ctas[3x+2]) of segment s = ctas[3x]
@@ -659,14 +891,13 @@ __global__ void __launch_bounds__(kT, 2) update_tc64_seg_kernel(int64_t n, const
                                                                 double* W) {
     extern __shared__ __align__(16) unsigned char tc_smem[];
     __shared__ int ew[8];
-    __shared__ double part[kWarps][4][32];
     const int64_t seg = ctas[3 * blockIdx.x];
     if (seg_active && !seg_active[seg]) return;
     const int m = ms[seg * ms_stride];
     const int64_t r1 = ctas[3 * blockIdx.x + 2];
     bool staged = false;
     for (int64_t row0 = ctas[3 * blockIdx.x + 1]; row0 < r1; row0 += 16 * kWarps)
-        update_group<B, true>(n, m, B, 1, kWarps, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew, part);
+        update_group<B, true>(n, m, B, 1, kWarps, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew);
 }
 
 int sms() {
@@ -692,7 +923,8 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
     }
     constexpr int NH = (B + 7) / 8;
     // One chunk per resident CTA where that gives at least 64 rows, at most the
-    // staged 512; with fewer than 512 rows the tiles are split into groups of
+    // staged kMaxRows, else chunks of equal size for several rounds; with fewer
+    // rows the tiles are split into groups of
     // one per warp, which take more rows each (an item's end, its FP64
     // conversions, costs as much as three steps).  n = 2e4, b = 4, m = 400: 36.7 us
     // in one group, 33.4 in four; m = 200: 21.2 and 21.0.
@@ -702,7 +934,8 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
     groups = std::max<int64_t>(std::min<int64_t>(groups, kMaxRows * resident / std::max<int64_t>(n, 1)), 1);
     const int per_group = (int)ceil_div(ntiles, groups);
     groups = ceil_div(ntiles, per_group);
-    const int64_t rc = std::min<int64_t>(std::max<int64_t>(ceil_div(ceil_div(n * groups, resident), 16) * 16, 64), kMaxRows);
+    const int64_t rounds = ceil_div(ceil_div(n * groups, resident), kMaxRows);
+    const int64_t rc = std::max<int64_t>(ceil_div(ceil_div(n * groups, resident * rounds), 16) * 16, 64);
     const int64_t chunks = ceil_div(n, rc) * groups;
     const int64_t ctas = std::min<int64_t>(chunks, resident);
     const int64_t per = (int64_t)m * B;
@@ -790,8 +1023,8 @@ bbl_status launch_update_seg(int64_t n, const int* ms, int ms_stride, const int6
 
 }  // namespace
 
-// (the chunks of a segmented Gram hold at most 512 rows)
 bool tc64_seg_supports(int b) { return b == 4 || b == 8; }
+int tc64_seg_chunk_rows() { return kMaxRows; }
 
 bbl_status gram_tc64_seg(int64_t n, int b, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
                          int nchunks, const int* active, double* partial, cudaStream_t st) {
