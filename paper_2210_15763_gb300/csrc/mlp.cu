@@ -109,13 +109,13 @@ __device__ __forceinline__ float row_dot16(const __nv_bfloat16* __restrict__ Wro
     return warp_sum16(acc);
 }
 
-// h1 of 16 samples (recomputed by every CTA; the first column of CTAs stores
+// h1 of 16 samples (recomputed by every CTA; the first row of CTAs stores
 // it), then z2 and h2 of 8 rows
 __global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, int O, const float* __restrict__ P,
                                                             const __nv_bfloat16* __restrict__ Wb,
                                                             const float* __restrict__ g, float* __restrict__ act) {
     extern __shared__ float sh[];
-    const int s0 = blockIdx.y * kFwS, ns = min(kFwS, batch - s0);
+    const int s0 = blockIdx.x * kFwS, ns = min(kFwS, batch - s0);
     const size_t st = 6 * H + 2 * O;
     const float* b1 = P + H;
     const float* b2 = P + 2 * H + H * H;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, in
         if (q < ns) {
             const float z = fmaf(bf(Wb, i), g[s0 + q], b1[i]);
             hv = gelu(z);
-            if (blockIdx.x == 0) {
+            if (blockIdx.y == 0) {
                 act[(s0 + q) * st + i] = z;
                 act[(s0 + q) * st + H + i] = hv;
             }
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, in
         sh[e] = hv;
     }
     __syncthreads();
-    const int o = blockIdx.x * kFwWarps + (threadIdx.x >> 5);
+    const int o = blockIdx.y * kFwWarps + (threadIdx.x >> 5);
     if (o >= H) return;
     const float z = row_dot16(Wb + H + (size_t)o * H, sh, H) + b2[o];
     const int q = (threadIdx.x & 31) >> 1;
@@ -152,14 +152,14 @@ __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, in
                                                             float* __restrict__ lossp) {
     extern __shared__ float sh[];
     __shared__ float red[kFwWarps];
-    const int s0 = blockIdx.y * kFwS, ns = min(kFwS, batch - s0);
+    const int s0 = blockIdx.x * kFwS, ns = min(kFwS, batch - s0);
     const size_t st = 6 * H + 2 * O;
     for (int e = threadIdx.x; e < kFwS * H; e += kFwThreads) {
         const int q = e / H, i = e - q * H;
         sh[e] = q < ns ? act[(s0 + q) * st + 3 * H + i] : 0.0f;
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, o = blockIdx.x * kFwWarps + warp;
+    const int warp = threadIdx.x >> 5, o = blockIdx.y * kFwWarps + warp;
     float l = 0.0f;
     if (o < O) {
         const float y = row_dot16(Wb + H + H * H + (size_t)o * H, sh, H) + P[3 * H + H * H + O * H + o];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, in
     if (threadIdx.x == 0) {
         float t = 0.0f;
         for (int w = 0; w < kFwWarps; ++w) t += red[w];
-        lossp[blockIdx.y * gridDim.x + blockIdx.x] = t;
+        lossp[blockIdx.x * gridDim.y + blockIdx.y] = t;
     }
 }
 
@@ -397,11 +397,11 @@ bbl_status launch_forward(const bbl_mlp* M, int batch, const float* g, float* y,
         BBL_CUDA(cudaFuncSetAttribute(output_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwS * 1024 * 4));
         attr = true;
     }
-    const unsigned groups = (unsigned)ceil_div(batch, kFwS);
-    hidden_kernel<<<dim3((unsigned)ceil_div(H, kFwWarps), groups), kFwThreads, sm, st>>>(
+    const unsigned groups = (unsigned)ceil_div(batch, kFwS);  // in x: any batch (y holds 65535 at most, rows 512)
+    hidden_kernel<<<dim3(groups, (unsigned)ceil_div(H, kFwWarps)), kFwThreads, sm, st>>>(
         batch, H, O, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), g, M->act.as<float>());
     BBL_LAUNCH_CHECK();
-    output_kernel<<<dim3((unsigned)ceil_div(O, kFwWarps), groups), kFwThreads, sm, st>>>(
+    output_kernel<<<dim3(groups, (unsigned)ceil_div(O, kFwWarps)), kFwThreads, sm, st>>>(
         batch, H, O, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), M->act.as<float>(), y, target,
         M->lossbuf.as<float>() + 8);
     BBL_LAUNCH_CHECK();

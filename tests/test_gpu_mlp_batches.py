@@ -1,0 +1,36 @@
+"""MLP calls at batches beyond 16 x 65535 samples (one grid dimension's limit)."""
+import numpy as np
+import pytest
+
+from oracle import mlp as OM
+from tests.gpu_util import need_gpu, to_dev
+from tests.test_gpu_learned import _setup, pack, unpack
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch", [1048560, 1048561, 1100003])
+def test_large_batch(batch):
+    torch, bbl = need_gpu()
+    H, O = 4, 3
+    p, g, tgt = _setup(H, O, 64, seed=7)
+    reps, rest = batch // 64, batch % 64
+    G, T = np.concatenate([np.tile(g, reps), g[:rest]]), np.concatenate([np.tile(tgt, (reps, 1)), tgt[:rest]])
+    net = bbl.MLP(H, O)
+    net.set_params(pack(p))
+    y = net.forward(to_dev(torch, G, torch.float32)).cpu().numpy()
+    small = net.forward(to_dev(torch, g, torch.float32)).cpu().numpy()
+    assert (y == np.concatenate([np.tile(small, (reps, 1)), small[:rest]])).all()
+    loss = net.loss_grad(to_dev(torch, G, torch.float32), to_dev(torch, T, torch.float32))
+    # means over the repeated samples
+    yr, c = OM.forward(p, g)
+    w = np.full(64, reps / batch) + (np.arange(64) < rest) / batch
+    d = yr - tgt
+    assert loss == pytest.approx(float((w[:, None] * d * d).sum() / O), rel=1e-4)
+    got = unpack(net.get_params()[1], H, O)
+    dy = 2.0 * w[:, None] * d / O
+    # FP32 sums of `batch` products in turn: batch 2^-25 of the sum of the magnitudes
+    # where all roundings of the repeated terms agree
+    tol = batch * 2.0 ** -25 + 1e-3
+    assert (np.abs(got["W3"] - dy.T @ c["h2"]) <= tol * (np.abs(dy).T @ np.abs(c["h2"]))).all()
+    assert (np.abs(got["b3"] - dy.sum(axis=0)) <= tol * np.abs(dy).sum(axis=0)).all()
