@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, in
 }
 
 // y of 8 output rows for 16 samples; with a target also dy = 2 (y - t) / N and
-// the CTA's partial loss
+// the CTA's part of the mean loss
 __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, int O, const float* __restrict__ P,
                                                             const __nv_bfloat16* __restrict__ Wb,
                                                             float* __restrict__ act, float* __restrict__ y_out,
@@ -170,8 +170,9 @@ __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, in
             if (y_out) y_out[(size_t)(s0 + q) * O + o] = y;
             if (target) {
                 const float d = y - target[(size_t)(s0 + q) * O + o];
-                a[6 * H + O + o] = 2.0f * d * (1.0f / ((float)batch * (float)O));
-                l = d * d;
+                const float inv = 1.0f / ((float)batch * (float)O);
+                a[6 * H + O + o] = 2.0f * d * inv;
+                l = d * d * inv;  // the mean's term: a sum of squares could overflow where the mean does not
             }
         }
     }
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(256) backward_w_kernel(int batch, int H, int O
             if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
             __syncthreads();
         }
-        if (threadIdx.x == 0) *loss = red[0] * (1.0f / ((float)batch * (float)O));
+        if (threadIdx.x == 0) *loss = red[0];
         return;
     }
     const int np = 3 * H + H * H + O * H + O;

@@ -34,3 +34,17 @@ def test_large_batch(batch):
     tol = batch * 2.0 ** -25 + 1e-3
     assert (np.abs(got["W3"] - dy.T @ c["h2"]) <= tol * (np.abs(dy).T @ np.abs(c["h2"]))).all()
     assert (np.abs(got["b3"] - dy.sum(axis=0)) <= tol * np.abs(dy).sum(axis=0)).all()
+
+
+@pytest.mark.parametrize("H,O,batch", [(4, 32, 64), (8, 3, 40), (16, 300, 5)])
+def test_loss_of_large_differences(H, O, batch):
+    """The mean is finite although the sum of the squares is not (FP32)."""
+    torch, bbl = need_gpu()
+    p, g, _ = _setup(H, O, batch, seed=2)
+    r = np.random.default_rng(1)
+    tgt = (r.uniform(0.8, 1.0, (batch, O)) * 1.2e18).astype(np.float32)
+    net = bbl.MLP(H, O)
+    net.set_params(pack(p))
+    loss = net.loss_grad(to_dev(torch, g, torch.float32), torch.from_numpy(tgt).cuda())
+    # squares, scaling and a sum of at most 1500 terms by trees: 2^-24 each
+    assert loss == pytest.approx(float((tgt.astype(np.float64) ** 2).mean()), rel=20 * 2.0 ** -24)
