@@ -376,9 +376,9 @@ int loss_parts(const bbl_mlp* M, int batch) {
 
 bbl_status ensure_batch(bbl_mlp* M, int batch) {
     if (batch <= M->cap_batch) return BBL_OK;
-    BBL_TRY(M->act.alloc(sizeof(float) * (size_t)batch * (6 * M->hidden + 2 * M->out)));
-    BBL_TRY(M->lossbuf.alloc(sizeof(float) * (size_t)(loss_parts(M, batch) + 8)));  // the loss, then its parts
-    M->cap_batch = batch;
+    // the buffers go before the larger ones come: until both are there, no
+    // capacity and no captured graph that points to them
+    M->cap_batch = 0;
     if (M->exec) {
         cudaGraphExecDestroy(M->exec);
         cudaGraphDestroy(M->graph);
@@ -386,6 +386,9 @@ bbl_status ensure_batch(bbl_mlp* M, int batch) {
         M->graph = nullptr;
         M->graph_batch = -1;
     }
+    BBL_TRY(M->act.alloc(sizeof(float) * (size_t)batch * (6 * M->hidden + 2 * M->out)));
+    BBL_TRY(M->lossbuf.alloc(sizeof(float) * (size_t)(loss_parts(M, batch) + 8)));  // the loss, then its parts
+    M->cap_batch = batch;
     return BBL_OK;
 }
 

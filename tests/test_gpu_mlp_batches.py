@@ -48,3 +48,17 @@ def test_loss_of_large_differences(H, O, batch):
     loss = net.loss_grad(to_dev(torch, g, torch.float32), torch.from_numpy(tgt).cuda())
     # squares, scaling and a sum of at most 1500 terms by trees: 2^-24 each
     assert loss == pytest.approx(float((tgt.astype(np.float64) ** 2).mean()), rel=20 * 2.0 ** -24)
+
+
+def test_a_batch_beyond_the_memory_leaves_the_network_usable():
+    torch, bbl = need_gpu()
+    p, g, tgt = _setup(1024, 8, 6, seed=3)
+    net = bbl.MLP(1024, 8)
+    net.set_params(pack(p))
+    x, t = to_dev(torch, g, torch.float32), to_dev(torch, tgt, torch.float32)
+    want = net.forward(x).cpu().numpy()
+    net.train(x, t, 1, 1e-12)
+    with pytest.raises(bbl.BBLError, match="OOM"):  # 40 TB of activations; refused before x is read
+        bbl._lib.check(bbl._lib.load().bbl_mlp_forward(net.handle, 1600000000, x.data_ptr(), x.data_ptr(), None))
+    np.testing.assert_allclose(net.forward(x).cpu().numpy(), want, atol=1e-5)
+    net.train(x, t, 1, 1e-12)
