@@ -1566,10 +1566,10 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
 // -------------------------------------------------------------------- Cholesky of the b x b Gram
 // status bits: 1 = non-finite Gram.  mask[i] = 1 for deflated columns.
 
-// 1 / d of a normal finite d, to about one unit in the last place: an FP32
-// seed on the mantissa and two Newton steps (four FP64 instructions in a chain;
-// an FP64 instruction occupies its scheduler for 64 cycles here, and the
-// division takes about ten).
+// 1 / d, rounded as the division rounds it but for one case in about 2^39: an FP32
+// seed on the mantissa and two Newton steps, the last from an error below 2^-45
+// (four FP64 instructions in a chain; an FP64 instruction occupies its scheduler
+// for 64 cycles here, and the division takes about ten).
 __device__ __forceinline__ double recip(double d) {
     const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
     if (ex < 64 || ex > 1980) return 1.0 / d;
@@ -1632,7 +1632,9 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
         const double d = ra[k];
         const int defl = !(d > thresh2) || bad;
         cnt += defl;
-        const double y = defl ? 0.0 : recip(d);
+        // a pivot whose reciprocal is not a normal number divides instead
+        const bool whole = d > 0x1p-1020 && d < 0x1p1020;
+        const double y = defl || !whole ? 0.0 : recip(d);
         if (lane == 0) {
             sh.deflated[k] = defl;
             sh.d[k] = defl ? 0.0 : d;
@@ -1644,7 +1646,7 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
 #pragma unroll
         for (int x = 0; x < E; ++x) {
             if (32 * x < bb && ei[x] > k) {
-                const double l = ra[ei[x]] * y;
+                const double l = whole || defl ? ra[ei[x]] * y : ra[ei[x]] / d;
                 if (!defl && ec[x] >= ei[x]) a[x] = fma(-l, ra[ec[x]], a[x]);
                 if (!defl && ec[x] <= k) z[x] = fma(-l, rz[ec[x]], z[x]);
                 if (ei[x] == k + 1) {
