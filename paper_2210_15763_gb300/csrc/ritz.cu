@@ -5,7 +5,7 @@
 //
 // Isolated eigenvalues are computed by slicing and block cyclic reduction
 // (ritz_cr.cu); the sequential kernels here run for bands that path does not
-// take (ritz_cr_supports) and for segments it could not certify (degenerate
+// take (ritz_cr_supports) and for the pairs it could not certify (degenerate
 // or nearly degenerate values), and otherwise return at once:
 //  1. bisect  - one CTA per wanted eigenvalue index i.  Sylvester's law of
 //               inertia: the number of negative pivots of the LDL^T
@@ -296,9 +296,9 @@ __global__ void __launch_bounds__(256) bisect_lane_kernel(int m, int nev, const 
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
-    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
+    if (sa.need && !sa.need[seg * nev + i]) return;
     Tg += seg * sa.sT;
     theta_out += seg * sa.sTh;
     width_out += seg * sa.sTh;
@@ -341,8 +341,13 @@ __global__ void __launch_bounds__(256) bisect_lane_kernel(int m, int nev, const 
     const float pivmindf = (float)(1e-13 * scale);
     const double glo = s_lo, ghi = s_hi;
     double lo = glo, hi = ghi;
-    const bool warm_used = warm && i < warm_count;
-    if (warm_used) {
+    const double* guess = sa.guess ? sa.guess + 2 * (seg * nev + i) : nullptr;
+    const bool guessed = guess && guess[0] < guess[1];  // the fast path's bracket
+    const bool warm_used = guessed || (warm && i < warm_count);
+    if (guessed) {
+        lo = fmax(glo, guess[0]);
+        hi = fmin(ghi, guess[1]);
+    } else if (warm_used) {
         const double w = warm[i];
         hi = fmin(ghi, w + 1e-9 * scale);
         lo = fmax(glo, w - 1e-3 * scale);
@@ -477,9 +482,9 @@ __global__ void __launch_bounds__(32 * kBisectWarps) bisect_kernel(int m, int p,
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
-    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
+    if (sa.need && !sa.need[seg * nev + i]) return;
     Tg += seg * sa.sT;
     theta_out += seg * sa.sTh;
     width_out += seg * sa.sTh;
@@ -526,7 +531,12 @@ __global__ void __launch_bounds__(32 * kBisectWarps) bisect_kernel(int m, int p,
     const double pivmin32 = 1e-7 * scale;
     const double glo = s_lo, ghi = s_hi;
     double lo = glo, hi = ghi;
-    if (warm && i < warm_count) {
+    const double* guess = sa.guess ? sa.guess + 2 * (seg * nev + i) : nullptr;
+    const bool guessed = guess && guess[0] < guess[1];  // the fast path's bracket
+    if (guessed) {
+        lo = fmax(glo, guess[0]);
+        hi = fmin(ghi, guess[1]);
+    } else if (warm && i < warm_count) {
         // T of an earlier block is a leading principal submatrix of this T, so
         // its i-th Ritz value bounds this one from above (Cauchy interlacing);
         // a guessed lower end is checked with the final FP64 counts below
@@ -544,7 +554,7 @@ __global__ void __launch_bounds__(32 * kBisectWarps) bisect_kernel(int m, int p,
     // counts at its ends (warp 0 at lo, warp 1 at hi).  A warm bracket that
     // fails the check (the value moved further down than guessed) is retried
     // once from the Gershgorin interval.
-    const bool warm_used = warm && i < warm_count && !(lo == glo && hi == ghi);
+    const bool warm_used = guessed || (warm && i < warm_count && !(lo == glo && hi == ghi));
     bool verified = false;
     for (int attempt = 0; attempt < (warm_used ? 2 : 1) && !verified; ++attempt) {
         if (attempt == 1) {
@@ -625,9 +635,9 @@ __global__ void __launch_bounds__(32) invit_kernel(int m, int p, const double* _
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
-    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
+    if (sa.need && !sa.need[seg * nev + i]) return;
     Tg += seg * sa.sT;
     theta += seg * sa.sTh;
     S += seg * sa.sS;
@@ -813,9 +823,9 @@ __global__ void __launch_bounds__(32) invit_df_kernel(int m, const double* __res
     const int i = blockIdx.x;
     const int seg = blockIdx.y;
     if (sa.active && !sa.active[seg]) return;
-    if (sa.need && !sa.need[seg]) return;
     if (sa.d_m) m = *sa.d_m;
     if (i >= min(nev, m)) return;
+    if (sa.need && !sa.need[seg * nev + i]) return;
     Tg += seg * sa.sT;
     theta += seg * sa.sTh;
     S += seg * sa.sS;
@@ -1053,9 +1063,10 @@ __global__ void __launch_bounds__(256) cluster_kernel(int m, int p, int ldS, con
     __shared__ unsigned long long s_scale_bits;
     const int seg = blockIdx.x;
     if (sa.active && !sa.active[seg]) return;
-    const bool certified = sa.need && !sa.need[seg];
     if (sa.d_m) m = *sa.d_m;
     const int nev = min(ldS, m);  // columns computed; S keeps row stride ldS
+    bool certified = sa.need != nullptr;  // all pairs
+    for (int k = 0; k < nev && certified; ++k) certified = sa.need[seg * ldS + k] == 0;
     Tb += seg * sa.sT;
     theta += seg * sa.sTh;
     S += seg * sa.sS;
@@ -1358,9 +1369,9 @@ bbl_status ritz_dev(int m, int p, int nev, const double* Tb, double* theta, doub
     BBL_TRY(set_ritz_attrs());
     SegArgs one{nullptr, nullptr, 0, 0, 0, 0, 0};
     if (ritz_cr_supports(m, p)) {
-        int* flag = nullptr;
-        BBL_TRY(ritz_cr(m, p, nev, 1, Tb, theta, S, ws, fast, &flag, one, st));
-        one.need = flag;
+        SegArgs rest = one;
+        BBL_TRY(ritz_cr(m, p, nev, 1, Tb, theta, S, ws, fast, &rest, one, st));
+        one = rest;
     }
     BBL_TRY(launch_bisect(dim3(nev), m, p, nev, Tb, theta, width, band_smem, band_bytes, one, warm, warm_count, st));
     BBL_TRY(launch_invit(dim3(nev), m, p, nev, Tb, theta, S, ws, one, st));
@@ -1394,9 +1405,9 @@ bbl_status ritz_dev_batched(int m_max, int p, int nev, int nseg, const double* T
     SegArgs sa{d_m, active, sT, sTh, sS, sWs, (int64_t)m_max * nev};
     if (ritz_cr_supports(m_max, p)) {
         void* fast = reinterpret_cast<char*>(ws) + ((sizeof(double) * (size_t)nseg * (size_t)sWs + 255) & ~size_t(255));
-        int* flag = nullptr;
-        BBL_TRY(ritz_cr(m_max, p, nev, nseg, Tb, theta, S, ws, fast, &flag, sa, st));
-        sa.need = flag;
+        SegArgs rest = sa;
+        BBL_TRY(ritz_cr(m_max, p, nev, nseg, Tb, theta, S, ws, fast, &rest, sa, st));
+        sa = rest;
     }
     dim3 g(nev, nseg);
     BBL_TRY(launch_bisect(g, m_max, p, nev, Tb, theta, width, band_smem, band_bytes, sa, nullptr, 0, st));

@@ -32,8 +32,8 @@
 // sigma0, the value lies in its bracket, the bracket holds one eigenvalue
 // and the FP64 residual is at most 1e-14 of the spectrum.  Otherwise
 // (degenerate or nearly degenerate values, extreme pivots, non-finite
-// input) need[seg] is set and the sequential kernels of ritz.cu compute the
-// segment as before.
+// input) its need flag is set and the sequential kernels of ritz.cu compute the
+// pair as before, from the bracket found here.
 #include <algorithm>
 
 #include "ritz.cuh"
@@ -76,7 +76,8 @@ struct Bracket1 {
 
 struct Lay {  // fast-path workspace
     Hdr* hdr;          // nseg
-    int* need;         // nseg
+    int* need;         // nseg x nev
+    double* guess;     // nseg x nev x 2
     Bracket1* br;      // nseg x nev
     int* c1;           // nseg x kMaxNs1
     int* c2;           // nseg x nev x kNs2
@@ -94,13 +95,15 @@ size_t layout(int m, int p, int nev, int nseg, void* base, Lay* l) {
     const int P = slice_width(p);
     const size_t bs = ((size_t)padded_rows(m, P) * (P + 1) + 3) & ~size_t(3);
     const size_t o1 = round256(sizeof(Hdr) * nseg);
-    const size_t o2 = o1 + round256(sizeof(int) * nseg);
+    const size_t og = o1 + round256(sizeof(int) * (size_t)nseg * nev);
+    const size_t o2 = og + round256(sizeof(double) * 2 * (size_t)nseg * nev);
     const size_t o3 = o2 + round256(sizeof(Bracket1) * (size_t)nseg * nev);
     const size_t o4 = o3 + round256(sizeof(int) * (size_t)nseg * kMaxNs1);
     const size_t o5 = o4 + round256(sizeof(int) * (size_t)nseg * nev * kNs2);
     if (l) {
         l->hdr = reinterpret_cast<Hdr*>(q);
         l->need = reinterpret_cast<int*>(q + o1);
+        l->guess = reinterpret_cast<double*>(q + og);
         l->br = reinterpret_cast<Bracket1*>(q + o2);
         l->c1 = reinterpret_cast<int*>(q + o3);
         l->c2 = reinterpret_cast<int*>(q + o4);
@@ -132,10 +135,11 @@ __device__ __forceinline__ bool in_band(int r, int d, int p) { return d <= p && 
 
 // The scaled band in FP32 (rows of P + 1 entries, columns past p zero; rows
 // m .. mp - 1 are padding, decoupled, with a large diagonal), its Gershgorin
-// interval, and need = 0.  One CTA per segment: done once, the slices and
+// interval, and need = 0 (1 if a band is not finite).  One CTA per segment: done once, the slices and
 // the reduction then copy FP32 rows.
-__global__ void __launch_bounds__(kPrepThreads) prep_kernel(int m, int p, int P, const double* __restrict__ Tg,
+__global__ void __launch_bounds__(kPrepThreads) prep_kernel(int m, int p, int P, int nev, const double* __restrict__ Tg,
                                                             Hdr* __restrict__ hdr, int* __restrict__ need,
+                                                            double* __restrict__ guess,
                                                             float* __restrict__ band, int64_t band_stride,
                                                             SegArgs sa) {
     __shared__ unsigned s_mx;
@@ -206,7 +210,10 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(int m, int p, int P,
         h.e = e;
         h.ok = ok ? 1 : 0;
         hdr[seg] = h;
-        need[seg] = ok ? 0 : 1;
+    }
+    if (tid < nev) {
+        need[seg * nev + tid] = ok ? 0 : 1;
+        guess[2 * (seg * nev + tid)] = guess[2 * (seg * nev + tid) + 1] = 0.0;  // no bracket
     }
 }
 
@@ -714,7 +721,8 @@ __global__ void __launch_bounds__(kVecThreads) vec_kernel(int m, int p, int nev,
                                                           const float* __restrict__ band, int64_t band_stride,
                                                           double* __restrict__ ws, int64_t ws_stride,
                                                           double* __restrict__ theta, double* __restrict__ S,
-                                                          int* __restrict__ need, SegArgs sa) {
+                                                          int* __restrict__ need, double* __restrict__ guess,
+                                                          SegArgs sa) {
     constexpr int BB = BS * BS;
     extern __shared__ __align__(16) unsigned char vk_smem[];
     __shared__ double red64[kVecWarps];
@@ -866,7 +874,11 @@ __global__ void __launch_bounds__(kVecThreads) vec_kernel(int m, int p, int nev,
         near_val = near_val && !good && val > (double)lo - (double)margin && val <= (double)hi + (double)margin;
     }
     if (!good) {
-        if (tid == 0) atomicOr(need + seg, 1);
+        if (tid == 0) {
+            need[seg * nev + i] = 1;
+            guess[2 * (seg * nev + i)] = ldexp((double)lo - 1e-6 * h.scale, h.e);
+            guess[2 * (seg * nev + i) + 1] = ldexp((double)hi + 1e-6 * h.scale, h.e);
+        }
         return;
     }
     // unit vector; the first entry of largest magnitude is positive
@@ -936,7 +948,7 @@ bbl_status launch_vec(int m, int p, int nev, int nseg, const double* Tb, double*
     }
     vec_kernel<BS><<<dim3(nev, nseg), kVecThreads, vecs + (in_smem ? mats : 0), st>>>(
         m, p, nev, Tb, in_smem, l.hdr, l.br, l.c2, l.band, l.band_stride, ws, (int64_t)ritz_cr_vec_doubles(m, p), theta, S,
-        l.need, sa);
+        l.need, l.guess, sa);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
 }
@@ -954,11 +966,12 @@ bool ritz_cr_supports(int m, int p) {
 }
 
 bbl_status ritz_cr(int m, int p, int nev, int nseg, const double* Tb, double* theta, double* S, double* ws, void* fast,
-                   int** need, SegArgs sa, cudaStream_t st) {
+                   SegArgs* out, SegArgs sa, cudaStream_t st) {
     Lay l;
     layout(m, p, nev, nseg, fast, &l);
-    *need = l.need;
-    prep_kernel<<<nseg, kPrepThreads, 0, st>>>(m, p, slice_width(p), Tb, l.hdr, l.need, l.band, l.band_stride, sa);
+    out->need = l.need;
+    out->guess = l.guess;
+    prep_kernel<<<nseg, kPrepThreads, 0, st>>>(m, p, slice_width(p), nev, Tb, l.hdr, l.need, l.guess, l.band, l.band_stride, sa);
     BBL_LAUNCH_CHECK();
     switch (slice_width(p)) {
         case 1: BBL_TRY(launch_slices<1>(m, nev, nseg, l, sa, st)); break;
