@@ -30,7 +30,7 @@
 //
 // A pair is accepted when the reduction counts exactly i eigenvalues below
 // sigma0, the value lies in its bracket, the bracket holds one eigenvalue
-// and the FP64 residual is at most 1e-14 of the spectrum.  Otherwise
+// and the FP64 residual is at most 1e-15 of the Gershgorin bound.  Otherwise
 // (degenerate or nearly degenerate values, extreme pivots, non-finite
 // input) its need flag is set and the sequential kernels of ritz.cu compute the
 // pair as before, from the bracket found here.
@@ -54,6 +54,7 @@ constexpr int kMaxNs1 = 4096, kNs2 = 512;
 constexpr int kSolvesF32 = 3;        // inverse iterations before the FP64 corrections
 constexpr int kMaxCorr = 8;          // FP64 corrections with one factorisation
 constexpr int kMaxTries = 3;         // factorisations (shifts) per eigenvalue
+constexpr float kAccepted = 1e-15f;  // residual of an accepted pair, relative to the Gershgorin bound
 
 // Shifts of the first round: one problem spreads over the GPU; many segments
 // share it (the second round then resolves 512 times finer).
@@ -769,6 +770,10 @@ __global__ void __launch_bounds__(kVecThreads) vec_kernel(int m, int p, int nev,
     // value in the scaled units; close enough at the start that the residual
     // y - val x carries the Rayleigh quotient's correction in FP32
     double val = 0.5 * ((double)lo + (double)hi);
+    // The sequential kernels leave 2e-15 to 4e-15 with their float-float factors
+    // (p = 1, 2, 4, 8) and 1e-16 to 3e-16 with FP64 ones, so there the corrections go on
+    // until the residual stalls (30 random bands per p: at most 4.6e-16 and 2.3e-16).
+    const float done = p == 1 || p == 2 || p == 4 || p == 8 ? 4e-16f : 0.0f;
     bool good = false, near_val = false;  // near_val: x and val are a pair to 1e-6
     for (int tries = 0; tries < kMaxTries && single && !good; ++tries) {
         // FP32 counts are those of a matrix within about 5e-7 of T: below the
@@ -858,8 +863,8 @@ __global__ void __launch_bounds__(kVecThreads) vec_kernel(int m, int p, int nev,
             near_val = rel <= 1e-6f;
             if (!(rel < 1e30f)) break;  // not a number
             // at FP64 rounding, or no longer falling by 4: judged by its size
-            if (rel <= 4e-16f || (it > 0 && rel > 0.25f * prev)) {
-                good = rel <= 1e-14f;
+            if (rel <= done || (it > 0 && rel > 0.25f * prev)) {
+                good = rel <= kAccepted;
                 break;
             }
             prev = rel;
