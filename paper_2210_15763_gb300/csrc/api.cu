@@ -25,6 +25,16 @@ void clear_error() { g_last_error.clear(); }
 static std::atomic<unsigned long long> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+int sm_count() {
+    static std::atomic<int> known[64];  // 0: not asked yet
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 152;
+    if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 152;
+    if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 bool is_device_pointer(const void* p) {
     if (!p) return false;
     cudaPointerAttributes at;

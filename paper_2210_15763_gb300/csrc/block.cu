@@ -858,16 +858,6 @@ __global__ void __launch_bounds__(kThreads) qr_pass_kernel(int64_t n, const doub
     }
 }
 
-int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    }
-    return n;
-}
-
 // Column groups of the split-K Gram for m basis columns: each thread of a
 // CTA owns CPT columns, so a group covers up to kThreads * CPT columns, and
 // each group has its own chunk ticket.
@@ -896,9 +886,10 @@ bbl_status gram_core(int64_t n, int m, const T* Q, const T* W, double* C, double
     // the buffer only for the reduction over row slots
     const size_t smem_max = sizeof(double) * kThreads * CPT * B;
     const size_t smem = (RS > 1 || sizeof(T) == 4) ? smem_max : 0;
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_kernel<T, B, CPT>, smem_max));
     static int occ = 0;
     if (occ == 0) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_kernel<T, B, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
         BBL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gram_kernel<T, B, CPT>, kThreads, smem_max));
         if (occ < 1) occ = 1;
     }
@@ -923,10 +914,10 @@ bbl_status gram_core(int64_t n, int m, const T* Q, const T* W, double* C, double
 template <typename T, int B>
 bbl_status launch_gram_rows(int64_t n, int m, const T* Q, const T* W, double* C, DevBuf& partials, cudaStream_t st) {
     using S = GramRowsShape<T, B>;
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_rows_kernel<T, B>, S::smem_bytes));
     static int occ = 0;
     if (occ == 0) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_rows_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)S::smem_bytes));
         BBL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gram_rows_kernel<T, B>, kThreads, S::smem_bytes));
         if (occ < 1) occ = 1;
     }
@@ -1165,11 +1156,8 @@ bbl_status launch_gram_generic(int64_t n, int m, int b, const T* Q, const T* W, 
     const size_t need = sizeof(double) * (size_t)nch * m * b;
     BBL_TRY(partials.grow(need));
     const size_t smem = sizeof(double) * kThreads * kMaxB;
-    static bool attr_set = false;
-    if (!attr_set) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_generic_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr_set = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_generic_kernel<T>, smem));
     dim3 grid((unsigned)nch, (unsigned)gy);
     gram_generic_kernel<T><<<grid, kThreads, smem, st>>>(n, m, b, rpc, TC, Q, W, partials.as<double>());
     BBL_LAUNCH_CHECK();
@@ -1981,12 +1969,8 @@ template <typename T, int B>
 bbl_status launch_gram_rows_seg(int64_t n, const int* d_m, const T* Q, const T* W, const int64_t* chunks, int nchunks,
                                 const int* active, double* partial, cudaStream_t st) {
     using S = GramRowsShape<T, B>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_rows_seg_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)S::smem_bytes));
-        attr_set = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_rows_seg_kernel<T, B>, S::smem_bytes));
     gram_rows_seg_kernel<T, B><<<(unsigned)nchunks, kThreads, S::smem_bytes, st>>>(n, d_m, chunks, active, Q, W,
                                                                                    partial);
     BBL_LAUNCH_CHECK();
@@ -2015,12 +1999,8 @@ bbl_status launch_gram_seg(int64_t n, int m_max, const int* d_m, const T* Q, con
                            int nchunks, const int* active, double* partial, cudaStream_t st) {
     const int cols = (m_max + CPT - 1) / CPT;
     const int gy = (cols + kThreads - 1) / kThreads;
-    static bool attr_set = false;
-    if (!attr_set) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_seg_dyn_kernel<T, B, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(sizeof(double) * kThreads * CPT * B)));
-        attr_set = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_seg_dyn_kernel<T, B, CPT>, sizeof(double) * kThreads * CPT * B));
     dim3 grid((unsigned)nchunks, (unsigned)gy);
     gram_seg_dyn_kernel<T, B, CPT><<<grid, kThreads, sizeof(double) * kThreads * CPT * B, st>>>(n, d_m, chunks, active,
                                                                                                 Q, W, partial);

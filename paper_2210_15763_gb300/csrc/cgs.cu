@@ -333,12 +333,8 @@ bbl_status update_gram_tc(int64_t n, int nblocks, const float* Q, const double* 
                           DevBuf& work, cudaStream_t st) {
     if (!update_gram_tc_supports(nblocks))
         return set_error(BBL_ERR_UNSUPPORTED, "update_gram_tc: %d blocks outside 1..%d", nblocks, kFuMaxBlocks);
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(cgs_update_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kFuSmemLimit));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, cgs_update_gram_kernel, kFuSmemLimit));
     const int stages = fu_stages(nblocks);
     const size_t smem = fu_smem_bytes(nblocks, stages);
     int occ = 0;

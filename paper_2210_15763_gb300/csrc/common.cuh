@@ -10,6 +10,7 @@
 #include <string>
 
 #include "../../include/bbl.h"
+#include "once.h"
 
 namespace bbl {
 
@@ -57,6 +58,27 @@ constexpr int kDF32 = 2;
 inline size_t dtype_size(int dt) { return (dt == BBL_FP64 || dt == kDF32) ? 8 : 4; }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// f() (a bbl_status) unless it has succeeded on the current device before
+template <typename F>
+inline bbl_status once_per_device(OncePerDevice& once, F&& f) {
+    int dev = 0;
+    BBL_CUDA(cudaGetDevice(&dev));
+    if (!once.need(dev)) return BBL_OK;
+    BBL_TRY(f());
+    once.done(dev);
+    return BBL_OK;
+}
+// the kernel may use that much dynamic shared memory
+template <typename K>
+inline bbl_status allow_smem(OncePerDevice& once, K kernel, size_t bytes) {
+    return once_per_device(once, [&]() -> bbl_status {
+        BBL_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        return BBL_OK;
+    });
+}
+// SMs of the current device
+int sm_count();
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 

@@ -751,11 +751,8 @@ size_t kron_pipe_smem(const bbl_matrix* A, int CB, int IPT, int NT) {
 template <typename T, int CB, int IPT, int NT>
 bbl_status launch_kron_pipe(const bbl_matrix* A, int b, const T* V, T* W, size_t smem, cudaStream_t st) {
     auto kern = kron_pipe_kernel<T, CB, IPT, NT>;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKronSmemMax));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, kern, kKronSmemMax));
     dim3 grid((unsigned)A->kron_nP, (unsigned)(b / CB));
     kern<<<grid, NT, smem, st>>>(make_desc(A), b, V, W);
     BBL_LAUNCH_CHECK();
@@ -770,11 +767,8 @@ bbl_status launch_kron_t(const bbl_matrix* A, int b, const T* V, T* W, size_t sm
         if (ps <= kKronSmemMax && A->kron_K + 3 <= 40) return launch_kron_pipe<T, CB, IPT, NT>(A, b, V, W, ps, st);
     }
     auto kern = kron_spmm_kernel<T, CB, IPT, NT>;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKronSmemMax));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, kern, kKronSmemMax));
     dim3 grid((unsigned)A->kron_nP, (unsigned)(b / CB));
     kern<<<grid, NT, smem, st>>>(make_desc(A), b, V, W);
     BBL_LAUNCH_CHECK();

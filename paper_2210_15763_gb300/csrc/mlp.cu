@@ -395,12 +395,9 @@ bbl_status ensure_batch(bbl_mlp* M, int batch) {
 bbl_status launch_forward(const bbl_mlp* M, int batch, const float* g, float* y, const float* target, cudaStream_t st) {
     const int H = M->hidden, O = M->out;
     const size_t sm = sizeof(float) * kFwS * H;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(hidden_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwS * 1024 * 4));
-        BBL_CUDA(cudaFuncSetAttribute(output_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwS * 1024 * 4));
-        attr = true;
-    }
+    static OncePerDevice hidden_once, output_once;
+    BBL_TRY(allow_smem(hidden_once, hidden_kernel, kFwS * 1024 * 4));
+    BBL_TRY(allow_smem(output_once, output_kernel, kFwS * 1024 * 4));
     const unsigned groups = (unsigned)ceil_div(batch, kFwS);  // in x: any batch (y holds 65535 at most, rows 512)
     hidden_kernel<<<dim3(groups, (unsigned)ceil_div(H, kFwWarps)), kFwThreads, sm, st>>>(
         batch, H, O, M->params.as<float>(), M->wbf.as<__nv_bfloat16>(), g, M->act.as<float>());
@@ -417,14 +414,9 @@ bbl_status launch_loss_grad(bbl_mlp* M, int batch, const float* g, const float* 
     const int H = M->hidden, O = M->out;
     const int V = H % 4 == 0 ? 4 : 1;
     const auto backward_act = V == 4 ? backward_act_kernel<4> : backward_act_kernel<1>;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(float) * (kBwThreads * kBwS + kBwS * (1024 + 4096))));
-        BBL_CUDA(cudaFuncSetAttribute(backward_act_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(float) * (kBwThreads * kBwS * 4 + kBwS * (1024 + 4096))));
-        attr = true;
-    }
+    static OncePerDevice once1, once4;
+    BBL_TRY(allow_smem(once1, backward_act_kernel<1>, sizeof(float) * (kBwThreads * kBwS + kBwS * (1024 + 4096))));
+    BBL_TRY(allow_smem(once4, backward_act_kernel<4>, sizeof(float) * (kBwThreads * kBwS * 4 + kBwS * (1024 + 4096))));
     BBL_TRY(launch_forward(M, batch, g, nullptr, target, st));
     backward_act<<<(unsigned)ceil_div(batch, kBwS), kBwThreads,
                    sizeof(float) * (kBwThreads * kBwS * V + kBwS * (H + O)), st>>>(

@@ -1271,8 +1271,8 @@ size_t ritz_workspace_bytes(int m, int p, int nev) {
 
 namespace {
 bbl_status set_ritz_attrs() {
-    static bool attr_set = false;
-    if (!attr_set) {
+    static OncePerDevice once;
+    return once_per_device(once, []() -> bbl_status {
         BBL_CUDA(cudaFuncSetAttribute(bisect_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
         BBL_CUDA(cudaFuncSetAttribute(bisect_lane_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
         BBL_CUDA(cudaFuncSetAttribute(bisect_lane_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
@@ -1288,9 +1288,8 @@ bbl_status set_ritz_attrs() {
         BBL_CUDA(cudaFuncSetAttribute(invit_df_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvitSmemMax));
         BBL_CUDA(cudaFuncSetAttribute(invit_df_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvitSmemMax));
         BBL_CUDA(cudaFuncSetAttribute(invit_df_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvitSmemMax));
-        attr_set = true;
-    }
-    return BBL_OK;
+        return BBL_OK;
+    });
 }
 
 // the register-window bisection for p in {1, 2, 4, 8, 16}, else the generic one

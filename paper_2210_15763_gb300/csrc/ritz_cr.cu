@@ -925,12 +925,9 @@ template <int P>
 bbl_status launch_slices(int m, int nev, int nseg, const Lay& l, SegArgs sa, cudaStream_t st) {
     const int ns1 = first_shifts(nseg);
     const size_t sm = slice_extra<P>() + sizeof(float) * (size_t)((padded_rows(m, P) * (P + 1) + 3) & ~3);
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(slice_first_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        BBL_CUDA(cudaFuncSetAttribute(slice_second_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        attr = true;
-    }
+    static OncePerDevice first_once, second_once;
+    BBL_TRY(allow_smem(first_once, slice_first_kernel<P>, kSmemMax));
+    BBL_TRY(allow_smem(second_once, slice_second_kernel<P>, kSmemMax));
     slice_first_kernel<P><<<dim3(ns1 / kSliceShifts, nseg), kSliceThreads, sm, st>>>(m, ns1, l.hdr, l.band,
                                                                                     l.band_stride, l.c1, sa);
     BBL_LAUNCH_CHECK();
@@ -946,11 +943,8 @@ bbl_status launch_vec(int m, int p, int nev, int nseg, const double* Tb, double*
     const int J = (m + BS - 1) / BS;
     const size_t vecs = vec_vectors_bytes<BS>(J), mats = sizeof(float) * vec_mat_floats<BS>(J);
     const int in_smem = vecs + mats <= kSmemMax ? 1 : 0;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(vec_kernel<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, vec_kernel<BS>, kSmemMax));
     vec_kernel<BS><<<dim3(nev, nseg), kVecThreads, vecs + (in_smem ? mats : 0), st>>>(
         m, p, nev, Tb, in_smem, l.hdr, l.br, l.c2, l.band, l.band_stride, ws, (int64_t)ritz_cr_vec_doubles(m, p), theta, S,
         l.need, l.guess, sa);

@@ -900,27 +900,13 @@ __global__ void __launch_bounds__(kT, 2) update_tc64_seg_kernel(int64_t n, const
         update_group<B, true>(n, m, B, 1, kWarps, 0, row0, r1, staged, Q, C + seg * cstride, W, tc_smem, ew);
 }
 
-int sms() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    }
-    return n;
-}
-
 constexpr int kFragBytes = kDig * 32 * (int)sizeof(uint2);  // a step's B fragments
 constexpr int kRingBytes = kWarps * kRing * kStepBytes;
 
 template <int B>
 bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, double* C, DevBuf& partials, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_tc64_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kRingBytes + kMaxRows / 16 * kFragBytes));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_tc64_kernel<B>, kRingBytes + kMaxRows / 16 * kFragBytes));
     constexpr int NH = (B + 7) / 8;
     // One chunk per resident CTA where that gives at least 64 rows, at most the
     // staged kMaxRows, else chunks of equal size for several rounds; with fewer
@@ -955,27 +941,23 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
 
 template <int B, bool SUB>
 bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double* C, double* W, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(update_tc64_kernel<B, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kRingBytes + kMaxCols / 16 * kFragBytes));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, update_tc64_kernel<B, SUB>, kRingBytes + kMaxCols / 16 * kFragBytes));
     const int64_t rtiles = ceil_div(n, 16);
     const int cols = std::min(m, kMaxCols), steps = (cols + 15) / 16;
     const int64_t ny = (kc + 7) / 8;
     // few rows: up to eight warps share a row tile's steps, so that the SMs' 16
     // warps have work
     int ks = 1;
-    while (ks < kWarps && rtiles * ks * 2 <= (int64_t)sms() * 2 * kWarps && steps >= ks * 4) ks <<= 1;
+    while (ks < kWarps && rtiles * ks * 2 <= (int64_t)sm_count() * 2 * kWarps && steps >= ks * 4) ks <<= 1;
     int tiles = kWarps / ks;
     // between one and two CTAs per SM: fewer tiles each, so that every SM has two
     // (n = 2e4, m = 200: 5 tiles, 250 CTAs, 26.2 us; with 8 five of the 152 SMs had
     // two CTAs, 27.1 us)
     const int64_t total = ceil_div(rtiles, tiles) * ny;
-    if (ks == 1 && total > sms() && total < (int64_t)2 * sms()) tiles = (int)ceil_div(rtiles * ny, (int64_t)2 * sms());
+    if (ks == 1 && total > sm_count() && total < (int64_t)2 * sm_count()) tiles = (int)ceil_div(rtiles * ny, (int64_t)2 * sm_count());
     const int64_t groups = ceil_div(rtiles, tiles);
-    const dim3 grid((unsigned)std::min<int64_t>(groups, (int64_t)sms() * 8), (unsigned)((kc + 7) / 8));
+    const dim3 grid((unsigned)std::min<int64_t>(groups, (int64_t)sm_count() * 8), (unsigned)((kc + 7) / 8));
     update_tc64_kernel<B, SUB><<<grid, kT, kRingBytes + (size_t)steps * kFragBytes, st>>>(n, m, kc, ks, tiles, Q, C, W);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
@@ -997,11 +979,8 @@ template <int B>
 bbl_status launch_gram_seg(int64_t n, const int* d_m, const double* Q, const double* W, const int64_t* chunks,
                            int nchunks, const int* active, double* partial, cudaStream_t st) {
     constexpr int kSmem = kRingBytes + kMaxRows / 16 * kFragBytes;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(gram_tc64_seg_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, gram_tc64_seg_kernel<B>, kSmem));
     gram_tc64_seg_kernel<B><<<(unsigned)nchunks, kT, kSmem, st>>>(n, d_m, chunks, active, Q, W, partial);
     BBL_LAUNCH_CHECK();
     return BBL_OK;
@@ -1011,11 +990,8 @@ template <int B>
 bbl_status launch_update_seg(int64_t n, const int* ms, int ms_stride, const int64_t* ctas, int nctas, const int* active,
                              const double* Q, const double* C, int64_t cstride, double* W, cudaStream_t st) {
     constexpr int kSmem = kRingBytes + kMaxCols / 16 * kFragBytes;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(update_tc64_seg_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, update_tc64_seg_kernel<B>, kSmem));
     update_tc64_seg_kernel<B><<<(unsigned)nctas, kT, kSmem, st>>>(n, ms, ms_stride, ctas, active, Q, C, cstride, W);
     BBL_LAUNCH_CHECK();
     return BBL_OK;

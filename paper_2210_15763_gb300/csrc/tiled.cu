@@ -383,11 +383,8 @@ constexpr size_t kTiledSmemMax = 200 * 1024;
 template <typename TM, typename TX, int CB>
 bbl_status launch_tiled_t(const bbl_matrix* A, int b, const TM* val, const TX* V, TX* W, cudaStream_t st) {
     auto kern = tiled_spmm_kernel<TM, TX, CB>;
-    static bool attr = false;
-    if (!attr) {
-        BBL_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTiledSmemMax));
-        attr = true;
-    }
+    static OncePerDevice once;
+    BBL_TRY(allow_smem(once, kern, kTiledSmemMax));
     const int T = A->tile;
     const size_t smem = 2 * (size_t)T * CB * sizeof(TX);
     dim3 grid((unsigned)A->t_nrb, (unsigned)(b / CB));
