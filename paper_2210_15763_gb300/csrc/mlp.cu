@@ -143,8 +143,15 @@ __global__ void __launch_bounds__(kFwThreads) hidden_kernel(int batch, int H, in
     }
 }
 
+// The squares are summed in units of the power of two above their number, which
+// rounds nothing: their plain sum could overflow where the mean does not.
+__device__ __forceinline__ float loss_unit(int batch, int O) {
+    const int e = (__float_as_int((float)batch * (float)O) >> 23) - 127;  // the number is in [2^e, 2^(e+1))
+    return __int_as_float((126 - e) << 23);
+}
+
 // y of 8 output rows for 16 samples; with a target also dy = 2 (y - t) / N and
-// the CTA's part of the mean loss
+// the CTA's sum of squares (in units of loss_unit)
 __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, int O, const float* __restrict__ P,
                                                             const __nv_bfloat16* __restrict__ Wb,
                                                             float* __restrict__ act, float* __restrict__ y_out,
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kFwThreads) output_kernel(int batch, int H, in
                 const float d = y - target[(size_t)(s0 + q) * O + o];
                 const float inv = 1.0f / ((float)batch * (float)O);
                 a[6 * H + O + o] = 2.0f * d * inv;
-                l = d * d * inv;  // the mean's term: a sum of squares could overflow where the mean does not
+                l = d * d * loss_unit(batch, O);
             }
         }
     }
@@ -286,7 +293,7 @@ __global__ void __launch_bounds__(256) backward_w_kernel(int batch, int H, int O
             if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
             __syncthreads();
         }
-        if (threadIdx.x == 0) *loss = red[0];
+        if (threadIdx.x == 0) *loss = red[0] * (1.0f / ((float)batch * (float)O) / loss_unit(batch, O));
         return;
     }
     const int np = 3 * H + H * H + O * H + O;
