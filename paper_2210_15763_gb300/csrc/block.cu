@@ -24,6 +24,7 @@
 
 #include <cuda_fp16.h>
 
+#include "async_mma.cuh"
 #include "common.cuh"
 #include "df32.cuh"
 
@@ -341,17 +342,6 @@ struct GramRowsShape {
 template <typename T>
 __device__ __forceinline__ T add_any(T a, T b) {
     return a + b;
-}
-
-// 16-byte asynchronous global -> shared copy; src_bytes = 0 writes zeros
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int src_bytes) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
 // warps per basis block when a chunk has fewer blocks than warps
@@ -982,15 +972,6 @@ __device__ __forceinline__ void ldsm_x2_trans(unsigned& r0, unsigned& r1, const 
     const unsigned a = (unsigned)__cvta_generic_to_shared(p);
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(a));
 }
-// D (16x8 FP32) += A (16x16 FP16, row) * B (16x8 FP16, col)
-__device__ __forceinline__ void mma_16816(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 template <bool GROUPED>
 __global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, int nitems, int groups,
                                                              const __half* __restrict__ Q, const float* __restrict__ W,
@@ -1074,7 +1055,7 @@ __global__ void __launch_bounds__(kThreads) gram_half_kernel(int64_t n, int m, i
                 ldsm_x4_trans(a[0], a[1], a[2], a[3], buf + (u * 32 + a_row) * B);
                 const int kk = (k % NST) * kHmSK + u;  // 16-row tile of the chunk
                 ldsm_x2_trans(bq[0], bq[1], ws + (kk * 16 + b_row) * B);
-                mma_16816(acc, a, bq);
+                mma_16816(acc, a, bq[0], bq[1]);
             }
             if ((k % NST) == NST - 1) {
                 // the pair's sums over this chunk: rows g (block 2p) and g + 8 (block 2p + 1), columns 2 tig, 2 tig + 1
@@ -1174,7 +1155,9 @@ bbl_status gram_typed(int64_t n, int b, int m, const T* Q, const T* W, double* C
         case 2: return launch_gram<T, 2, 2>(n, m, Q, W, C, partials, st);
         case 4: return launch_gram_rows<T, 4>(n, m, Q, W, C, partials, st);
         case 8: return launch_gram_rows<T, 8>(n, m, Q, W, C, partials, st);
-        case 16: return launch_gram<T, 16, 2>(n, m, Q, W, C, partials, st);
+        case 16:  // (FP64: on the tensor cores, tc64.cu)
+            if constexpr (!std::is_same<T, double>::value) return launch_gram<T, 16, 2>(n, m, Q, W, C, partials, st);
+            [[fallthrough]];
         default: return launch_gram_generic<T>(n, m, b, Q, W, C, partials, st);
     }
 }
@@ -1410,7 +1393,7 @@ __global__ void __launch_bounds__(256) apply_half_old_kernel(int64_t n, int nblo
     auto products = [&](int q0, const Group& x) {
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (q0 + u < npo) mma_16816(d, x.a[u], x.b[u]);
+            if (q0 + u < npo) mma_16816(d, x.a[u], x.b[u][0], x.b[u][1]);
     };
     Group g0;
     if constexpr (AHEAD) {
@@ -1534,7 +1517,12 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
             case 2: apply_kernel<T, 2, 2, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
             case 4: apply_kernel<T, 4, 4, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
             case 8: apply_kernel<T, 8, 8, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
-            case 16: apply_kernel<T, 16, 16, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
+            case 16:  // (the FP64 update: on the tensor cores, tc64.cu)
+                if constexpr (!(SUB && std::is_same<T, double>::value)) {
+                    apply_kernel<T, 16, 16, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W);
+                    break;
+                }
+                [[fallthrough]];
             default: apply_generic_kernel<T, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, b, kc, Q, C, W);
         }
     } else {
@@ -1543,7 +1531,12 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
             case 2: apply_kernel<T, 2, 0, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
             case 4: apply_kernel<T, 4, 0, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
             case 8: apply_kernel<T, 8, 0, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
-            case 16: apply_kernel<T, 16, 0, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W); break;
+            case 16:  // (FP64 Ritz vectors: tc64.cu)
+                if constexpr (!std::is_same<T, double>::value) {
+                    apply_kernel<T, 16, 0, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, kc, Q, C, W);
+                    break;
+                }
+                [[fallthrough]];
             default: apply_generic_kernel<T, SUB, TA, TO><<<grid, kThreads, 0, st>>>(n, m, b, kc, Q, C, W);
         }
     }
@@ -2027,11 +2020,18 @@ bbl_status apply_seg_typed(int64_t n, int b, int kc, const int* ms, int mss, con
     switch (b) {
         case 1: return launch_apply_seg<T, SUB, TA, TO, 1>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
         case 2: return launch_apply_seg<T, SUB, TA, TO, 2>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
-        case 4: return launch_apply_seg<T, SUB, TA, TO, 4>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
-        case 8: return launch_apply_seg<T, SUB, TA, TO, 8>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
+        case 4:  // (FP64 updates of 4 and 8 columns: tc64.cu)
+            if constexpr (!(SUB && std::is_same<T, double>::value))
+                return launch_apply_seg<T, SUB, TA, TO, 4>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
+            break;
+        case 8:
+            if constexpr (!(SUB && std::is_same<T, double>::value))
+                return launch_apply_seg<T, SUB, TA, TO, 8>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
+            break;
         case 16: return launch_apply_seg<T, SUB, TA, TO, 16>(n, kc, ms, mss, ctas, nctas, active, Q, C, cstride, W, st);
-        default: return set_error(BBL_ERR_UNSUPPORTED, "batched: b=%d (supported: 1, 2, 4, 8, 16)", b);
+        default: break;
     }
+    return set_error(BBL_ERR_UNSUPPORTED, "batched: b=%d (supported: 1, 2, 4, 8, 16)", b);
 }
 
 }  // namespace
@@ -2050,7 +2050,6 @@ int gram_seg_chunk_rows(int b, int dtype) {
 bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, const void* Q, const void* W,
                     const int64_t* chunks, int nchunks, const int* seg_chunk_ptr, int nseg, const int* active,
                     double* partial, double* C, cudaStream_t st) {
-    constexpr int kC = 4;
     // against a whole basis the FP64 products run on the tensor cores; the self
     // Gram of one block (m_max = b) fills too little of a tile of 16 columns
     const bool tc = dtype == BBL_FP64 && tc64_seg_supports(b) && m_max >= 32;
@@ -2077,8 +2076,6 @@ bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, cons
         switch (b) {
             case 1: BBL_TRY((launch_gram_seg<double, 1, 1>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
             case 2: BBL_TRY((launch_gram_seg<double, 2, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
-            case 4: BBL_TRY((launch_gram_seg<double, 4, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
-            case 8: BBL_TRY((launch_gram_seg<double, 8, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
             case 16: BBL_TRY((launch_gram_seg<double, 16, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
             default: return set_error(BBL_ERR_UNSUPPORTED, "batched: b=%d", b);
         }
@@ -2088,9 +2085,6 @@ bbl_status gram_seg(int64_t n, int b, int m_max, const int* d_m, int dtype, cons
         switch (b) {
             case 1: BBL_TRY((launch_gram_seg<float, 1, 1>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
             case 2: BBL_TRY((launch_gram_seg<float, 2, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
-            case 4: BBL_TRY((launch_gram_seg<float, 4, kC>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
-            case 8: BBL_TRY((launch_gram_seg<float, 8, kC>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
-            case 16: BBL_TRY((launch_gram_seg<float, 16, 2>(n, m_max, d_m, q, w, chunks, nchunks, active, partial, st))); break;
             default: return set_error(BBL_ERR_UNSUPPORTED, "batched: b=%d", b);
         }
     }
@@ -2106,7 +2100,7 @@ bbl_status apply_seg(int64_t n, int b, int kc, const int* ms, int ms_stride, int
                      cudaStream_t st) {
     if (dtype == BBL_FP64) {
         auto q = static_cast<const double*>(Q);
-        if (sub && kc == b && tc64_seg_supports(b))
+        if (sub && tc64_seg_supports(b))  // (kc is b)
             return update_tc64_seg(n, b, ms, ms_stride, ctas, nctas, active, q, C, cstride, static_cast<double*>(W), st);
         if (sub) return apply_seg_typed<double, true, double, double>(n, b, kc, ms, ms_stride, ctas, nctas, active, q, C, cstride,
                                                                       static_cast<double*>(W), st);

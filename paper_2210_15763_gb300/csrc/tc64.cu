@@ -46,6 +46,7 @@
 
 #include <cuda_fp16.h>
 
+#include "async_mma.cuh"
 #include "common.cuh"
 
 namespace bbl {
@@ -100,14 +101,6 @@ struct Acc {
         return fma((double)L, 0x1p-8, (double)h[e]);
     }
 };
-
-__device__ __forceinline__ void mma_f16(float (&d)[4], const unsigned (&a)[4], const uint2 b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
-}
 
 // exponent field of a double's high word, in place (bits 20..30)
 __device__ __forceinline__ int exp_bits(double v) { return __double2hiint(v) & 0x7ff00000; }
@@ -214,7 +207,7 @@ template <int I>
 __device__ __forceinline__ void mma_digit(Acc& acc, const Pair (&p)[4], const uint2 (&b)[kDig]) {
     const unsigned a[4] = {p[0].digit<I>(), p[1].digit<I>(), p[2].digit<I>(), p[3].digit<I>()};
 #pragma unroll
-    for (int j = 0; j < kDig && I + j < kOrd; ++j) mma_f16(acc.f[I + j], a, b[j]);
+    for (int j = 0; j < kDig && I + j < kOrd; ++j) mma_16816(acc.f[I + j], a, b[j].x, b[j].y);
 }
 
 // 16 terms: pairs p (fragment registers 0..3 of A), B's digits at frag[j * 32 + lane]
@@ -224,7 +217,7 @@ __device__ __forceinline__ void mma_step(Acc& acc, const Pair (&p)[4], const uin
     for (int j = 0; j < kDig; ++j) b[j] = frag[j * 32 + lane];
     mma_digit<7>(acc, p, b);
     const unsigned a[4] = {p[0].lead(), p[1].lead(), p[2].lead(), p[3].lead()};
-    mma_f16(acc.c, a, make_uint2(b[0].x & 0x7fff7fffu, b[0].y & 0x7fff7fffu));
+    mma_16816(acc.c, a, b[0].x & 0x7fff7fffu, b[0].y & 0x7fff7fffu);
     mma_digit<0>(acc, p, b);
     mma_digit<1>(acc, p, b);
     mma_digit<2>(acc, p, b);
@@ -449,20 +442,6 @@ __device__ __forceinline__ void again(unsigned bad, int terms, Term&& term, Put&
         }
 }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool ok) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 __device__ __forceinline__ double not_a_number() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 // v: the sum over orders in units of order 4 (2^64); the scales of A and B are
@@ -562,7 +541,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
                     void* dst = buf + (j * CPB + r * CPR + swizzle<B>(r, q)) * 16;
                     const double* src = p + (int64_t)j * n * B + (16 * s + r) * B + 2 * q;
                     if (full) cp_async16(dst, src);
-                    else cp_async16(dst, (j < nblk && 16 * s + r < rows) ? src : Q, j < nblk && 16 * s + r < rows);
+                    else cp_async16(dst, (j < nblk && 16 * s + r < rows) ? src : Q, j < nblk && 16 * s + r < rows ? 16 : 0);
                 }
             }
             cp_async_commit();
@@ -765,7 +744,7 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
                     const double* src = Q + ((int64_t)(a / B) * n + r) * B + a % B;
                     double2* dst = ring + (s % kRing) * 128 + i * 32;
                     if (full) cp_async16(dst, src);
-                    else cp_async16(dst, (a < m && r < row_end) ? src : Q, a < m && r < row_end);
+                    else cp_async16(dst, (a < m && r < row_end) ? src : Q, a < m && r < row_end ? 16 : 0);
                 }
             }
             cp_async_commit();
