@@ -1547,13 +1547,12 @@ bbl_status apply_typed(int64_t n, int b, int m, int kc, const T* Q, const double
 // -------------------------------------------------------------------- Cholesky of the b x b Gram
 // status bits: 1 = non-finite Gram.  mask[i] = 1 for deflated columns.
 
-// 1 / d, rounded as the division rounds it but for one case in about 2^39: an FP32
-// seed on the mantissa and two Newton steps, the last from an error below 2^-45
-// (four FP64 instructions in a chain; an FP64 instruction occupies its scheduler
-// for 64 cycles here, and the division takes about ten).
+// 1 / d for d in 2^-959 .. 2^957, rounded as the division rounds it but for one
+// case in about 2^39: an FP32 seed on the mantissa and two Newton steps, the last
+// from an error below 2^-45 (four FP64 instructions in a chain; an FP64 instruction
+// occupies its scheduler for 64 cycles here, and the division takes about ten).
 __device__ __forceinline__ double recip(double d) {
-    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
-    if (ex < 64 || ex > 1980) return 1.0 / d;
+    const int hi = __double2hiint(d), ex = hi >> 20;
     const double m = __hiloint2double(hi - (ex - 1023) * (1 << 20), __double2loint(d));
     double y = (double)__frcp_rn((float)m);
     y = fma(y, fma(-m, y, 1.0), y);
@@ -1574,6 +1573,7 @@ struct CholShared {
     double L[kMaxB * kMaxB];      // row k: D[k] L[.][k]
     double Z[kMaxB * kMaxB];      // row k of L^{-1}
     double row[2][2][kMaxB];      // row k of the Schur complement and of L^{-1}
+    double scaled[kMaxB];         // row k times a power of two
     double d[kMaxB], root[kMaxB]; // D (0 for deflated columns) and its square roots
     int deflated[kMaxB];
 };
@@ -1613,9 +1613,20 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
         const double d = ra[k];
         const int defl = !(d > thresh2) || bad;
         cnt += defl;
-        // a pivot whose reciprocal is not a normal number divides instead
-        const bool whole = d > 0x1p-1020 && d < 0x1p1020;
-        const double y = defl || !whole ? 0.0 : recip(d);
+        const double* rl = ra;
+        double y = 0.0;
+        const int ex = __double2hiint(d) >> 20;
+        if (!defl) {
+            if ((unsigned)ex - 64u <= 1916u) {
+                y = recip(d);
+            } else {  // far pivots: they and their row by a power of two
+                const double f = __hiloint2double((ex < 64 ? 1623 : 423) << 20, 0);
+                if (lane < b) sh.scaled[lane] = ra[lane] * f;
+                __syncwarp();
+                rl = sh.scaled;
+                y = recip(d * f);
+            }
+        }
         if (lane == 0) {
             sh.deflated[k] = defl;
             sh.d[k] = defl ? 0.0 : d;
@@ -1627,7 +1638,7 @@ __device__ __forceinline__ void chol_core(int b, double thresh2, int relative, C
 #pragma unroll
         for (int x = 0; x < E; ++x) {
             if (32 * x < bb && ei[x] > k) {
-                const double l = whole || defl ? ra[ei[x]] * y : ra[ei[x]] / d;
+                const double l = rl[ei[x]] * y;
                 if (!defl && ec[x] >= ei[x]) a[x] = fma(-l, ra[ec[x]], a[x]);
                 if (!defl && ec[x] <= k) z[x] = fma(-l, rz[ec[x]], z[x]);
                 if (ei[x] == k + 1) {
