@@ -4,8 +4,8 @@
 // A sequential band factorisation is a chain of m dependent row steps: on
 // one CTA per eigenvalue the float-float LU with its three triangular solves
 // took 1.71 ms and the one-CTA bisection 1.31 ms at m = 728, p = 8, nev = 8,
-// with 8 of 152 SMs busy.  The kernels here take 0.16 ms for the same pairs
-// (prep 6, slices 29 + 30, vec 80 us; the whole call 6.48 -> 0.37 ms), bound by
+// with 8 of 152 SMs busy.  The kernels here take 0.15 ms for the same pairs
+// (prep 6, slices 29 + 30, vec 79 us; the whole call 6.5 -> 0.20 to 0.26 ms), bound by
 // the latency of their dependent steps:
 //
 //  1. slice   counts the eigenvalues below many shifts at once (Sylvester
