@@ -290,25 +290,26 @@ __device__ __forceinline__ int scale_field(double v) {
 struct LineScale {
     int E0 = 0, E1 = 0;
     unsigned nz0 = 0, nz1 = 0;  // not zero: the lane has seen entries that are not zero
-    // shift words of the entries; for the whole warp: 0 if all are at most 31,
-    // bit 0 if some are larger, bit 1 if an entry exceeds its scale by more than
-    // kOver bits
-    __device__ __forceinline__ unsigned shifts(const double (&x)[8], unsigned (&s)[8]) {
+    // shift words of the entries; for the whole warp: 0 if all are at most 31 (no
+    // entry is zero, none above its scale by more than kOver bits), else 1
+    __device__ __forceinline__ unsigned cut(const double (&x)[8], unsigned (&s)[8]) {
         unsigned bits = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             s[k] = shift_word((k & 2) ? E1 : E0, x[k]);
             bits |= s[k] & 0x7e0u;
         }
-        if (!__any_sync(0xffffffffu, bits)) {
-            nz0 = nz1 = 1u;
-            return 0;
-        }
-        bool over = false;
+        if (__any_sync(0xffffffffu, bits)) return 1;
+        nz0 = nz1 = 1u;
+        return 0;
+    }
+    // whether an entry of the warp exceeds its scale by more than kOver bits
+    __device__ __forceinline__ bool over(const double (&x)[8]) const {
+        bool far = false;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-            over = over || (int)(((unsigned)__double2hiint(x[k]) >> 20) & 0x7ffu) > ((k & 2) ? E1 : E0) + kOver;
-        return __any_sync(0xffffffffu, over) ? 3 : 1;
+            far = far || (int)(((unsigned)__double2hiint(x[k]) >> 20) & 0x7ffu) > ((k & 2) ? E1 : E0) + kOver;
+        return __any_sync(0xffffffffu, far);
     }
     __device__ __forceinline__ void seen(const double (&x)[8]) {
 #pragma unroll
@@ -348,23 +349,22 @@ __device__ __forceinline__ void step(Acc& acc, LineScale& sc, const double (&x)[
     unsigned s[8];
     Pair p[4];
     const bool first = sc.E0 == 0;
-    const unsigned how = first ? 3u : sc.shifts(x, s);
-    if (how == 0) {  // no entry is zero
+    unsigned how = first ? 1u : sc.cut(x, s);
+    if (how && (first || sc.over(x))) {
+        if (!first) flush();
+        const int e0 = sc.E0, e1 = sc.E1;
+        sc.raise(x);
+        const float d0 = down2(sc.E0 - e0), d1 = down2(sc.E1 - e1);
+        acc.c[0] *= d0;
+        acc.c[1] *= d0;
+        acc.c[2] *= d1;
+        acc.c[3] *= d1;
+        how = sc.cut(x, s);  // (on ordinary data the first step goes on like the others)
+    }
+    if (how == 0) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) p[r].template set<false>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
     } else {
-        if (how & 2) {
-            if (!first) flush();
-            const int e0 = sc.E0, e1 = sc.E1;
-            sc.raise(x);
-            const float d0 = down2(sc.E0 - e0), d1 = down2(sc.E1 - e1);
-            acc.c[0] *= d0;
-            acc.c[1] *= d0;
-            acc.c[2] *= d1;
-            acc.c[3] *= d1;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s[k] = shift_word((k & 2) ? sc.E1 : sc.E0, x[k]);
-        }
         sc.seen(x);
 #pragma unroll
         for (int r = 0; r < 4; ++r) p[r].template set<true>(x[2 * r], x[2 * r + 1], s[2 * r], s[2 * r + 1]);
@@ -450,6 +450,32 @@ __device__ __forceinline__ double not_a_number() { return __longlong_as_double(0
 __device__ __forceinline__ double unscale(double v, int ea, int eb) {
     if (ea >= 0x7ff || eb >= 0x7ff) return not_a_number();
     return scale_by(v, 64 + ea + eb - 2156);
+}
+
+// The sums of a Gram item (basis columns j0 .. j0 + 15, rows from r on, columns
+// c0 .. c0 + 7 of W) and of an update (16 rows from r on, below row_end) that the
+// digits do not certify: results at res[32 e] of the lane.  Lines and columns past
+// the operands' are zeros.  Kept out of line: the hot kernels' code stays short.
+template <int B>
+__device__ __noinline__ void again_gram(unsigned bad, int terms, int64_t n, int m, int j0, int64_t r, int c0,
+                                        const double* __restrict__ Q, const double* __restrict__ W, double* res) {
+    again(bad, terms,
+          [&](int line, int c, int k, double& a, double& b) {
+              const int j = j0 + line;
+              a = j < m ? Q[((int64_t)(j / B) * n + r + k) * B + j % B] : 0.0;
+              b = c0 + c < B ? W[(r + k) * B + c0 + c] : 0.0;
+          },
+          [&](int e, double v) { res[32 * e] = v; });
+}
+template <int B>
+__device__ __noinline__ void again_update(unsigned bad, int m, int64_t n, int kc, int64_t r, int64_t row_end, int c0,
+                                          const double* Q, const double* __restrict__ C, double* res) {
+    again(bad, m,
+          [&](int line, int c, int k, double& a, double& b) {
+              a = r + line < row_end ? Q[((int64_t)(k / B) * n + r + line) * B + k % B] : 0.0;
+              b = c0 + c < kc ? C[(int64_t)k * kc + c0 + c] : 0.0;
+          },
+          [&](int e, double v) { res[32 * e] = v; });
 }
 
 // -------------------------------------------------------------------- C = Q^T W
@@ -582,15 +608,7 @@ __device__ __forceinline__ void gram_chunk(int64_t n, int m, int tile0, int ntil
         line_fields(sc, E);
         const unsigned bad = uncertified(acc.c, E, ew[2 * t], ew[2 * t + 1]);
         if (__any_sync(0xffffffffu, bad)) {
-            // (lines past the last basis column and columns past W's are zeros, which are certified)
-            again(bad, min(16 * s1, rows) - 16 * s0,
-                  [&](int line, int c, int k, double& a, double& b) {
-                      const int64_t r = r0 + 16 * s0 + k;
-                      const int j = 16 * tile + line;
-                      a = j < m ? Q[((int64_t)(j / B) * n + r) * B + j % B] : 0.0;
-                      b = c0 + c < B ? W[r * B + c0 + c] : 0.0;
-                  },
-                  [&](int e, double v) { mine[32 * e] = v; });
+            again_gram<B>(bad, min(16 * s1, rows) - 16 * s0, n, m, 16 * tile, r0 + 16 * s0, c0, Q, W, mine);
         }
         if (parts == 1) {
 #pragma unroll
@@ -823,19 +841,12 @@ __device__ __forceinline__ void update_group(int64_t n, int m, int kc, int ks, i
                     bad &= ~(1u << e);
             }
         }
-        // (rows past the end and columns past C's are zeros, which are certified
-        // unless the other operand is not finite)
-        again(bad, m,
-              [&](int line, int c, int k, double& a, double& b) {
-                  const int64_t r = rt + line;
-                  a = r < row_end ? Q[((int64_t)(k / B) * n + r) * B + k % B] : 0.0;
-                  b = c0 + c < kc ? C[(int64_t)k * kc + c0 + c] : 0.0;
-              },
-              [&](int e, double v) {
+        double* res = reinterpret_cast<double*>(smem + warp * kRing * kStepBytes) + lane;  // the warp's ring, free now
 #pragma unroll
-                  for (int q = 0; q < 4; ++q)
-                      if (q == e) out[q] = v;
-              });
+        for (int e = 0; e < 4; ++e) res[32 * e] = out[e];
+        again_update<B>(bad, m, n, kc, rt, row_end, c0, Q, C, res);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) out[e] = res[32 * e];
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
