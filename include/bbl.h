@@ -285,14 +285,15 @@ bbl_status bbl_spmm_f64(const bbl_matrix* A, int b, const double* V, double* W, 
  *   coeff   device FP64 [passes][nblocks*b][b] (row-major), or NULL
  * dtype: element type of basis and W (FP64 / FP32; FP32 accumulates the
  * coefficients in FP64 across row chunks).  passes in 1..2.
- * FP64, b in {4, 8, 16} and at least 16 basis columns (C also b = 2 from 32 on):
- * the products are formed on the tensor cores from 64-bit splits of the entries
- * relative to their column's (C) or row's (W) largest within a chunk.  Each sum is
- * checked, and one whose terms are too small for that is formed again by FP64 FMA,
- * as are those with an infinity or a NaN: for entries of any range a sum of N
- * products errs by at most 2 N x 2^-53 of the sum of their magnitudes (|W|
- * included in the update), and by less than FP64 sums in sequence on Lanczos
- * bases.  The same holds for bbl_block_gram and bbl_ritz_vectors.       */
+ * FP64, b in {4, 8, 16} from 16 to 40 basis columns on, for C also b = 2 from 32 or 48
+ * on (where that is faster): the products are formed on the tensor cores from
+ * 64-bit splits of the entries relative to their column's (C) or row's (W)
+ * largest within a chunk.  Each sum is checked, and one whose terms are too small
+ * for that is formed again by FP64 FMA, as are those with an infinity or a NaN:
+ * for entries of any range a sum of N products errs by at most 2 N x 2^-53 of the
+ * sum of their magnitudes (|W| included in the update), and by less than FP64
+ * sums in sequence on Lanczos bases.  The same holds for bbl_block_gram and
+ * bbl_ritz_vectors.                                                     */
 bbl_status bbl_block_reorth(int64_t n, int b, int nblocks, bbl_dtype dtype, const void* basis, void* W,
                             double* coeff, int passes, void* stream);
 

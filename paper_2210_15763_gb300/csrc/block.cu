@@ -1757,7 +1757,7 @@ int gram_worker_sms() { return std::max(1, sm_count() - kRitzReserveSMs); }
 bbl_status gram(int64_t n, int b, int nblocks, int dtype, const void* Q, const void* W, double* C, DevBuf& partials,
                 cudaStream_t st) {
     const int m = nblocks * b;
-    if (dtype == BBL_FP64 && tc64_gram_supports(b, m))
+    if (dtype == BBL_FP64 && tc64_gram_supports(n, b, m))
         return gram_tc64(n, b, m, static_cast<const double*>(Q), static_cast<const double*>(W), C, partials, st);
     if (dtype == BBL_FP64)
         return gram_typed<double>(n, b, m, static_cast<const double*>(Q), static_cast<const double*>(W), C, partials, st);

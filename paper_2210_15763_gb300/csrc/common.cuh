@@ -327,9 +327,9 @@ bbl_status ritz_vectors(int64_t n, int b, int nblocks, int dtype, const void* Q,
 bbl_status cholqr2_dev(int64_t n, int b, int dtype, void* W, double* B, double defl_abs2, int* d_ndefl,
                        int* d_deflmask, DevBuf& partials, DevBuf& small, cudaStream_t st);
 // tc64.cu: FP64 C = Q^T W and W (-)= Q C (C, W of kc columns) on the tensor
-// cores, to FP64 accuracy, for the b and m (basis columns) that the supports
+// cores, to FP64 accuracy, for the n, b and m (basis columns) that the supports
 // functions name and a 16-byte aligned Q
-bool tc64_gram_supports(int b, int m);
+bool tc64_gram_supports(int64_t n, int b, int m);
 bool tc64_update_supports(int b, int m);
 bbl_status gram_tc64(int64_t n, int b, int m, const double* Q, const double* W, double* C, DevBuf& partials,
                      cudaStream_t st);

@@ -37,7 +37,7 @@
 //
 // Digits are cut by integer instructions in registers from a ring of
 // asynchronous copies.  At n = 6e5, b = 8, 90 blocks (3.5 GB, 0.51 ms at the copy
-// rate) the Gram takes 1.25 ms and the update 1.21 ms (with 56 bits and no check
+// rate) the Gram takes 1.23 ms and the update 1.20 ms (with 56 bits and no check
 // 1.09 and 1.12).  What bounds them is the latency of the cutting at four warps per
 // scheduler (integer pipe about half, tensor pipe a third active, DRAM a third of
 // the copy rate).
@@ -903,7 +903,7 @@ bbl_status launch_gram(int64_t n, int m, const double* Q, const double* W, doubl
     // rows the tiles are split into groups of
     // one per warp, which take more rows each (an item's end, its FP64
     // conversions, costs as much as three steps).  n = 2e4, b = 4, m = 400: 36.7 us
-    // in one group, 33.4 in four; m = 200: 21.2 and 21.0.
+    // in one group, 33.4 in four; m = 200: 21.2 and 21.0 (with 56-bit splits; now 36.4 and 22.3).
     const int64_t resident = (int64_t)2 * gram_worker_sms();
     const int ntiles = (m + 15) / 16;
     int64_t groups = (ntiles + kWarps - 1) / kWarps;
@@ -943,7 +943,7 @@ bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double
     int tiles = kWarps / ks;
     // between one and two CTAs per SM: fewer tiles each, so that every SM has two
     // (n = 2e4, m = 200: 5 tiles, 250 CTAs, 26.2 us; with 8 five of the 152 SMs had
-    // two CTAs, 27.1 us)
+    // two CTAs, 27.1 us, with 56-bit splits; now 28.5)
     const int64_t total = ceil_div(rtiles, tiles) * ny;
     if (ks == 1 && total > sm_count() && total < (int64_t)2 * sm_count()) tiles = (int)ceil_div(rtiles * ny, (int64_t)2 * sm_count());
     const int64_t groups = ceil_div(rtiles, tiles);
@@ -955,13 +955,21 @@ bbl_status launch_update(int64_t n, int m, int kc, const double* Q, const double
 
 }  // namespace
 
-// Measured against the FP64 FMA kernels (GB300): at b >= 4 the split is faster
-// from 16 columns on (n = 1e6, b = 8, m = 80: Gram 1592 us, update 1052 us);
-// with one block (m = 8) half of each tile is padding and the operands' own
-// split is not shared by many columns, and with b = 1 (Gram, update) and
-// b = 2 (update) the FMA kernels have no more than two products per entry.
-bool tc64_gram_supports(int b, int m) { return (b == 2 && m >= 32) || ((b == 4 || b == 8 || b == 16) && m >= 16); }
-bool tc64_update_supports(int b, int m) { return (b == 4 || b == 8 || b == 16) && m >= 16; }
+// Measured against the FP64 FMA kernels (us, FMA / split): the split is faster from
+// 16 columns on with b = 8 (n = 1e6: Gram 332 / 115, update 217 / 117; m = 80: 1592 / 329,
+// 1052 / 270; n = 2000: 10.4 / 6.1, 11.5 / 6.1) and b = 16; with one block (m = 8) half of each
+// tile is padding.  With b = 4 the Gram from 16 on (n = 1e6: 177 / 114; n = 3e4: 10.8 / 10.8), for
+// few rows from 40 on (n = 4000, m = 24: 6.3 / 7.5, 40: 8.6 / 8.0), the update from 32 on
+// (n = 1e6, m = 16: 115 / 158, 28: 184 / 177, 32: 219 / 186; n = 3e4, m = 32: 11.2 / 10.5).  With b = 2
+// the Gram from 32 on (n = 4000: 23.5 / 7.7), for many rows, where the FMA kernel is full, from 48
+// on (n = 1e6, m = 32: 132 / 154, 40: 246 / 254, 48: 251 / 233; n = 2e5, m = 32: 39.3 / 38.0).  With b = 1,
+// and in the update b = 2, the FMA kernels have no more than two products per entry.
+bool tc64_gram_supports(int64_t n, int b, int m) {
+    if (b == 2) return m >= (n <= 400000 ? 32 : 48);
+    if (b == 4) return m >= (n < 10000 ? 40 : 16);
+    return (b == 8 || b == 16) && m >= 16;
+}
+bool tc64_update_supports(int b, int m) { return (b == 4 && m >= 32) || ((b == 8 || b == 16) && m >= 16); }
 
 namespace {
 

@@ -96,3 +96,17 @@ def test_many_rows(n, b, m):
     r = np.random.default_rng(n)
     Q, W = r.standard_normal((m // b, n, b)), r.standard_normal((n, b))
     _check(Q, W, cols=np.unique(r.integers(0, m, 24)), rows=np.unique(np.r_[r.integers(0, n, 500), n - 1]))
+
+
+@pytest.mark.parametrize("b,m", [(2, 30), (2, 32), (2, 46), (2, 48), (4, 12), (4, 16), (4, 28), (4, 32), (4, 36), (4, 40), (8, 8), (8, 16), (16, 16)])
+def test_either_side_of_the_dispatch(b, m):
+    r = np.random.default_rng(b + m)
+    for n in (333, 10001):
+        _check(r.standard_normal((m // b, n, b)), r.standard_normal((n, b)), rows=np.arange(0, n, 7))
+
+
+@pytest.mark.parametrize("n", [400000, 400001])
+def test_two_columns_of_many_rows(n):
+    r = np.random.default_rng(n)
+    Q, W = r.standard_normal((16, n, 2)), r.standard_normal((n, 2))
+    _check(Q, W, cols=np.arange(0, 32, 3), rows=np.r_[0:200, n - 200:n])
