@@ -62,3 +62,19 @@ def test_a_batch_beyond_the_memory_leaves_the_network_usable():
         bbl._lib.check(bbl._lib.load().bbl_mlp_forward(net.handle, 1600000000, x.data_ptr(), x.data_ptr(), None))
     np.testing.assert_allclose(net.forward(x).cpu().numpy(), want, atol=1e-5)
     net.train(x, t, 1, 1e-12)
+
+
+@pytest.mark.parametrize("H,O", [(1, 1), (5, 7), (16, 48), (31, 2), (31, 3), (4, 252), (4, 253)])
+def test_small_networks_forward(H, O):
+    """Either side of the one-kernel forward: a batch in one call and in two large enough
+    for the general kernels gives the same bits, and the oracle's values."""
+    torch, bbl = need_gpu()
+    p, g, _ = _setup(H, O, 400, seed=H + O)
+    net = bbl.MLP(H, O)
+    net.set_params(pack(p))
+    few = net.forward(to_dev(torch, g, torch.float32)).cpu().numpy()
+    many = net.forward(to_dev(torch, np.tile(g, 2), torch.float32)).cpu().numpy()
+    assert (many == np.tile(few, (2, 1))).all()
+    ref = OM.forward(p, g)[0]
+    # FP32 sums of at most 31 products, twice, and the FP32 error function
+    assert np.abs(few - ref).max() <= 1e-5 * (np.abs(ref).max() + 1.0)
