@@ -290,7 +290,7 @@ bbl_status bbl_spmm_f64(const bbl_matrix* A, int b, const double* V, double* W, 
  * 64-bit splits of the entries relative to their column's (C) or row's (W)
  * largest within a chunk.  Each sum is checked, and one whose terms are too small
  * for that is formed again by FP64 FMA, as are those with an infinity or a NaN:
- * for entries of any range a sum of N products errs by at most 2 N x 2^-53 of the
+ * for entries of any range a sum of N products errs by at most 3 N x 2^-53 of the
  * sum of their magnitudes (|W| included in the update), and by less than FP64
  * sums in sequence on Lanczos bases.  The same holds for bbl_block_gram and
  * bbl_ritz_vectors.                                                     */

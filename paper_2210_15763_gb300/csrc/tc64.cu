@@ -21,19 +21,20 @@
 // What the cut loses is measured against a line's largest entry, and a sum whose
 // own terms are all far below that (a basis column with one large entry opposite
 // a zero, a row that is tiny where the coefficients are large) would lose bits that
-// FP64 sums keep.  So each sum certifies itself: one more product, of the two
-// leading digits' magnitudes, gives Sigma = sum |q||w| in units of 2^96 of the
-// (56-bit) integers' product, to two digits.  What is dropped and truncated is at most 2^50 per term,
-// and about 2^46.5 with a random sign: 2^51 over 512 terms.  From Sigma = 64 = 2^102 on that is
-// 4 x 2^-53 of sum |q||w| over 512 terms (2 N x 2^-53 for N terms if all signs
-// agree; the bound of an FP64 sum in sequence is N x 2^-53).  A sum below, or with
-// an operand that is not finite, is formed again by FP64 FMA, which also treats
-// infinities and numbers below the digits' range as FP64 does.  In a Lanczos run
-// that is about one sum in 10^5.  The largest error of any sum, relative to its
-// sum of magnitudes, on orthonormal bases (n = 2e4, b = 4, 360 columns; n = 2e5, b = 8,
-// 400): Gram 9.1e-17 and 1.1e-16, update 5.8e-17 and 7.4e-17; FP64 FMA kernels
-// 1.3e-16 and 1.8e-16, 1.9e-16 and 2.8e-16; 56-bit integers without the check
-// 9.2e-17 and 1.2e-16, 6.1e-16 and 6.1e-16.
+// FP64 sums keep.  So each sum certifies itself: one more product, of the leading
+// digits' magnitudes, gives Sigma, which is at most twice sum |q||w| in units of
+// 2^96 of the (56-bit) integers' product.  What is dropped and truncated is at most
+// 2^50.5 per term, and about 2^46.5 with a random sign: 2^51 over 512 terms.  From
+// Sigma = 128 on, sum |q||w| of 2^102 and more, that is 4 x 2^-53 of it over 512 terms
+// (3 N x 2^-53 for N terms if all signs agree; the bound of an FP64 sum in sequence
+// is N x 2^-53).  A sum below, or with an operand that is not finite, is formed
+// again by FP64 FMA, which also treats infinities and numbers below the digits'
+// range as FP64 does.  In a Lanczos run that is about one sum in 10^5 (the update
+// counts |W|, by which its difference rounds, towards Sigma).  The largest error
+// of any sum, relative to its sum of magnitudes, on orthonormal bases (n = 2e4, b = 4,
+// 360 columns; n = 2e5, b = 8, 400): Gram 9.1e-17 and 1.1e-16, update 5.8e-17 and
+// 7.4e-17; FP64 FMA kernels 1.3e-16 and 1.8e-16, 1.9e-16 and 2.8e-16; 56-bit
+// integers without the check 9.2e-17 and 1.2e-16, 6.1e-16 and 6.1e-16.
 //
 // Digits are cut by integer instructions in registers from a ring of
 // asynchronous copies.  At n = 6e5, b = 8, 90 blocks (3.5 GB, 0.51 ms at the copy
@@ -57,7 +58,7 @@ constexpr int kWarps = kT / 32;
 constexpr int kDig = 8;            // digits of 8 bits
 constexpr int kOrd = 8;            // orders summed (of the products' 15)
 constexpr int kExact = 5;          // orders kept exactly
-constexpr float kCertified = 64.0f;   // a sum's Sigma from which the digits' error is that of FP64 sums
+constexpr float kCertified = 128.0f;  // a sum's Sigma from which the digits' error is that of FP64 sums
 constexpr int kOver = 2;           // bits by which an entry may exceed its line's scale (the first digit's spare bits)
 constexpr int kMaxRows = 448;      // Gram: rows per CTA (two CTAs per SM by their shared memory)
 constexpr int kMaxCols = 512;      // update: coefficient rows staged at once
